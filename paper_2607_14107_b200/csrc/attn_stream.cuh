@@ -124,7 +124,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             auto clean = [&](int kt) {          // tile last written by an earlier forward: loadable before the dependency wait
                 const int lo = kt * KEYS, hi = lo + KEYS;
                 return hi <= a.dirty_lo || lo >= a.dirty_hi;
@@ -154,7 +154,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc_s = instr_desc_bf16(ROWS, KEYS);
             const uint32_t idesc_o = instr_desc_bf16(ROWS, DH) | (1u << 16);       // B (= V) is MN-major
             bool ok = mbar_wait(bar_q, 0, abort_flag);

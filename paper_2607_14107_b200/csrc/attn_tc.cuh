@@ -211,7 +211,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     volatile int* abort_flag = &abort_sh;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // Key tiles outside [dirty_lo, dirty_hi) were last written by an earlier forward, which the host has
             // waited for: their K / V can be on their way while the previous kernel still runs.
             auto tile_clean = [&](int j) {
@@ -242,7 +242,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc_s = instr_desc_bf16(ROWS, KEYS);
             const uint32_t idesc_o = instr_desc_bf16(ROWS, DH) | (1u << 16);       // B (= V) is MN-major
             bool ok = mbar_wait(bar_q, 0, abort_flag);

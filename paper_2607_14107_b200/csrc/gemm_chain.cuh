@@ -194,17 +194,17 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
         const int n_units = (int)(u_end - u_begin);
         const int pre = min(stages, n_units);
         int tile = (int)(u_begin / kb_total), kb = (int)(u_begin - (long long)tile * kb_total);
-        for (int i = 0; i < pre; ++i) {
-            const int it = p_units + i;
-            const int s = it % stages;
-            if (it >= stages && !mbar_wait(empty0 + 8 * s, ((uint32_t)(it / stages) & 1u) ^ 1u, abort_flag)) return;
+        Ring r(p_units, stages);
+        for (int i = 0; i < pre; ++i, r.next(stages)) {
+            const int s = r.slot;
+            if (p_units + i >= stages && !mbar_wait(empty0 + 8 * s, r.phase ^ 1u, abort_flag)) return;
             mbar_expect_tx(full0 + 8 * s, STAGE_BYTES);
             tma_load_2d_hint(smem_base + s * STAGE_BYTES + A_BYTES, &maps.w[p], full0 + 8 * s, 0, (tile * kb_total + kb) * BLOCK_F, pol);
             if (++kb == kb_total) { kb = 0; ++tile; }
         }
     };
 
-    if (warp == 0 && lane == 0) producer_weights_ahead(0);
+    if (warp == 0 && elect_one()) producer_weights_ahead(0);
 
     for (int p = 0; p < ca.n; ++p) {
         const ChainProb& P = ca.p[p];
@@ -213,7 +213,7 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
         const int n_units = (int)(u_end - u_begin);
 
         if (warp == 0) {
-            if (lane == 0) {
+            if (elect_one()) {
                 // ---- producer: activations of the slots whose weights are already on their way, then the rest
                 bool ok = true;
                 if (p == 0) pdl_wait();
@@ -223,15 +223,15 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
                 }
                 const int pre = min(stages, n_units);
                 int tile = (int)(u_begin / kb_total), kb = (int)(u_begin - (long long)tile * kb_total);
-                for (int i = 0; i < pre && ok; ++i) {
-                    const int s = (p_units + i) % stages;
+                Ring r(p_units, stages);
+                for (int i = 0; i < pre && ok; ++i, r.next(stages)) {
+                    const int s = r.slot;
                     tma_load_2d(smem_base + s * STAGE_BYTES, &maps.a[p], full0 + 8 * s, kb * BLOCK_K, 0);
                     if (++kb == kb_total) { kb = 0; ++tile; }
                 }
-                for (int i = pre; i < n_units && ok; ++i) {
-                    const int it = p_units + i;
-                    const int s = it % stages;
-                    if (it >= stages && !mbar_wait(empty0 + 8 * s, ((uint32_t)(it / stages) & 1u) ^ 1u, abort_flag)) break;
+                for (int i = pre; i < n_units && ok; ++i, r.next(stages)) {
+                    const int s = r.slot;
+                    if (p_units + i >= stages && !mbar_wait(empty0 + 8 * s, r.phase ^ 1u, abort_flag)) break;
                     const uint32_t dst = smem_base + s * STAGE_BYTES;
                     mbar_expect_tx(full0 + 8 * s, STAGE_BYTES);
                     tma_load_2d_hint(dst + A_BYTES, &maps.w[p], full0 + 8 * s, 0, (tile * kb_total + kb) * BLOCK_F, pol);
@@ -240,21 +240,23 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
                 }
                 p_units += n_units;
                 if (p + 1 < ca.n) producer_weights_ahead(p + 1);      // while this projection drains and reduces
+                p_units -= n_units;
             }
+            p_units += n_units;
         } else if (warp == 1) {
-            if (lane == 0) {
+            const bool issuer = elect_one();
+            if (issuer) {
                 const uint32_t idesc = instr_desc_bf16(BLOCK_T, BLOCK_F);
                 bool seg_start = true;
                 int kb = (int)(u_begin % kb_total);
-                for (int i = 0; i < n_units; ++i, kb = (kb + 1 == kb_total) ? 0 : kb + 1) {
-                    const int it = p_units + i;
-                    const int s = it % stages;
-                    const uint32_t ph = (uint32_t)(it / stages) & 1u;
+                Ring r(p_units, stages);
+                for (int i = 0; i < n_units; ++i, kb = (kb + 1 == kb_total) ? 0 : kb + 1, r.next(stages)) {
+                    const int s = r.slot;
                     if (seg_start && seg > 1) {
                         if (!mbar_wait(accum_empty + 8 * (seg & 1), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag)) break;
                         tc_fence_after();
                     }
-                    if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) break;
+                    if (!mbar_wait(full0 + 8 * s, r.phase, abort_flag)) break;
                     tc_fence_after();
                     const uint32_t sa = smem_base + s * STAGE_BYTES;
                     const uint64_t da = smem_desc_sw128(sa), dw = smem_desc_sw128(sa + A_BYTES);
@@ -270,8 +272,9 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
                         seg_start = true;
                     }
                 }
-                p_units += n_units;
             }
+            p_units += n_units;
+            seg = __shfl_sync(0xffffffffu, seg, __ffs(__ballot_sync(0xffffffffu, issuer)) - 1);     // the warp's other lanes keep in step
         } else if (warp < 6) {
             // ---- epilogue warps: TMEM lane = token, column = feature
             if (p == 0) pdl_wait();
@@ -369,9 +372,6 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
                 u = seg_end;
             }
         }
-        // the MMA warp's other lanes and the producer's keep the counters in step
-        if (warp == 0) p_units = __shfl_sync(0xffffffffu, p_units, 0);
-        if (warp == 1) { p_units = __shfl_sync(0xffffffffu, p_units, 0); seg = __shfl_sync(0xffffffffu, seg, 0); }
 
         // ---- reduction of the split tiles of projection p (all warps)
         if (n_units > 0) {

@@ -10,10 +10,9 @@
 //    These loads carry the evict_first L2 policy when every weight byte is used once per launch
 //    (a single token tile): a weight stream with the default policy pushed activations, partial tiles,
 //    the K/V cache and instruction lines out of L2 (14 % of the decode time).
-//  * One 128 x 256 x 16 MMA consumes 8 KB of weights and the tensor pipe issues one every ~150 ns at
-//    the rate HBM delivers them, so the instruction shape is made as large as it gets: M = 128 tokens
-//    x N = 256 features.  With the features on the small side of the instruction the tensor pipe, not
-//    HBM, was the limit (~4 TB/s).  Rows beyond the live tokens are out-of-bounds rows of the
+//  * One 128 x 256 x 16 MMA consumes 8 KB of weights and takes the tensor pipe 128 cycles, whatever part of its
+//    128 token rows is live: M = 128 tokens x N = 256 features is the shape that moves most weights per
+//    instruction.  Rows beyond the live tokens are out-of-bounds rows of the
 //    activation tensor map: TMA fills them with zeros without reading memory.
 //  * Schedule.  Tile ids are rasterised (tile_ft) so that consecutive ids form a compact block of the
 //    output.  With more tiles than CTAs, CTA c first takes the whole tiles c, c + G, ...: the grid
@@ -64,6 +63,25 @@ constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // ~2 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of a converged warp.  The single-thread roles (TMA producer, MMA issuer) branch on this rather than on
+// lane == 0: behind an elected branch the descriptors and barrier addresses stay in uniform registers.  Together with
+// ring positions that are counted instead of divided (Ring), the issuer's work per k block no longer limits the tensor
+// pipe: main loop alone (no loads, no epilogue), 128 x 256 x 16 MMAs: 215 -> 148 cycles each, where the pipe takes 128;
+// 1024 rows x 24576 features x 4096 with loads: 183 -> 156 us.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+// Position in a ring of operand slots: slot and the parity of its current use, for unit number `unit`.
+struct Ring {
+    int slot;
+    uint32_t phase;
+    __device__ __forceinline__ Ring(int unit, int stages) : slot(unit % stages), phase((uint32_t)(unit / stages) & 1u) {}
+    __device__ __forceinline__ void next(int stages) {
+        if (++slot == stages) { slot = 0; phase ^= 1u; }
+    }
+};
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -412,7 +430,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     }
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // weights do not depend on the previous kernel: request the first stages right away
             const int pre = min(g.stages, n_units);
             const uint64_t pol = l2_policy_evict_first();
@@ -465,10 +483,10 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                         tma_load_2d(smem_base + i * STAGE_T + hh * A_BYTES, &map_a, full0 + 8 * i, ia.kb * BLOCK_K, ia.t * BT + hh * BLOCK_T);
                 }
             }
-            for (int i = pre; i < n_units; ++i, advance(iw)) {
-                const int s = i % g.stages;
-                const uint32_t ph = (uint32_t)(i / g.stages) & 1u;
-                if (!mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag)) break;
+            Ring r(pre, g.stages);
+            for (int i = pre; i < n_units; ++i, advance(iw), r.next(g.stages)) {
+                const int s = r.slot;
+                if (!mbar_wait(empty0 + 8 * s, r.phase ^ 1u, abort_flag)) break;
                 const uint32_t dst = smem_base + s * STAGE_T;
                 if (PAIR) {
                     if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * STAGE_T);
@@ -485,16 +503,16 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = instr_desc_bf16(BLOCK_T * CG, BLOCK_F);
             int seg = 0;
             bool seg_start = true;
             const int tail_kb0 = (int)(u_begin % kb_total);
             const int dp_units = dp * kb_total;
             int kb = dp > 0 ? 0 : tail_kb0;
-            for (int i = 0; i < n_units; ++i, kb = (i == dp_units) ? tail_kb0 : ((kb + 1 == kb_total) ? 0 : kb + 1)) {
-                const int s = i % g.stages;
-                const uint32_t ph = (uint32_t)(i / g.stages) & 1u;
+            Ring r(0, g.stages);
+            for (int i = 0; i < n_units; ++i, kb = (i == dp_units) ? tail_kb0 : ((kb + 1 == kb_total) ? 0 : kb + 1), r.next(g.stages)) {
+                const int s = r.slot;
                 if (TT == 1 && seg_start && seg > 1) {
                     // the epilogue must have drained this buffer's previous segment (seg - 2)
                     if (!mbar_wait(accum_empty + 8 * (seg & 1), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag)) break;
@@ -505,7 +523,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                     if (!mbar_wait(accum_empty, (uint32_t)(seg - 1) & 1u, abort_flag)) break;
                     tc_fence_after();
                 }
-                if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) break;
+                if (!mbar_wait(full0 + 8 * s, r.phase, abort_flag)) break;
                 if (i == 0) SK_STAMP(3);
                 tc_fence_after();
                 const uint32_t sa = smem_base + s * STAGE_T;
