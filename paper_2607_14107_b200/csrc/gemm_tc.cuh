@@ -163,6 +163,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(bar_cluster), "r"(x), "r"(y)
         : "memory");
 }
+__device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int x, int y, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+        ::"r"(dst), "l"(map), "r"(bar_cluster), "r"(x), "r"(y), "l"(policy)
+        : "memory");
+}
 // D (256 x N, 128 rows in each CTA's tensor memory) += A (128 rows per CTA) x B (N / 2 rows per CTA); descriptors are
 // the issuing CTA's, the peer's operands sit at the same shared-memory offsets
 __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
@@ -228,7 +234,7 @@ __host__ __device__ inline uint32_t instr_desc_bf16(int m, int n) {
 struct SkArgs {
     int M, N_out, K, stages;
     int tiles_f, tiles_t;
-    float* partial;     // [2 * gridDim.x][tokens per CTA tile][BLOCK_F] fp32
+    float* partial;     // [2 * gridDim.x][BLOCK_T][BLOCK_F] fp32
     int* tile_counter;  // arrivals [tile] and, done_offset further on, finished shares [tile]; zero before
                         // launch, zero again after
     int done_offset;
@@ -301,19 +307,17 @@ __device__ __forceinline__ void red_add_v4(float* dst, uint32_t a, uint32_t b, u
                  "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
 }
 
-// TT = 128-row halves of a token tile.  TT = 2 (steps of several hundred rows, where the operands come from L2 and
-// the tensor pipe is the limit): a CTA tile is 256 tokens x 256 features, two MMAs per k step share one weight tile, so
-// a k block costs 64 KB of operands for twice the work of the 48 KB of TT = 1; both accumulators (2 x 256 columns) fill
-// the tensor memory, so the epilogue of a segment no longer overlaps the next segment's MMAs.
-//
-// CG = 2 (with TT = 1; launched as clusters of two CTAs): a CTA pair works on a tile of 256 tokens x 256 features.  Each
-// CTA loads its 128 tokens and HALF of the weight tile (128 features), the even CTA issues one MMA for both tensor cores
-// (tcgen05.mma.cta_group::2, M = 256), and each CTA ends up with its 128 tokens x 256 features in its own tensor memory:
-// 32 KB of operands per CTA and k block instead of 48, so six stages fit and the operand supply (bytes in flight against
-// the load latency) no longer limits the MMA rate, while the two accumulators keep the epilogue overlapped.  The schedule
+// CG = 2 (launched as clusters of two CTAs; every projection of more than 128 rows): a CTA pair works on a tile of 256
+// tokens x 256 features.  Each CTA loads its 128 tokens and HALF of the weight tile (128 features), the even CTA issues one
+// MMA for both tensor cores (tcgen05.mma.cta_group::2, M = 256), and each CTA ends up with its 128 tokens x 256 features in
+// its own tensor memory: 32 KB of operands per CTA and k block instead of 48, so six stages fit, and the two accumulators
+// keep the epilogue overlapped with the next segment's MMAs.  Bound by the tensor pipe, at full load by the power limit
+// (8192 x 24576 x 4096: 133 cycles per MMA without loads; with them 1.3 - 1.5 PFLOP/s at 1.4 - 1.5 GHz).  Measured against
+// two 128-row MMAs per k step on one CTA (256-token tile, no epilogue overlap; removed) and against 128-token tiles,
+// K = 4096: 256 x 12288 47 / 60 / 64 us, 512 x 24576 101 / 130 / 110 us, 896 x 24576 158 / 207 / 161 us.  The schedule
 // treats the pair as one CTA (stream-K ranges, whole tiles first); everything after the MMAs (epilogue, partial tiles,
 // reduction pass) is per CTA on its own 128 rows, with partial-tile slots and tile counters of its own.
-template <typename T, int EPI, int TT = 1, int CG = 1>
+template <typename T, int EPI, int CG = 1>
 __global__ void __launch_bounds__(FIX_THREADS, 1)
 gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_a,
                SkArgs g, EpiArgs e, PostArgs post, SelFuse sf) {
@@ -326,13 +330,11 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     __shared__ int fx_n;
     __shared__ volatile int fx_ready;
 
-    constexpr int BT = BLOCK_T * TT;                       // tokens per CTA tile
-    constexpr uint32_t A_BYTES_T = A_BYTES * TT;           // activations of a stage: TT boxes of [128][64]
+    constexpr int BT = BLOCK_T;                            // tokens per CTA tile
     constexpr uint32_t W_BYTES_C = W_BYTES / CG;           // weights of a stage in this CTA's shared memory
-    constexpr uint32_t STAGE_T = A_BYTES_T + W_BYTES_C;
+    constexpr uint32_t STAGE_T = A_BYTES + W_BYTES_C;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr bool PAIR = CG == 2;
-    static_assert(!PAIR || TT == 1, "CTA pairs take 128-token halves");
     const int rank = PAIR ? (int)(blockIdx.x & 1u) : 0;                  // CTA within its pair (cluster of two along x)
     // scheduling unit: a CTA, or a CTA pair (both CTAs of a pair run the same schedule)
     const int G = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x, cta = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
@@ -420,7 +422,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     }
 
     if constexpr (EPI == EPI_RESID) {
-        if (sf.on && cta == 0 && warp >= 6 && warp < 14) {
+        if (sf.on && blockIdx.x == 0 && warp >= 6 && warp < 14) {
             __shared__ float sel_dsh[SEL_SMALL_W];
             __shared__ int sel_flags[SEL_SMALL_W];
             __syncwarp();
@@ -457,17 +459,21 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             It iw = start();
             // pairs: the bytes of both CTAs' loads are counted on the even CTA's barrier, which alone expects them
             const uint32_t full_pair = PAIR ? mapa_u32(full0, 0) : 0u;
+            auto load_w_pair = [&](uint32_t dst, uint32_t bar, const It& it) {        // this CTA's 128 features of the weight tile
+                const int y = (it.f * kb_total + it.kb) * BLOCK_F + rank * (BLOCK_F / 2);
+                if (g.w_stream) tma_load_2d_pair_hint(dst, &map_w, bar, 0, y, pol);
+                else tma_load_2d_pair(dst, &map_w, bar, 0, y);
+            };
             for (int i = 0; i < pre; ++i, advance(iw)) {
                 if (PAIR) {
                     if (rank == 0) mbar_expect_tx(full0 + 8 * i, 2 * STAGE_T);
-                    tma_load_2d_pair(smem_base + i * STAGE_T + A_BYTES_T, &map_w, full_pair + 8 * i, 0,
-                                     (iw.f * kb_total + iw.kb) * BLOCK_F + rank * (BLOCK_F / 2));
+                    load_w_pair(smem_base + i * STAGE_T + A_BYTES, full_pair + 8 * i, iw);
                     continue;
                 }
                 mbar_expect_tx(full0 + 8 * i, STAGE_T);
-                if (g.w_stream) tma_load_2d_hint(smem_base + i * STAGE_T + A_BYTES_T, &map_w, full0 + 8 * i, 0,
+                if (g.w_stream) tma_load_2d_hint(smem_base + i * STAGE_T + A_BYTES, &map_w, full0 + 8 * i, 0,
                                                  (iw.f * kb_total + iw.kb) * BLOCK_F, pol);
-                else tma_load_2d(smem_base + i * STAGE_T + A_BYTES_T, &map_w, full0 + 8 * i, 0, (iw.f * kb_total + iw.kb) * BLOCK_F);
+                else tma_load_2d(smem_base + i * STAGE_T + A_BYTES, &map_w, full0 + 8 * i, 0, (iw.f * kb_total + iw.kb) * BLOCK_F);
             }
             pdl_wait();
             SK_STAMP(2);
@@ -478,9 +484,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                         tma_load_2d_pair(smem_base + i * STAGE_T, &map_a, full_pair + 8 * i, ia.kb * BLOCK_K, (ia.t * CG + rank) * BT);
                         continue;
                     }
-#pragma unroll
-                    for (int hh = 0; hh < TT; ++hh)
-                        tma_load_2d(smem_base + i * STAGE_T + hh * A_BYTES, &map_a, full0 + 8 * i, ia.kb * BLOCK_K, ia.t * BT + hh * BLOCK_T);
+                    tma_load_2d(smem_base + i * STAGE_T, &map_a, full0 + 8 * i, ia.kb * BLOCK_K, ia.t * BT);
                 }
             }
             Ring r(pre, g.stages);
@@ -490,16 +494,14 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 const uint32_t dst = smem_base + s * STAGE_T;
                 if (PAIR) {
                     if (rank == 0) mbar_expect_tx(full0 + 8 * s, 2 * STAGE_T);
-                    tma_load_2d_pair(dst + A_BYTES_T, &map_w, full_pair + 8 * s, 0, (iw.f * kb_total + iw.kb) * BLOCK_F + rank * (BLOCK_F / 2));
+                    load_w_pair(dst + A_BYTES, full_pair + 8 * s, iw);
                     tma_load_2d_pair(dst, &map_a, full_pair + 8 * s, iw.kb * BLOCK_K, (iw.t * CG + rank) * BT);
                     continue;
                 }
                 mbar_expect_tx(full0 + 8 * s, STAGE_T);
-                if (g.w_stream) tma_load_2d_hint(dst + A_BYTES_T, &map_w, full0 + 8 * s, 0, (iw.f * kb_total + iw.kb) * BLOCK_F, pol);
-                else tma_load_2d(dst + A_BYTES_T, &map_w, full0 + 8 * s, 0, (iw.f * kb_total + iw.kb) * BLOCK_F);
-#pragma unroll
-                for (int hh = 0; hh < TT; ++hh)
-                    tma_load_2d(dst + hh * A_BYTES, &map_a, full0 + 8 * s, iw.kb * BLOCK_K, iw.t * BT + hh * BLOCK_T);
+                if (g.w_stream) tma_load_2d_hint(dst + A_BYTES, &map_w, full0 + 8 * s, 0, (iw.f * kb_total + iw.kb) * BLOCK_F, pol);
+                else tma_load_2d(dst + A_BYTES, &map_w, full0 + 8 * s, 0, (iw.f * kb_total + iw.kb) * BLOCK_F);
+                tma_load_2d(dst, &map_a, full0 + 8 * s, iw.kb * BLOCK_K, iw.t * BT);
             }
         }
     } else if (warp == 1) {
@@ -513,36 +515,27 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             Ring r(0, g.stages);
             for (int i = 0; i < n_units; ++i, kb = (i == dp_units) ? tail_kb0 : ((kb + 1 == kb_total) ? 0 : kb + 1), r.next(g.stages)) {
                 const int s = r.slot;
-                if (TT == 1 && seg_start && seg > 1) {
+                if (seg_start && seg > 1) {
                     // the epilogue must have drained this buffer's previous segment (seg - 2)
                     if (!mbar_wait(accum_empty + 8 * (seg & 1), (uint32_t)((seg >> 1) - 1) & 1u, abort_flag)) break;
-                    tc_fence_after();
-                }
-                if (TT == 2 && seg_start && seg > 0) {
-                    // one pair of accumulators: the epilogue must have drained the previous segment
-                    if (!mbar_wait(accum_empty, (uint32_t)(seg - 1) & 1u, abort_flag)) break;
                     tc_fence_after();
                 }
                 if (!mbar_wait(full0 + 8 * s, r.phase, abort_flag)) break;
                 if (i == 0) SK_STAMP(3);
                 tc_fence_after();
                 const uint32_t sa = smem_base + s * STAGE_T;
-                const uint64_t dw = smem_desc_sw128(sa + A_BYTES_T);
+                const uint64_t da = smem_desc_sw128(sa), dw = smem_desc_sw128(sa + A_BYTES);
+                const uint32_t acc = tmem_base + (uint32_t)((seg & 1) * BLOCK_F);
 #pragma unroll
-                for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-#pragma unroll
-                    for (int hh = 0; hh < TT; ++hh) {
-                        if (PAIR)
-                            umma_bf16_pair(tmem_base + (uint32_t)((seg & 1) * BLOCK_F), smem_desc_sw128(sa) + (uint64_t)(k * 2),
-                                           dw + (uint64_t)(k * 2), idesc, (!seg_start || k > 0) ? 1u : 0u);
-                        else
-                            umma_bf16(tmem_base + (uint32_t)((TT == 1 ? (seg & 1) : hh) * BLOCK_F), smem_desc_sw128(sa + hh * A_BYTES) + (uint64_t)(k * 2),
-                                      dw + (uint64_t)(k * 2), idesc, (!seg_start || k > 0) ? 1u : 0u);
-                    }
+                for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
+                    const uint32_t add = (!seg_start || k > 0) ? 1u : 0u;
+                    if (PAIR) umma_bf16_pair(acc, da + (uint64_t)(k * 2), dw + (uint64_t)(k * 2), idesc, add);
+                    else umma_bf16(acc, da + (uint64_t)(k * 2), dw + (uint64_t)(k * 2), idesc, add);
+                }
                 if (PAIR) umma_commit_pair(empty0 + 8 * s); else umma_commit(empty0 + 8 * s);
                 seg_start = false;
                 if (kb == kb_total - 1 || i == n_units - 1) {
-                    if (PAIR) umma_commit_pair(accum_full + 8 * (seg & 1)); else umma_commit(accum_full + (TT == 1 ? 8 * (seg & 1) : 0));
+                    if (PAIR) umma_commit_pair(accum_full + 8 * (seg & 1)); else umma_commit(accum_full + 8 * (seg & 1));
                     if (i == n_units - 1) SK_STAMP(4);
                     ++seg;
                     seg_start = true;
@@ -577,90 +570,87 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             tile_ft(tile, g.tiles_f, g.tiles_t, tile_f, tile_t);
             const int n0 = tile_f * BLOCK_F;
             const bool whole = (k0 == 0 && k1 == kb_total);
-            if (!mbar_wait(accum_full + (TT == 1 ? 8 * (seg & 1) : 0), (uint32_t)(TT == 1 ? (seg >> 1) : seg) & 1u, abort_flag)) break;
+            if (!mbar_wait(accum_full + 8 * (seg & 1), (uint32_t)(seg >> 1) & 1u, abort_flag)) break;
             tc_fence_after();
             const int which = (k0 == 0) ? 1 : 0;     // slot 0: my range starts inside this tile
+            const int m = (tile_t * CG + rank) * BT + t_local;
+            const bool live = m < Mv;
+            const bool warp_live = (tile_t * CG + rank) * BT + q * 32 < Mv;      // any live token in this warp's quarter
+            const uint32_t taddr = taddr0 + (uint32_t)((seg & 1) * BLOCK_F);
+            if (whole) {
+                if (warp_live) {
+                    // this warp's 16-column chunks (dealt round-robin over the groups); the tensor-memory load
+                    // of the next chunk is in flight during the epilogue of the current one
+                    const int step = 16 * groups;
+                    int c0 = 16 * gi;
+                    uint32_t ra[16], rb[16];
+                    float v[16];
+                    if (c0 < BLOCK_F) tmem_ld16_issue(taddr + (uint32_t)c0, ra);
+                    while (c0 < BLOCK_F) {
+                        const int c1 = c0 + step;
+                        tmem_ld_wait16(ra);
+                        if (c1 < BLOCK_F) tmem_ld16_issue(taddr + (uint32_t)c1, rb);
+                        if (live) {
 #pragma unroll
-            for (int hh = 0; hh < TT; ++hh) {
-                const int m = (tile_t * CG + rank) * BT + hh * BLOCK_T + t_local;
-                const bool live = m < Mv;
-                const bool warp_live = (tile_t * CG + rank) * BT + hh * BLOCK_T + q * 32 < Mv;      // any live token in this warp's quarter
-                const uint32_t taddr = taddr0 + (uint32_t)((TT == 1 ? (seg & 1) : hh) * BLOCK_F);
-                if (whole) {
-                    if (warp_live) {
-                        // this warp's 16-column chunks of the half (dealt round-robin over the groups); the tensor-memory load
-                        // of the next chunk is in flight during the epilogue of the current one
-                        const int step = 16 * groups;
-                        int c0 = 16 * (((gi - hh * (BLOCK_F / 16)) % groups + groups) % groups);
-                        uint32_t ra[16], rb[16];
-                        float v[16];
+                            for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(ra[i]);
+                            epilogue16<T, EPI>(e, m, n0 + c0, v);
+                        }
+                        if (c1 >= BLOCK_F) break;
+                        c0 = c1 + step;
+                        tmem_ld_wait16(rb);
                         if (c0 < BLOCK_F) tmem_ld16_issue(taddr + (uint32_t)c0, ra);
-                        while (c0 < BLOCK_F) {
-                            const int c1 = c0 + step;
-                            tmem_ld_wait16(ra);
-                            if (c1 < BLOCK_F) tmem_ld16_issue(taddr + (uint32_t)c1, rb);
-                            if (live) {
+                        if (live) {
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(ra[i]);
-                                epilogue16<T, EPI>(e, m, n0 + c0, v);
-                            }
-                            if (c1 >= BLOCK_F) break;
-                            c0 = c1 + step;
-                            tmem_ld_wait16(rb);
-                            if (c0 < BLOCK_F) tmem_ld16_issue(taddr + (uint32_t)c0, ra);
-                            if (live) {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(rb[i]);
-                                epilogue16<T, EPI>(e, m, n0 + c1, v);
-                            }
+                            for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(rb[i]);
+                            epilogue16<T, EPI>(e, m, n0 + c1, v);
                         }
                     }
-                } else if ((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate) {
-                    // partial segment of a projection whose output rows are the residual rows: add it onto them in L2
-                    bool row_ok = live;
-                    float* dst = e.out_f32 + (size_t)m * e.ld_out + n0;
-                    if (EPI == EPI_DOWN && live) {
-                        const int r0 = e.list ? __ldcg(e.list + m) : m;
-                        const int4 rw = __ldg(reinterpret_cast<const int4*>(e.rows) + r0);       // {seq, pos, widx, aidx}
-                        row_ok = rw.y >= 0;
-                        dst = (e.within && rw.z >= 0) ? e.packet + ((size_t)rw.x * e.W_max + rw.z) * e.ld_out + n0
-                                                      : e.out_f32 + (size_t)r0 * e.ld_out + n0;
-                    }
-                    if (warp_live) {
-                        for (int c0 = 0; c0 < BLOCK_F; c0 += 64) {
-                            if ((hh * (BLOCK_F / 64) + (c0 >> 6)) % groups != gi) continue;
-                            uint32_t r[4][16];
+                }
+            } else if ((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate) {
+                // partial segment of a projection whose output rows are the residual rows: add it onto them in L2
+                bool row_ok = live;
+                float* dst = e.out_f32 + (size_t)m * e.ld_out + n0;
+                if (EPI == EPI_DOWN && live) {
+                    const int r0 = e.list ? __ldcg(e.list + m) : m;
+                    const int4 rw = __ldg(reinterpret_cast<const int4*>(e.rows) + r0);       // {seq, pos, widx, aidx}
+                    row_ok = rw.y >= 0;
+                    dst = (e.within && rw.z >= 0) ? e.packet + ((size_t)rw.x * e.W_max + rw.z) * e.ld_out + n0
+                                                  : e.out_f32 + (size_t)r0 * e.ld_out + n0;
+                }
+                if (warp_live) {
+                    for (int c0 = 0; c0 < BLOCK_F; c0 += 64) {
+                        if ((c0 >> 6) % groups != gi) continue;
+                        uint32_t r[4][16];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) tmem_ld16_issue(taddr + (uint32_t)(c0 + 16 * j), r[j]);
-                            tmem_ld_wait();
-                            if (row_ok) {
+                        for (int j = 0; j < 4; ++j) tmem_ld16_issue(taddr + (uint32_t)(c0 + 16 * j), r[j]);
+                        tmem_ld_wait();
+                        if (row_ok) {
 #pragma unroll
-                                for (int j = 0; j < 4; ++j)
+                            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                                    for (int c = 0; c < 16; c += 4)
-                                        red_add_v4(dst + c0 + 16 * j + c, r[j][c], r[j][c + 1], r[j][c + 2], r[j][c + 3]);
-                            }
+                                for (int c = 0; c < 16; c += 4)
+                                    red_add_v4(dst + c0 + 16 * j + c, r[j][c], r[j][c + 1], r[j][c + 2], r[j][c + 3]);
                         }
                     }
-                } else {
-                    // partial segment: publish it now, reduce later (pass 2), so that publishing never
-                    // waits on another CTA
-                    float* part = g.partial + ((size_t)(2 * slot_cta + which) * BT + hh * BLOCK_T + t_local) * BLOCK_F;
-                    if (warp_live) {
-                        // 64 columns per round trip to TMEM (four loads in flight, one wait)
-                        for (int c0 = 0; c0 < BLOCK_F; c0 += 64) {
-                            if ((hh * (BLOCK_F / 64) + (c0 >> 6)) % groups != gi) continue;
-                            uint32_t r[4][16];
+                }
+            } else {
+                // partial segment: publish it now, reduce later (pass 2), so that publishing never
+                // waits on another CTA
+                float* part = g.partial + ((size_t)(2 * slot_cta + which) * BT + t_local) * BLOCK_F;
+                if (warp_live) {
+                    // 64 columns per round trip to TMEM (four loads in flight, one wait)
+                    for (int c0 = 0; c0 < BLOCK_F; c0 += 64) {
+                        if ((c0 >> 6) % groups != gi) continue;
+                        uint32_t r[4][16];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) tmem_ld16_issue(taddr + (uint32_t)(c0 + 16 * j), r[j]);
-                            tmem_ld_wait();
-                            if (live) {
+                        for (int j = 0; j < 4; ++j) tmem_ld16_issue(taddr + (uint32_t)(c0 + 16 * j), r[j]);
+                        tmem_ld_wait();
+                        if (live) {
 #pragma unroll
-                                for (int j = 0; j < 4; ++j)
+                            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                                    for (int c = 0; c < 16; c += 4)
-                                        *reinterpret_cast<uint4*>(part + c0 + 16 * j + c) = make_uint4(r[j][c], r[j][c + 1], r[j][c + 2], r[j][c + 3]);
-                            }
+                                for (int c = 0; c < 16; c += 4)
+                                    *reinterpret_cast<uint4*>(part + c0 + 16 * j + c) = make_uint4(r[j][c], r[j][c + 1], r[j][c + 2], r[j][c + 3]);
                         }
                     }
                 }
@@ -669,7 +659,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             __syncwarp();
             if (lane == 0) {
                 if (PAIR) mbar_arrive_cluster(mapa_u32(accum_empty + 8 * (seg & 1), 0));      // the even CTA issues the MMAs
-                else mbar_arrive(accum_empty + (TT == 1 ? 8 * (seg & 1) : 0));
+                else mbar_arrive(accum_empty + 8 * (seg & 1));
             }
             if (!whole && !((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate)) {
                 __threadfence();

@@ -51,18 +51,11 @@ struct Switches {
     int refresh_simt = 0;    // POLESTAR_REFRESH_SIMT
     int fuse_prep = 0;       // POLESTAR_FUSE_PREP (measured negative result, kept with its test)
     int fold_norm = 0;       // POLESTAR_FOLD_NORM (same)
-    int tall_rows = 2048;    // POLESTAR_GEMM_TALL_ROWS: projections of at least this many rows use 256-token CTA tiles
-                             // (measured on the 4096-wide QKV projection alone: 4096 rows 0.72 -> 0.75 of the bf16 peak, 8192
-                             // rows 0.70 -> 0.79, 16384 rows 0.66 -> 0.78, 2048 rows 0.67 -> 0.64, 1024 rows 0.56 -> 0.51; in
-                             // the long-generation decode, whose refresh steps have 2048 rows, 335 -> 339 tokens/s with the
-                             // threshold at 2048, no change at 512)
-    int tall_rows_ffn = 512; // POLESTAR_GEMM_TALL_ROWS_FFN: the same threshold for the gate/up projection, whose epilogue is short
-                             // enough for the tall tile to pay from 512 rows on (follows POLESTAR_GEMM_TALL_ROWS when only that is set)
-    int one_tall = 1;        // POLESTAR_GEMM_ONE_TALL: projections of 129 - 256 rows run as one 256-token tile
     int accumulate = 1;      // POLESTAR_GEMM_ACCUMULATE: O / down projections of the chained kernel add their parts onto
                              // the residual rows in L2 (0: ordered reduction of published partial tiles, bit-reproducible)
     int chain_qkv = 0;       // POLESTAR_CHAIN_QKV (same)
-    int pair_rows = 1 << 30; // POLESTAR_GEMM_PAIR_ROWS: projections of at least this many rows run on CTA pairs (tcgen05 cta_group::2)
+    int pair_rows = tc::BLOCK_T + 1;   // POLESTAR_GEMM_PAIR_ROWS: projections of at least this many rows run on CTA pairs (tcgen05
+                             // cta_group::2); below, a single 128-token tile streams the weights on all SMs
     int epi_groups = 3;      // POLESTAR_GEMM_EPI_GROUPS: groups of four warps that drain an accumulator when a projection
                              // has several token tiles (1: the four epilogue warps alone)
     int l2promo = (int)CU_TENSOR_MAP_L2_PROMOTION_L2_128B;   // POLESTAR_TMA_L2PROMO
@@ -90,9 +83,6 @@ static Switches read_switches() {
     w.fuse_prep = env_int("POLESTAR_FUSE_PREP", w.fuse_prep);
     w.fold_norm = env_int("POLESTAR_FOLD_NORM", w.fold_norm);
     w.accumulate = env_int("POLESTAR_GEMM_ACCUMULATE", w.accumulate);
-    w.one_tall = env_int("POLESTAR_GEMM_ONE_TALL", w.one_tall);
-    w.tall_rows = env_int("POLESTAR_GEMM_TALL_ROWS", w.tall_rows);
-    w.tall_rows_ffn = env_int("POLESTAR_GEMM_TALL_ROWS_FFN", getenv("POLESTAR_GEMM_TALL_ROWS") ? w.tall_rows : w.tall_rows_ffn);
     w.chain_qkv = env_int("POLESTAR_CHAIN_QKV", w.chain_qkv);
     w.l2promo = env_int("POLESTAR_TMA_L2PROMO", w.l2promo);
     w.gemm_trace = env_int("POLESTAR_GEMM_TRACE", w.gemm_trace);
@@ -263,15 +253,11 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     if (M <= 0) return POLESTAR_OK;
     // weights: tile-major [chunks * 256][64]; activations: exactly M rows, so that the rows of a token tile
     // beyond M are out of bounds and arrive as zeros without being read
-    // Steps of several hundred rows (operands from L2, tensor-bound): CTA tiles of 256 tokens, two MMAs per k step on
-    // one weight tile (64 KB of operands per k block for twice the work of 48 KB)
-    // From POLESTAR_GEMM_PAIR_ROWS rows on: CTA pairs on tiles of 256 tokens (one MMA over both SMs, half a weight tile each)
-    const bool pair = ws.pairs > 0 && M >= ws.sw.pair_rows && !(sel && sel->on);
-    // (129 - 256 rows, e.g. a refresh step plus its proxy rows: one 256-token tile keeps the step a single token tile, so
-    // every weight byte is still read once and streamed with evict_first, instead of two token tiles sharing the weights)
-    const bool one_tall = M > tc::BLOCK_T && M <= 2 * tc::BLOCK_T && ws.sw.one_tall;
-    const int TT = (!pair && (one_tall || M >= (EPI == EPI_SWIGLU ? ws.sw.tall_rows_ffn : ws.sw.tall_rows))) ? 2 : 1;
-    const int BT = tc::BLOCK_T * (pair ? 2 : TT);          // tokens per scheduling unit's tile
+    // More than one token tile of 128 rows (POLESTAR_GEMM_PAIR_ROWS): CTA pairs on tiles of 256 tokens (one MMA over both SMs,
+    // half a weight tile each).  Up to 256 rows that is still a single token tile: every weight byte is read once and
+    // streamed with evict_first.
+    const bool pair = ws.pairs > 0 && M >= ws.sw.pair_rows;
+    const int BT = tc::BLOCK_T * (pair ? 2 : 1);           // tokens per scheduling unit's tile
     const int tiles_f = N_out / tc::BLOCK_F, tiles_t = (M + BT - 1) / BT;
     // When a multiple of the tile count fits on >= 85 % of the SMs, the grid takes it: CTA ranges then never
     // cross a tile boundary, so every CTA has one segment (one fix-up instead of two, or none at all).
@@ -295,7 +281,6 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     // flight, and less shared memory per block leaves room for the next kernel's blocks to become resident early); two
     // stages are 4 % slower.  Four stages when operands come from L2 (several token tiles).
     g.stages = std::max(2, std::min(4, ws.sw.stages > 0 ? ws.sw.stages : (tiles_t == 1 ? 3 : 4)));
-    if (TT == 2) g.stages = std::min(g.stages, 3);          // 64 KB per stage
     if (pair) g.stages = 6;                                 // 32 KB per stage and CTA
     g.partial = ws.partial; g.tile_counter = ws.counters; g.done_offset = ws.n_counters / 2; g.status = ws.status;
     g.w_stream = (g.tiles_t == 1 && ws.sw.evict_first) ? 1 : 0;
@@ -303,8 +288,7 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     // POLESTAR_TRACE builds: nanosecond stamps of the launches of one epilogue kind, kept in the tail of the partial workspace
     g.trace = (ws.sw.gemm_trace == EPI) ? (long long*)((char*)ws.partial + ws.partial_bytes - 16384) : nullptr;
     const size_t smem = pair ? (size_t)g.stages * (tc::A_BYTES + tc::W_BYTES / 2) + 1024
-                             : (size_t)g.stages * (tc::STAGE_BYTES + (TT - 1) * tc::A_BYTES) + 1024;
-    auto kern = TT == 2 ? tc::gemm_sk_kernel<__nv_bfloat16, EPI, 2> : tc::gemm_sk_kernel<__nv_bfloat16, EPI, 1>;
+                             : (size_t)g.stages * tc::STAGE_BYTES + 1024;
     const unsigned n_ctas = (unsigned)(pair ? 2 * G : G);
     PostArgs pa;
     memset(&pa, 0, sizeof(pa));
@@ -318,10 +302,10 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     if (sel) sfz = *sel; else memset(&sfz, 0, sizeof(sfz));
     if (sfz.on) g.epi_groups = 1;          // the selection runs on warps 6-13 of the first CTA
     if (pair) {
-        CK(launch_k_cluster(tc::gemm_sk_kernel<__nv_bfloat16, EPI, 1, 2>, dim3(n_ctas), dim3(tc::FIX_THREADS), smem, st, 2u, *mw, *ma, g, e, pa, sfz));
+        CK(launch_k_cluster(tc::gemm_sk_kernel<__nv_bfloat16, EPI, 2>, dim3(n_ctas), dim3(tc::FIX_THREADS), smem, st, 2u, *mw, *ma, g, e, pa, sfz));
         return POLESTAR_OK;
     }
-    CK(launch_k(kern, dim3((unsigned)G), dim3(tc::FIX_THREADS), smem, st, *mw, *ma, g, e, pa, sfz));
+    CK(launch_k(tc::gemm_sk_kernel<__nv_bfloat16, EPI>, dim3((unsigned)G), dim3(tc::FIX_THREADS), smem, st, *mw, *ma, g, e, pa, sfz));
     return POLESTAR_OK;
 }
 
@@ -427,7 +411,7 @@ struct Buffers {
 
 static const int CONF_CHUNKS = 32;
 static const int FORCED_COMMIT_MAX = 512;
-static const size_t GEMM_PARTIAL_BYTES = ((size_t)80 << 20) + 16384 + 65536;   // 2 slots x 148 CTAs x 256 x 256 fp32
+static const size_t GEMM_PARTIAL_BYTES = ((size_t)80 << 20) + 16384 + 65536;   // at least 2 slots x 148 CTAs x 128 x 256 fp32
 // One projection of a chained launch (gemm_chain.cuh): A [M, K] x W [N_out, K]^T with epilogue `epi`.
 struct ChainSpec {
     const void* A; const void* W;
@@ -724,7 +708,7 @@ static int resident_gemm_pairs() {
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV, 1, 2>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaOccupancyMaxActiveClusters(&n, tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV, 2>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
     return n;
 }
 
@@ -738,12 +722,6 @@ static cudaError_t set_kernel_attributes() {
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_DOWN>), gemm_smem);
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_LOGITS>), gemm_smem);
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV_REFRESH>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV, 1, 2>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_RESID, 1, 2>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_SWIGLU, 1, 2>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_DOWN, 1, 2>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_LOGITS, 1, 2>), gemm_smem);
-    PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV_REFRESH, 1, 2>), gemm_smem);
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV, 2>), gemm_smem);
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_RESID, 2>), gemm_smem);
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_SWIGLU, 2>), gemm_smem);
