@@ -678,6 +678,112 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 }
 
 // ---------------------------------------------------------------------------------------
+// The same product for fp32 models: 16 x 32 outputs per CTA, the K dimension split over the CTA's eight warps.
+// These models are small (tens of rows, K of a few hundred), so a launch is a latency chain, not a throughput problem:
+// 64 x 64 tiles leave most SMs idle and every 16-wide K slice is a round trip to L2.  Here the operands of three
+// 64-wide K slices are in flight at once (cp.async ring; the weights' share of it before the dependency wait), each
+// warp multiplies eight k of a slice, and the eight partial tiles are added in warp order through shared memory.
+// Rows / columns beyond the matrix and k beyond K arrive as zeros.  Needs K % 4 == 0 and 16-byte aligned operands.
+// Measured against 64 x 64 tiles (rows x columns x K): 32 x 768 x 256 5.6 / 29 us, 32 x 256 x 1024 11 / 109 us,
+// 128 x 2048 x 256 11 / 31 us, 512 x 2048 x 256 29 / 37 us, 4096 x 4096 x 1024 1160 / 1522 us: faster at every size, so the
+// 64 x 64 tiles above are left with bf16 operands and unaligned ones.
+// ---------------------------------------------------------------------------------------
+constexpr int LAT_TM = 16, LAT_TN = 32, LAT_KC = 64, LAT_STAGES = 4, LAT_LD = LAT_KC + 4;
+constexpr int LAT_SMEM = LAT_STAGES * (LAT_TM + LAT_TN) * LAT_LD * 4;
+__device__ __forceinline__ void cp_async16_zfill(float* dst, const float* src, bool ok) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int n = ok ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+template <int EPI>
+__global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__ A, const float* __restrict__ Wt,
+                                                       int M, int Nout, int K, EpiArgs e) {
+    constexpr int STAGE = (LAT_TM + LAT_TN) * LAT_LD;
+    static_assert(8 * LAT_TM * LAT_TN <= LAT_STAGES * STAGE, "the partial tiles reuse the operand ring");
+    extern __shared__ __align__(16) float lat_sm[];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int m0 = blockIdx.y * LAT_TM, n0 = blockIdx.x * LAT_TN;
+    const int slices = (K + LAT_KC - 1) / LAT_KC;
+    // thread t copies 16 bytes of A (row t / 16, k chunk t % 16) and twice 16 bytes of W (rows t / 16 and t / 16 + 16)
+    const int cr = t >> 4, ck = (t & 15) * 4;
+    auto load_w = [&](int s) {
+        const int k = s * LAT_KC + ck;
+        float* st = lat_sm + (s % LAT_STAGES) * STAGE + LAT_TM * LAT_LD;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int n = n0 + cr + 16 * i;
+            const bool ok = n < Nout && k < K;
+            cp_async16_zfill(st + (cr + 16 * i) * LAT_LD + ck, ok ? Wt + (size_t)n * K + k : Wt, ok);
+        }
+    };
+    auto load_a = [&](int s) {
+        const int k = s * LAT_KC + ck;
+        const bool ok = m0 + cr < M && k < K;
+        cp_async16_zfill(lat_sm + (s % LAT_STAGES) * STAGE + cr * LAT_LD + ck, ok ? A + (size_t)(m0 + cr) * K + k : A, ok);
+    };
+    pdl_trigger();
+    for (int s = 0; s < min(LAT_STAGES - 1, slices); ++s) load_w(s);       // no kernel of a forward writes weights
+    pdl_wait();
+    trace_stamp(7);
+    const int Mv = e.m_count ? min(M, *e.m_count) : M;
+    if (m0 >= Mv) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+    }
+    for (int s = 0; s < LAT_STAGES - 1; ++s) {
+        if (s < slices) load_a(s);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    const int mi = lane >> 3, ni = lane & 7;    // outputs: rows mi + 4 i, columns ni + 8 j
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int s = 0; s < slices; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(LAT_STAGES - 2) : "memory");
+        __syncthreads();                        // slice s has landed for every thread; the slot of slice s - 1 is free
+        if (s + LAT_STAGES - 1 < slices) { load_w(s + LAT_STAGES - 1); load_a(s + LAT_STAGES - 1); }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const float* as = lat_sm + (s % LAT_STAGES) * STAGE + warp * 8;
+        const float* ws = as + LAT_TM * LAT_LD;
+#pragma unroll
+        for (int kk = 0; kk < 8; kk += 4) {
+            float4 a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(as + (mi + 4 * i) * LAT_LD + kk);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(ws + (ni + 8 * j) * LAT_LD + kk);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    float* red = lat_sm + warp * (LAT_TM * LAT_TN);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) red[(mi + 4 * i) * LAT_TN + ni + 8 * j] = acc[i][j];
+    __syncthreads();
+    const int m = m0 + (t >> 4), n = n0 + (t & 15) * 2;
+    float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const float2 v = *reinterpret_cast<const float2*>(lat_sm + w * (LAT_TM * LAT_TN) + t * 2);
+        sum.x += v.x; sum.y += v.y;
+    }
+    if (m < Mv && n + 1 < Nout) epilogue_pair<float, EPI>(e, m, n, sum.x, sum.y);
+}
+
+// ---------------------------------------------------------------------------------------
 // Attention rows with drift, CUDA-core version: one warp per (row, head).
 //   logp_j = s_j - logsumexp(s), s_j = q.k_j / sqrt(dh) over all N cache rows (Eq. 3, no mask);
 //   out = sum_j p_j v_j;  recorded rows: kl = sum_j p_j (logp_j - prev_j), prev <- logp (Eq. 4).
@@ -733,10 +839,28 @@ __global__ void attention_simt_kernel(AttnArgs a) {
     const T* V = (const T*)a.vc + (size_t)seq * a.N * dkv + g * dh;
     // scores
     float mx = -INFINITY;
+    // (one warp per row and head: a chain of dependent loads.  fp32 heads of 32-multiples are read in 16-byte pieces,
+    // eight in flight; the products are added in the same order)
+    const bool vec = sizeof(T) == 4 && (dh & 31) == 0 && (dq & 3) == 0 && (dkv & 3) == 0 && (((uintptr_t)a.q | (uintptr_t)a.kc) & 15) == 0;
     for (int j = lane; j < a.N; j += 32) {
         const T* kj = K + (size_t)j * dkv;
         float s = 0.f;
-        for (int c = 0; c < dh; ++c) s = fmaf(to_f<T>(q[c]), to_f<T>(kj[c]), s);
+        if (vec) {
+            const float4* k4 = reinterpret_cast<const float4*>(kj);
+            const float4* q4 = reinterpret_cast<const float4*>(q);
+            for (int c = 0; c < (dh >> 2); c += 8) {
+                float4 kv[8], qv[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { kv[i] = k4[c + i]; qv[i] = q4[c + i]; }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    s = fmaf(qv[i].x, kv[i].x, s); s = fmaf(qv[i].y, kv[i].y, s);
+                    s = fmaf(qv[i].z, kv[i].z, s); s = fmaf(qv[i].w, kv[i].w, s);
+                }
+            }
+        } else {
+            for (int c = 0; c < dh; ++c) s = fmaf(to_f<T>(q[c]), to_f<T>(kj[c]), s);
+        }
         s *= a.scale;
         sc[j] = s;
         mx = fmaxf(mx, s);
@@ -765,7 +889,15 @@ __global__ void attention_simt_kernel(AttnArgs a) {
         T* o = (T*)a.out + (size_t)r * dq + h * dh;
         for (int c = lane; c < dh; c += 32) {
             float acc = 0.f;
-            for (int j = 0; j < a.N; ++j) acc = fmaf(sc[j], to_f<T>(V[(size_t)j * dkv + c]), acc);
+            int j = 0;
+            for (; j + 16 <= a.N; j += 16) {          // sixteen rows of V in flight, added in ascending order
+                T v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = V[(size_t)(j + i) * dkv + c];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) acc = fmaf(sc[j + i], to_f<T>(v[i]), acc);
+            }
+            for (; j < a.N; ++j) acc = fmaf(sc[j], to_f<T>(V[(size_t)j * dkv + c]), acc);
             o[c] = from_f<T>(acc);
         }
     }

@@ -220,6 +220,14 @@ static bool weight_is_tiled(int dtype, int n_out, int k) { return dtype == POLES
 template <typename T, int EPI>
 static int launch_gemm_simt(const void* A, const void* W, int M, int N_out, int K, const EpiArgs& e, cudaStream_t st) {
     if (M <= 0) return POLESTAR_OK;
+    if constexpr (sizeof(T) == 4) {
+        // fp32: the K-split kernel wherever its 16-byte loads apply
+        if (K % 4 == 0 && ((((uintptr_t)A | (uintptr_t)W)) & 15) == 0 && (M + LAT_TM - 1) / LAT_TM <= 65535) {
+            CK(launch_k(gemm_f32_kernel<EPI>, dim3((N_out + LAT_TN - 1) / LAT_TN, (M + LAT_TM - 1) / LAT_TM), dim3(256), (size_t)LAT_SMEM, st,
+                        (const float*)A, (const float*)W, M, N_out, K, e));
+            return POLESTAR_OK;
+        }
+    }
     dim3 grid((N_out + 63) / 64, (M + 63) / 64);
     const int w_tiled = weight_is_tiled(sizeof(T) == 2 ? POLESTAR_BF16 : POLESTAR_F32, N_out, K) ? 1 : 0;
     gemm_simt_kernel<T, EPI><<<grid, 256, 0, st>>>((const T*)A, (const T*)W, M, N_out, K, w_tiled, e);
@@ -730,6 +738,11 @@ static cudaError_t set_kernel_attributes() {
     PS_ATTR((tc::gemm_sk_kernel<__nv_bfloat16, EPI_QKV_REFRESH, 2>), gemm_smem);
     PS_ATTR(tc::gemm_chain_kernel<__nv_bfloat16>, gemm_smem);
     PS_ATTR(atc::attention_tc_kernel, (int)atc::smem_bytes(atc::MAX_KT));
+    PS_ATTR(gemm_f32_kernel<EPI_QKV>, LAT_SMEM);
+    PS_ATTR(gemm_f32_kernel<EPI_RESID>, LAT_SMEM);
+    PS_ATTR(gemm_f32_kernel<EPI_SWIGLU>, LAT_SMEM);
+    PS_ATTR(gemm_f32_kernel<EPI_DOWN>, LAT_SMEM);
+    PS_ATTR(gemm_f32_kernel<EPI_LOGITS>, LAT_SMEM);
     PS_ATTR(kmeans_kernel, KM_SMEM_BYTES);
     PS_ATTR(ast::attention_stream_kernel, (int)ast::smem_bytes());
     PS_ATTR(attention_simt_kernel<float>, (int)SIMT_ATTN_SMEM_MAX);

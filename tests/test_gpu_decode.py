@@ -497,3 +497,48 @@ def test_call_order_errors():
         gpu.step()
     assert e.value.code == Bd.E_DONE
     assert not (gpu.tokens() == m.mask_id).any()
+
+
+@pytest.mark.parametrize("kw", [
+    dict(d_model=200, n_heads=3, n_kv_heads=1, head_dim=40, d_ffn=328, vocab=1030, mask_id=1029, eos_id=1028),     # K of 200 / 120 / 328: a last slice of 8, 56, 8; N % 32 != 0
+    dict(d_model=64, n_heads=1, n_kv_heads=1, head_dim=32, d_ffn=8, vocab=34, mask_id=33, eos_id=32),          # a single slice of 64, 32 and 8; fewer columns than a tile
+    dict(d_model=512, n_heads=2, n_kv_heads=2, head_dim=96, d_ffn=1096, vocab=514, mask_id=513, eos_id=512),     # more slices than the operand ring holds
+])
+def test_c1_projection_edges(kw):
+    # fp32 projections: remainders of the K slices and of the 16 x 32 tiles (block 20: 20 and 80 rows), GQA
+    seen = run_forced("c1", 8, model=kw, tau_upd=1, logit_scale=12.0, prompt_len=37, gen_len=40, block=20, max_steps=8)
+    assert seen["refresh"] > 0
+
+
+@pytest.mark.parametrize("frac", [0.0, 0.25, 1.0])
+@pytest.mark.parametrize("batch", [1, 3])
+def test_c1b_free_selection_equals_the_same_selection_imposed(batch, frac):
+    # an imposed selection lays the feed-forward projections out for every row of the step, a top-k selection for the rows
+    # it can have: the same rows must come out (the order in which partial products meet differs, hence bf16 tolerance)
+    m, p = I.config("c1b")
+    p = dataclasses.replace(p, batch=batch, prompt_len=70, gen_len=128, block=64, max_steps=16, tau_upd=-1, select_frac=frac)
+    packed, prompt = Bd.pack_weights(m, I.make_weights(m)), I.make_prompt(m, p).numpy()
+    free, imposed = Bd.Polestar(m, packed, p, prompt), Bd.Polestar(m, packed, p, prompt)
+    free.commit()
+    got = free.tokens()[:, p.prompt_len:]
+    pos = np.full((batch, p.gen_len), -1, np.int32)
+    tok = np.full((batch, p.gen_len), -1, np.int32)
+    for s in range(batch):              # near-ties of random logits may fall either way: both sides commit the same tokens
+        done = np.nonzero(got[s] != m.mask_id)[0]
+        pos[s, :len(done)], tok[s, :len(done)] = p.prompt_len + done, got[s, done]
+    imposed.force_commit(pos, tok)
+    imposed.commit()
+    assert np.array_equal(free.tokens(), imposed.tokens())
+    free.step()
+    for l in range(m.n_layers):
+        cnt, idx = free.read(Bd.READ_SEL_COUNT, l), free.read(Bd.READ_SEL_IDX, l)
+        sel = np.full((batch, free.W_max), -1, np.int32)
+        for s in range(batch):
+            sel[s, :cnt[s]] = idx[s, :cnt[s]]
+        assert cnt.max() <= int(frac * free.W_max + 0.5)
+        imposed.force_select(l, sel)
+    imposed.step()
+    for what in (Bd.READ_LOGITS, Bd.READ_KCACHE, Bd.READ_VCACHE):
+        a, b = free.read(what, m.n_layers - 1 if what != Bd.READ_LOGITS else 0), imposed.read(what, m.n_layers - 1 if what != Bd.READ_LOGITS else 0)
+        close(a, b, TOL[m.dtype], f"{what}")
+    free.destroy(); imposed.destroy()
