@@ -996,18 +996,35 @@ __device__ int select_one(const float* D, int W, int mode, int k, float thresh, 
             __syncthreads();
             const unsigned prefix = s.prefix;
 #pragma unroll
-            for (int u = 0; u < SEL_ITEMS; ++u)
-                if (cand[u] && (key[u] & himask) == prefix) atomicAdd(&s.hist[(key[u] >> shift) & 255u], 1);
+            for (int u = 0; u < SEL_ITEMS; ++u) {
+                // (one addition per distinct bucket of a warp: drift values share their leading bytes)
+                const bool in = cand[u] && (key[u] & himask) == prefix;
+                const unsigned bkt = in ? (key[u] >> shift) & 255u : 256u;
+                const unsigned same = __match_any_sync(0xffffffffu, bkt);
+                if (in && (t & 31) == __ffs(same) - 1) atomicAdd(&s.hist[bkt], __popc(same));
+            }
             __syncthreads();
-            if (t == 0) {
-                int left = s.kleft, bsel = 0;
-                for (int bkt = 255; bkt >= 0; --bkt) {
-                    const int c = s.hist[bkt];
-                    if (c >= left) { bsel = bkt; break; }
-                    left -= c;
+            if (t < 32) {
+                // the bucket that holds the k-th candidate, from the top: lane t owns buckets 255 - 8 t ... 248 - 8 t
+                int c[8], sum = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { c[j] = s.hist[255 - 8 * t - j]; sum += c[j]; }
+                int inc = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int up = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (t >= o) inc += up;
                 }
-                s.kleft = left;
-                s.prefix = prefix | ((unsigned)bsel << shift);
+                int left = s.kleft;
+                __syncwarp();
+                if (inc - sum < left && inc >= left) {        // (one lane: the counts add up to at least k)
+                    left -= inc - sum;
+                    int j = 0;
+#pragma unroll
+                    for (int i = 0; i < 7; ++i) if (j == i && c[i] < left) { left -= c[i]; ++j; }
+                    s.kleft = left;
+                    s.prefix = prefix | ((unsigned)(255 - 8 * t - j) << shift);
+                }
             }
             __syncthreads();
         }
