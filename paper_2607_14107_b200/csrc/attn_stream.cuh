@@ -9,11 +9,12 @@
 //            the row's log-sum-exp
 //   pass 2   S_t again (K comes back through the ring, from L2); p = 2^(t - lse), normalised BEFORE it is rounded
 //            to bf16 (the rounding point of a plain implementation), the drift sum A = sum p (s - s_old) against the
-//            stored row, the new stored row s, and P into shared memory as the A operand of O += P V_t (V as an
+//            stored row, the new stored row s, and P into tensor memory as the A operand of O += P V_t (V as an
 //            MN-major operand, accumulated in tensor memory over the tiles); S_{t+1} is computed while the
 //            warps work on S_t
-//   rows     the stored rows move as 512-byte bulk copies per row and tile between global memory and a staging tile
-//            in shared memory: the statistics warps never wait on global memory
+//   rows     the stored rows move as tensor boxes (or 512-byte bulk copies per row) between global memory and two staging
+//            tiles in shared memory: the statistics warps never wait on global memory.  Q and P are tensor-memory operands
+//            to make room for the second staging tile
 //   end      O from tensor memory to the output rows, KL = A - (lse - lse_old)
 //
 // Computing S twice costs tensor time (which this kernel has to spare) and saves the rescaling of a running
@@ -30,11 +31,34 @@ using namespace atc;
 constexpr int THREADS = 576;              // warp 0: TMA, warp 1: MMA + tensor memory, warps 2..17: statistics / epilogue
 constexpr int NS = 2;                     // slots of the operand ring (K and V tiles in the order the tensor core uses them)
 constexpr uint32_t XPITCH = 512 + 16;     // bytes per row of the stored-row staging tile (the pad spreads the rows over the banks)
-constexpr uint32_t X_BYTES = ROWS * XPITCH;
+constexpr uint32_t XQ_BYTES = 17 * 1024;  // a lane quarter's share of a staging tile: 32 rows of XPITCH bytes, or four swizzled [32 rows][32 keys] boxes
+constexpr uint32_t XBOX_BYTES = 32 * 128;
+constexpr uint32_t X_BYTES = 4 * XQ_BYTES;
+static_assert(32 * XPITCH <= XQ_BYTES && 4 * XBOX_BYTES <= XQ_BYTES, "staging tile");
 constexpr uint32_t TILE_BYTES = 2 * BOX_BYTES;       // [128][128] bf16 as two [128][64] boxes
-constexpr uint32_t TMEM_COLS = 512;       // S0, S1, O (128 columns each)
+// Tensor memory: S0, S1, O (128 fp32 columns each), P and Q (two bf16 per column).  Both A operands live there, which
+// leaves shared memory for two staging tiles.
+constexpr uint32_t TMEM_COLS = 512, COL_O = 2 * KEYS, COL_P = COL_O + DH, COL_Q = COL_P + KEYS / 2;
+static_assert(COL_Q + DH / 2 <= TMEM_COLS, "tensor memory");
 
-__host__ __device__ constexpr size_t smem_bytes() { return (size_t)(2 + NS) * TILE_BYTES + X_BYTES + 1024; }     // Q, P, ring, X
+__host__ __device__ constexpr size_t smem_bytes() { return (size_t)NS * TILE_BYTES + 2 * X_BYTES + 1024; }     // ring, X0, X1
+
+// A from tensor memory (lane = row, K-major, two bf16 per column), B from shared memory
+__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// 16 columns of this thread's lane, complete on return (the whole warp calls)
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 
 __device__ __forceinline__ void bar_sync_stat() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 // one row segment global -> shared (bytes counted on the mbarrier) and shared -> global (bulk group); 16-byte aligned
@@ -46,24 +70,31 @@ __device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t byt
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
 }
 
+// [32 rows][32 keys] boxes of the stored rows (128-byte swizzle in shared memory)
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
+                 ::"l"(map), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
+}
+
 struct Args {
     AttnArgs a;
+    int maps;               // bit 0: map_p describes a.pprev, bit 1: map_r describes a.aprev (else null rows or unaligned: plain path)
     int rows_per_seq;       // forward rows per sequence (stand-alone: n_rows)
     int tiles_per_seq;      // 128-row tiles per sequence
     int* status;            // set to 1 when a bounded wait gave up (null: nowhere to report)
 };
 
 __global__ void __launch_bounds__(THREADS, 1)
-attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                        const __grid_constant__ CUtensorMap map_v, Args g) {
+attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                        const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r, Args g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars[4 + 2 * NS + 4 + 2];
-    __shared__ int cta_prev_sh;                    // any row of this CTA records
+    __shared__ uint64_t bars[4 + 2 * NS + 4 + 8 + 4];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     __shared__ float* prev_sh[ROWS];
     __shared__ float* lsep_sh[ROWS];
     __shared__ int valid_sh[ROWS];
+    __shared__ int box_row_sh[4], box_map_sh[4];   // lane quarters whose 32 stored rows are consecutive: first row, which map (-1: not so)
     __shared__ float2 part_ml[4][ROWS];            // (maximum, sum) of each column quarter
     __shared__ float part_A[3][ROWS];              // drift sums of the upper three column quarters
 
@@ -80,24 +111,23 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t smem_base = smem_u32(smem);
-    const uint32_t q_s = smem_base, p_s = smem_base + TILE_BYTES;
-    auto ring_s = [&](int s) { return smem_base + (uint32_t)(2 + s) * TILE_BYTES; };
+    auto ring_s = [&](int s) { return smem_base + (uint32_t)s * TILE_BYTES; };
     const uint32_t bar_q = smem_u32(&bars[0]), bar_o = smem_u32(&bars[1]), bar_pfull = smem_u32(&bars[2]), bar_pfree = smem_u32(&bars[3]);
     auto bar_full = [&](int s) { return smem_u32(&bars[4 + s]); };
     auto bar_free = [&](int s) { return smem_u32(&bars[4 + NS + s]); };
     auto bar_sfull = [&](int s) { return smem_u32(&bars[4 + 2 * NS + s]); };
     auto bar_sfree = [&](int s) { return smem_u32(&bars[6 + 2 * NS + s]); };
-    const uint32_t bar_x = smem_u32(&bars[8 + 2 * NS]), bar_w = smem_u32(&bars[9 + 2 * NS]);
-    const uint32_t x_s = smem_base + (uint32_t)(2 + NS) * TILE_BYTES;
+    // staging tiles, per lane quarter (32 rows, the four warps that share them): "X_b may be worked on", "the warps are done with it"
+    auto bar_x = [&](int b, int q) { return smem_u32(&bars[8 + 2 * NS + 4 * b + q]); };
+    auto bar_w = [&](int q) { return smem_u32(&bars[16 + 2 * NS + q]); };
+    auto x_s = [&](int b) { return smem_base + (uint32_t)NS * TILE_BYTES + (uint32_t)b * X_BYTES; };
 
     if (threadIdx.x == 0) {
-        mbar_init(bar_q, 1); mbar_init(bar_o, 1); mbar_init(bar_pfull, 16); mbar_init(bar_pfree, 1);
+        mbar_init(bar_q, 16); mbar_init(bar_o, 1); mbar_init(bar_pfull, 16); mbar_init(bar_pfree, 1);
         for (int s = 0; s < NS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_free(s), 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(bar_sfull(s), 1); mbar_init(bar_sfree(s), 16); }
-        mbar_init(bar_x, ROWS);
-        mbar_init(bar_w, 16);
+        for (int q = 0; q < 4; ++q) { mbar_init(bar_x(0, q), 32); mbar_init(bar_x(1, q), 32); mbar_init(bar_w(q), 4); }
         abort_sh = 0;
-        cta_prev_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -144,10 +174,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 if (!clean(unit_tile(u, is_v))) break;
                 load(u);
             }
-            pdl_wait();      // q, and the K / V rows written this step, come from the projection that ran just before
+            pdl_wait();      // the K / V rows written this step come from the projection that ran just before
             trace_stamp(7);
-            mbar_expect_tx(bar_q, TILE_BYTES);
-            for (int kb = 0; kb < 2; ++kb) tma_load_2d(q_s + kb * BOX_BYTES, &map_q, bar_q, h * DH + kb * 64, row0);
             for (; u < 3 * n && ok; ++u) {
                 if (u >= NS) ok = mbar_wait(bar_free(u % NS), (uint32_t)(u / NS - 1) & 1u, abort_flag);
                 if (ok) load(u);
@@ -157,7 +185,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         if (elect_one()) {
             const uint32_t idesc_s = instr_desc_bf16(ROWS, KEYS);
             const uint32_t idesc_o = instr_desc_bf16(ROWS, DH) | (1u << 16);       // B (= V) is MN-major
-            bool ok = mbar_wait(bar_q, 0, abort_flag);
+            bool ok = mbar_wait(bar_q, 0, abort_flag);          // q is in tensor memory
             int u = 0;                   // operand units consumed so far
             auto take = [&]() {          // next unit of the ring: its slot, once the tile has landed
                 const int sl = u % NS;
@@ -172,9 +200,8 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < DH / UMMA_K; ++k) {
-                    const uint64_t da = smem_desc_sw128(q_s + (k >> 2) * BOX_BYTES) + (uint64_t)((k & 3) * 2);
                     const uint64_t db = smem_desc_sw128(ring_s(sl) + (k >> 2) * BOX_BYTES) + (uint64_t)((k & 3) * 2);
-                    umma_bf16(tmem_base + (uint32_t)(b * KEYS), da, db, idesc_s, k > 0 ? 1u : 0u);
+                    umma_bf16_ta(tmem_base + (uint32_t)(b * KEYS), tmem_base + COL_Q + (uint32_t)(k * (UMMA_K / 2)), db, idesc_s, k > 0 ? 1u : 0u);
                 }
                 umma_commit(bar_free(sl));
                 umma_commit(bar_sfull(b));
@@ -189,10 +216,9 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < KEYS / UMMA_K; ++k) {
-                    // A = P: K-major, 64 keys per 128-byte row;  B = V_j: 16 keys = two 8-row groups further down
-                    const uint64_t da = smem_desc_sw128(p_s + (k >> 2) * BOX_BYTES) + (uint64_t)((k & 3) * 2);
+                    // B = V_j: 16 keys = two 8-row groups further down
                     const uint64_t db = smem_desc_mn_sw128(ring_s(sl) + (uint32_t)k * 2048u, BOX_BYTES);
-                    umma_bf16(tmem_base + 2u * KEYS, da, db, idesc_o, (j > 0 || k > 0) ? 1u : 0u);
+                    umma_bf16_ta(tmem_base + COL_O, tmem_base + COL_P + (uint32_t)(k * (UMMA_K / 2)), db, idesc_o, (j > 0 || k > 0) ? 1u : 0u);
                 }
                 umma_commit(bar_free(sl));
                 umma_commit(bar_pfree);
@@ -209,7 +235,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         pdl_wait();            // the row table, q and the stored rows all come from earlier kernels of the stream
         if (cq == 0) {
             float* prev = nullptr; float* lsep = nullptr;
-            int valid = 0;
+            int valid = 0, stored = -1, arr = -1;              // index of the stored row, 0: pprev, 1: aprev
             if (row < n_in_tile) {
                 const int r = row0 + row;
                 if (a.rows) {
@@ -220,19 +246,42 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                             // recorded drift rows: the window rows, or (centroid proxies) the clusters' proxy rows
                             const size_t i = a.cluster_K > 0 ? ((size_t)rw.x * a.cluster_K + row_cluster(rw.z)) * a.n_heads + h
                                                              : ((size_t)rw.x * a.W_max + rw.z) * a.n_heads + h;
-                            prev = a.pprev + i * a.N; lsep = a.pprev_lse + i;
+                            prev = a.pprev + i * a.N; lsep = a.pprev_lse + i; stored = (int)(i / a.n_heads); arr = 0;
                         } else if (rw.w >= 0 && a.aprev) {
                             const size_t i = ((size_t)rw.x * a.B + rw.w) * a.n_heads + h;
-                            prev = a.aprev + i * a.N; lsep = a.aprev_lse + i;
+                            prev = a.aprev + i * a.N; lsep = a.aprev_lse + i; stored = (int)(i / a.n_heads); arr = 1;
                         }
                     }
                 } else {
                     valid = 1;
-                    if (a.pprev) { const size_t i = (size_t)r * a.n_heads + h; prev = a.pprev + i * a.N; lsep = a.pprev_lse + i; }
+                    if (a.pprev) { const size_t i = (size_t)r * a.n_heads + h; prev = a.pprev + i * a.N; lsep = a.pprev_lse + i; stored = r; arr = 0; }
                 }
             }
             prev_sh[row] = prev; lsep_sh[row] = lsep; valid_sh[row] = valid;
-            if (prev) cta_prev_sh = 1;
+            // (rows behind the last one of a stand-alone call lie outside its map: loads fill, stores leave them out)
+            const int s0 = __shfl_sync(0xffffffffu, stored, 0), arr0 = __shfl_sync(0xffffffffu, arr, 0);
+            const bool run = __all_sync(0xffffffffu, (stored == s0 + lane && arr == arr0) || (!a.rows && s0 >= 0 && s0 + lane >= a.n_rows)) != 0;
+            if (lane == 0) { box_row_sh[quarter] = s0; box_map_sh[quarter] = (run && s0 >= 0 && ((g.maps >> arr0) & 1)) ? arr0 : -1; }
+        }
+        {
+            // this thread's 32 channels of its row of q, straight into tensor memory
+            uint32_t qw[16];
+            if (row < n_in_tile) {
+                const uint4* src = reinterpret_cast<const uint4*>((const __nv_bfloat16*)a.q + (size_t)(row0 + row) * dq + h * DH + cq * 32);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 v = __ldcg(src + i);
+                    qw[4 * i] = v.x; qw[4 * i + 1] = v.y; qw[4 * i + 2] = v.z; qw[4 * i + 3] = v.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) qw[i] = 0u;
+            }
+            __syncwarp();
+            tmem_st16(taddr0 + COL_Q + (uint32_t)(cq * 16), qw);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_q);
         }
         bar_sync_stat();
         float* const prev = prev_sh[row];
@@ -240,14 +289,46 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         // tensor-memory loads are warp-wide (.sync.aligned): whether a warp reads at all is decided per warp
         const bool warp_valid = __any_sync(0xffffffffu, valid) != 0;
         const bool use_old = prev != nullptr && a.record_kl != 0;
-        const bool vec = (a.N & 3) == 0;
+        const bool vec = (a.N & 3) == 0 && (((uintptr_t)a.pprev | (uintptr_t)a.aprev) & 15) == 0;
         // stored rows are handled a warp at a time: nothing of it runs in a warp none of whose rows is recorded
         const bool warp_prev = __any_sync(0xffffffffu, prev != nullptr) != 0;
-        const bool warp_old = warp_prev && a.record_kl != 0;
         float lse_old = 0.f;
         if (cq == 0 && lsep_sh[row] && a.record_kl) lse_old = __ldcg(lsep_sh[row]);
         const float scale2 = a.scale * LOG2E_F;
         bool ok = true;
+
+        // Stored rows travel through two staging tiles X_0 / X_1 in shared memory, a lane quarter (32 rows, four warps) at a
+        // time: the statistics warps never touch global memory, and DRAM sees whole row segments.  A quarter whose 32 stored
+        // rows are consecutive moves them as swizzled [32 rows][32 keys] tensor boxes (four copies per tile), any other as
+        // one 512-byte bulk copy per row, issued by the row's first thread.  "X_b may be worked on for tile j" is phase
+        // j / 2 of bar_x(b, quarter): the quarter's 32 first threads arrive on it once the store of tile j - 2 has read X_b,
+        // together with the bytes of the old rows of tile j when there are any: tile j + 1 is on its way while tile j is
+        // worked on.  2048 rows x 2048 keys x 32 heads, rows read and written: one staging tile and row copies 434 us, two
+        // 381, boxes 293 (without any stored rows: 159); 256 x 2048: 102 / 94 / 74.  Rows whose length is not a multiple of four floats (no 16-byte alignment) go the plain way:
+        // every thread reads and writes its own row segment.
+        const bool use_x = vec && warp_prev;                     // (the same in the four warps of a quarter, like everything here)
+        const bool boxes = use_x && box_map_sh[quarter] >= 0;
+        const CUtensorMap* const map_x = box_map_sh[quarter] == 1 ? &map_r : &map_p;
+        auto x_quarter = [&](int b) { return x_s(b) + (uint32_t)quarter * XQ_BYTES; };
+        auto x_ready = [&](int j) {         // first threads: X may take tile j; request the old rows if there are any
+            const int b = j & 1, keys = min(KEYS, a.N - j * KEYS);
+            if (boxes) {
+                if (lane == 0 && a.record_kl) {
+                    const int nb = (keys + 31) >> 5;
+                    mbar_expect_tx(bar_x(b, quarter), (uint32_t)nb * XBOX_BYTES);
+                    for (int c = 0; c < nb; ++c)
+                        tma_load_3d(x_quarter(b) + (uint32_t)c * XBOX_BYTES, map_x, bar_x(b, quarter), j * KEYS + 32 * c, h, box_row_sh[quarter]);
+                } else {
+                    mbar_arrive(bar_x(b, quarter));
+                }
+            } else if (use_old) {
+                mbar_expect_tx(bar_x(b, quarter), (uint32_t)keys * 4u);
+                bulk_load(x_quarter(b) + (uint32_t)lane * XPITCH, prev + j * KEYS, (uint32_t)keys * 4u, bar_x(b, quarter));
+            } else {
+                mbar_arrive(bar_x(b, quarter));
+            }
+        };
+        if (use_x && cq == 0) { x_ready(0); if (n > 1) x_ready(1); }
 
         // ---- pass 1: running (maximum, sum) of this thread's columns (four independent chains each: two or four warps
         // per scheduler cannot hide one long dependent chain) ----
@@ -259,12 +340,6 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             if (!ok) break;
             tc_fence_after();
             const int kb = t * KEYS + cq * 32;
-            if (use_old && vec && cq == 0 && (t & 3) == 0) {
-                // pass 2 will want the stored row: bring it into L2 in pieces of four tiles (2 KB contiguous per row:
-                // a DRAM page is opened for more than a sector or two)
-                const int c0 = t * KEYS, nb = min(4 * KEYS, a.N - c0) * 4;
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(prev + c0), "r"(nb) : "memory");
-            }
             if (warp_valid) {
                 uint32_t r[2][16];
 #pragma unroll
@@ -323,26 +398,11 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         }
 
         // ---- pass 2: probabilities (normalised before they are rounded to bf16), P, then drift sum and the new stored row ----
-        // Stored rows travel as bulk copies between global memory and the staging tile X (one 512-byte segment per row
-        // and tile, issued by the row's first thread): the statistics warps only ever touch shared memory, and DRAM
-        // sees whole row segments.  "X is ready for tile j" is phase j of bar_x: the 128 issuing threads arrive on it
-        // once the bulk store of tile j - 1 has read their row out of X, together with the bytes of the old row of
-        // tile j when there is one.  Rows whose length is not a multiple of four floats (no 16-byte alignment) go the
-        // plain way: every thread reads and writes its own row segment.
         float A4[4] = {0.f, 0.f, 0.f, 0.f};
         const float neg_lse2 = -lse2;
-        const bool use_x = vec && cta_prev_sh != 0;              // (the same in every thread of the CTA)
-        const uint32_t x_row = x_s + (uint32_t)row * XPITCH + (uint32_t)cq * 128u;
-        auto x_ready = [&](int j) {         // row's first thread: X may take tile j; request the old row segment if there is one
-            const int nb = min(KEYS, a.N - j * KEYS) * 4;
-            if (use_old) {
-                mbar_expect_tx(bar_x, (uint32_t)nb);
-                bulk_load(x_s + (uint32_t)row * XPITCH, prev + j * KEYS, (uint32_t)nb, bar_x);
-            } else {
-                mbar_arrive(bar_x);
-            }
-        };
-        if (use_x && cq == 0) x_ready(0);
+        // this thread's 128 bytes of its row: sixteen-byte chunk c at x_seg + ((c ^ x_swz) << 4)
+        const uint32_t x_seg = boxes ? (uint32_t)cq * XBOX_BYTES + (uint32_t)lane * 128u : (uint32_t)lane * XPITCH + (uint32_t)cq * 128u;
+        const uint32_t x_swz = boxes ? (uint32_t)(lane & 7) : 0u;
         for (int j = 0; j < n && ok; ++j) {
             const int t = n + j, b = t & 1;
             const int kb = j * KEYS + cq * 32;
@@ -391,57 +451,64 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                 ok = __all_sync(0xffffffffu, ok) != 0;
                 if (!ok) break;
             }
-            // P as the A operand of P V: row `row`, 16-byte chunks of its 128-byte row (64 keys per box), XOR-swizzled
-            const uint32_t p_row = p_s + (uint32_t)(cq >> 1) * BOX_BYTES + (uint32_t)row * 128u;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const uint32_t dst = p_row + (uint32_t)((((cq & 1) * 4 + c) ^ (row & 7)) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pw[4 * c]), "r"(pw[4 * c + 1]), "r"(pw[4 * c + 2]),
-                             "r"(pw[4 * c + 3]) : "memory");
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            // P as the A operand of P V
+            tc_fence_after();
+            __syncwarp();
+            tmem_st16(taddr0 + COL_P + (uint32_t)(cq * 16), pw);
+            tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_pfull);
             // ---- the tensor core has what it needs; now the stored row of this tile
             if (use_x) {
-                if (warp_prev) {
-                    ok = mbar_wait(bar_x, (uint32_t)j & 1u, abort_flag) && ok && !*abort_flag;
-                    ok = __all_sync(0xffffffffu, ok) != 0;
-                    if (ok && warp_valid) {
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            float o0, o1, o2, o3;
-                            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o0), "=f"(o1), "=f"(o2), "=f"(o3) : "r"(x_row + 16u * c) : "memory");
-                            float sn[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i)       // (rounded products, never fused into the subtraction below: an unchanged row gives exactly zero)
-                                sn[i] = __fmul_rn(__fmul_rn(__uint_as_float(r[c >> 2][4 * (c & 3) + i]), scale2), LN2_F);
-                            if (use_old) {
-                                const float od[4] = {o0, o1, o2, o3};
-#pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    if (pr[4 * c + i] > 0.f) A4[i] = fmaf(pr[4 * c + i], sn[i] - od[i], A4[i]);      // (p = 0: also the masked entries)
-                            }
-                            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(x_row + 16u * c), "f"(sn[0]), "f"(sn[1]), "f"(sn[2]), "f"(sn[3]) : "memory");
-                        }
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the bulk store reads what was just written
+                const int xb = j & 1;
+                if (cq == 0 && j > 0) {
+                    // the bulk store of the previous tile has read its staging tile by now: the tile after this one may come
+                    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
+                    if (j + 1 < n) x_ready(j + 1);
                 }
-                // every row of X is complete once all sixteen warps have passed here (an mbarrier, not a named barrier:
+                ok = mbar_wait(bar_x(xb, quarter), (uint32_t)(j >> 1) & 1u, abort_flag) && ok && !*abort_flag;
+                ok = __all_sync(0xffffffffu, ok) != 0;
+                if (!ok) break;
+                const uint32_t x = x_quarter(xb) + x_seg;
+                if (warp_valid) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        float o0, o1, o2, o3;
+                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o0), "=f"(o1), "=f"(o2), "=f"(o3) : "r"(x + (((uint32_t)c ^ x_swz) << 4)) : "memory");
+                        float sn[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)       // (rounded products, never fused into the subtraction below: an unchanged row gives exactly zero)
+                            sn[i] = __fmul_rn(__fmul_rn(__uint_as_float(r[c >> 2][4 * (c & 3) + i]), scale2), LN2_F);
+                        if (use_old) {
+                            const float od[4] = {o0, o1, o2, o3};
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (pr[4 * c + i] > 0.f) A4[i] = fmaf(pr[4 * c + i], sn[i] - od[i], A4[i]);      // (p = 0: also the masked entries)
+                        }
+                        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(x + (((uint32_t)c ^ x_swz) << 4)), "f"(sn[0]), "f"(sn[1]), "f"(sn[2]), "f"(sn[3]) : "memory");
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the bulk store reads what was just written
+                // the quarter's rows are complete once its four warps have passed here (an mbarrier, not a named barrier:
                 // its wait is bounded like every other)
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_w);
+                if (lane == 0) mbar_arrive(bar_w(quarter));
                 if (cq == 0) {
-                    ok = mbar_wait(bar_w, (uint32_t)j & 1u, abort_flag) && ok && !*abort_flag;
+                    ok = mbar_wait(bar_w(quarter), (uint32_t)j & 1u, abort_flag) && ok && !*abort_flag;
                     ok = __all_sync(0xffffffffu, ok) != 0;
                     if (!ok) break;
-                    if (prev) {
-                        const int nb = min(KEYS, a.N - j * KEYS) * 4;
-                        bulk_store(prev + j * KEYS, x_s + (uint32_t)row * XPITCH, (uint32_t)nb);
+                    const int keys = min(KEYS, a.N - j * KEYS);
+                    if (boxes) {
+                        if (lane == 0) {
+                            for (int c = 0; c < (keys + 31) >> 5; ++c)
+                                tma_store_3d(map_x, x_quarter(xb) + (uint32_t)c * XBOX_BYTES, j * KEYS + 32 * c, h, box_row_sh[quarter]);
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
+                    } else if (prev) {
+                        bulk_store(prev + j * KEYS, x_quarter(xb) + (uint32_t)lane * XPITCH, (uint32_t)keys * 4u);
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                     }
-                    if (j + 1 < n) x_ready(j + 1);
                 }
             } else if (warp_valid && prev && valid) {
 #pragma unroll
@@ -464,7 +531,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
         if (ok && warp_valid) {
             uint32_t r[2][16];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) tmem_ld16_issue(taddr0 + 2u * KEYS + (uint32_t)(cq * 32 + 16 * u), r[u]);
+            for (int u = 0; u < 2; ++u) tmem_ld16_issue(taddr0 + COL_O + (uint32_t)(cq * 32 + 16 * u), r[u]);
             tmem_ld_wait();
             if (valid && a.out) {
                 __nv_bfloat16* dst = (__nv_bfloat16*)a.out + (size_t)(row0 + row) * dq + h * DH + cq * 32;

@@ -176,6 +176,19 @@ static bool make_map3(CUtensorMap* out, const void* base, uint64_t batch, uint64
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// fp32 stored attention rows [rows][heads][keys], box = 32 rows x 1 head x 32 keys, 128-byte swizzle
+static bool make_map_rows(CUtensorMap* out, const void* base, uint64_t rows, uint64_t heads, uint64_t keys, int l2promo) {
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {keys, heads, rows};
+    cuuint64_t strides[2] = {keys * 4, keys * heads * 4};
+    cuuint32_t box[3] = {32, 1, 32};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, (CUtensorMapL2promotion)l2promo,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 struct MapCache {
     std::map<std::tuple<const void*, uint64_t, uint64_t, uint32_t>, CUtensorMap> m;
     int l2promo = (int)CU_TENSOR_MAP_L2_PROMOTION_L2_128B;
@@ -186,6 +199,15 @@ struct MapCache {
         if (it != m.end()) return &it->second;
         CUtensorMap tm;
         if (!make_map3(&tm, base, batch, rows, width, l2promo)) return nullptr;
+        return &m.emplace(key, tm).first->second;
+    }
+    // stored attention rows: keyed with box_rows = 0x40000000 | heads
+    const CUtensorMap* get_rows(const void* base, uint64_t rows, uint64_t heads, uint64_t keys) {
+        auto key = std::make_tuple(base, rows, keys, (uint32_t)(0x40000000u | (uint32_t)heads));
+        auto it = m.find(key);
+        if (it != m.end()) return &it->second;
+        CUtensorMap tm;
+        if (!make_map_rows(&tm, base, rows, heads, keys, l2promo)) return nullptr;
         return &m.emplace(key, tm).first->second;
     }
     const CUtensorMap* get(const void* base, uint64_t rows, uint64_t K, uint32_t box_rows) {
@@ -377,14 +399,23 @@ static int launch_attention_stream(MapCache& maps, const AttnArgs& a, cudaStream
     g.rows_per_seq = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
     g.tiles_per_seq = (g.rows_per_seq + ast::ROWS - 1) / ast::ROWS;
     g.status = status;
-    const int dq = a.n_heads * a.head_dim, dkv = a.n_kv * a.head_dim;
+    const int dkv = a.n_kv * a.head_dim;
     const int kv_batch = a.rows ? batch : 1;
-    const CUtensorMap* mq = maps.get(a.q, (uint64_t)a.n_rows, (uint64_t)dq, ast::ROWS);
     const CUtensorMap* mk = maps.get3(a.kc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
     const CUtensorMap* mv = maps.get3(a.vc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
-    if (!mq || !mk || !mv) return POLESTAR_E_CUDA;
+    if (!mk || !mv) return POLESTAR_E_CUDA;
+    // stored rows as tensor boxes where their layout allows (16-byte row pitch); the kernel decides per 32 rows
+    const CUtensorMap *mp = mk, *mr = mk;
+    g.maps = 0;
+    if (a.N % 4 == 0 && !(((uintptr_t)a.pprev | (uintptr_t)a.aprev) & 15)) {
+        const uint64_t p_rows = a.rows ? (uint64_t)batch * (uint64_t)(a.cluster_K > 0 ? a.cluster_K : a.W_max) : (uint64_t)a.n_rows;
+        if (a.pprev && (mp = maps.get_rows(a.pprev, p_rows, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 1;
+        if (a.rows && a.aprev && (mr = maps.get_rows(a.aprev, (uint64_t)batch * a.B, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 2;
+        if (!mp) mp = mk;
+        if (!mr) mr = mk;
+    }
     dim3 grid((unsigned)(g.tiles_per_seq * batch), (unsigned)a.n_heads);
-    CK(launch_k(ast::attention_stream_kernel, grid, dim3(ast::THREADS), ast::smem_bytes(), st, *mq, *mk, *mv, g));
+    CK(launch_k(ast::attention_stream_kernel, grid, dim3(ast::THREADS), ast::smem_bytes(), st, *mk, *mv, *mp, *mr, g));
     return POLESTAR_OK;
 }
 
