@@ -1295,26 +1295,27 @@ __global__ void build_head_list_kernel(StepDesc sd, const int* y, int mask_id, c
         HeadSrc h; h.kind = 0; h.index = (i / sd.B) * sd.rows_per_seq + act_off + (i % sd.B);
         list[i] = h;
     }
-    __syncthreads();
-    if (t == 0) {
-        int n = nb;
-        if (use_suffix) {
-            for (int s = 0; s < sd.batch; ++s) {
-                if (!sd.refresh.v[s]) continue;
-                const int c = sel_cnt[s];
-                for (int i = 0; i < c; ++i) {
-                    const int w = sel_idx[s * sd.W_max + i];
-                    if (w < sd.n_pre) continue;
-                    const int pos = window_pos(sd, w);
-                    if (y[s * sd.N + pos] != mask_id) continue;
+    // the block compacts a sequence's selected rows in order (one thread walking them all: 48 us for a batch of eight)
+    __shared__ int sc[33];
+    int n = nb;
+    if (use_suffix) {
+        for (int s = 0; s < sd.batch; ++s) {
+            if (!sd.refresh.v[s]) continue;
+            const int c = sel_cnt[s];
+            for (int i0 = 0; i0 < c; i0 += blockDim.x) {
+                const int w = i0 + t < c ? sel_idx[s * sd.W_max + i0 + t] : -1;
+                const bool take = w >= sd.n_pre && y[s * sd.N + window_pos(sd, w)] == mask_id;
+                int total;
+                const int o = n + block_excl_scan(take ? 1 : 0, sc, &total);
+                if (take) {
                     HeadSrc h; h.kind = 1; h.index = s * sd.W_max + w;
-                    list[n] = h; suf_seq[n - nb] = s; suf_w[n - nb] = w;
-                    ++n;
+                    list[o] = h; suf_seq[o - nb] = s; suf_w[o - nb] = w;
                 }
+                n += total;
             }
         }
-        *count = n;
     }
+    if (t == 0) *count = n;
     (void)act_row0_stride;
 }
 
@@ -1340,18 +1341,33 @@ __global__ void conf_partial_kernel(const float* logits, const int* m_count, int
     int arg = 0x7fffffff;
     if ((V & 3) == 0) {
         const float4* l4 = reinterpret_cast<const float4*>(l);
-        for (int v4 = (v0 >> 2) + threadIdx.x; v4 < (v1 >> 2); v4 += blockDim.x) {
-            const float4 x = __ldg(l4 + v4);
-            const float xs[4] = {x.x, x.y, x.z, x.w};
-            const float m4 = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
-            const float nm = fmaxf(mx, m4);
-            sum = sum * expf(mx - nm) + expf(x.x - nm) + expf(x.y - nm) + expf(x.z - nm) + expf(x.w - nm);
-            mx = nm;
+        // four loads in flight, one rescaling per sixteen values (entries past the chunk are -inf: exp 0, never the maximum)
+        const int e4 = v1 >> 2;
+        for (int b4 = (v0 >> 2) + threadIdx.x; b4 < e4; b4 += 4 * blockDim.x) {
+            float4 x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int v = 4 * v4 + u;
-                if (v != mask_id && (xs[u] > mxe || (xs[u] == mxe && v < arg))) { mxe = xs[u]; arg = v; }
+            for (int k = 0; k < 4; ++k) {
+                const int v4 = b4 + k * (int)blockDim.x;
+                x[k] = v4 < e4 ? __ldg(l4 + v4) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
             }
+            float nm = mx;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) nm = fmaxf(nm, fmaxf(fmaxf(x[k].x, x[k].y), fmaxf(x[k].z, x[k].w)));
+            const float ref = nm == -INFINITY ? 0.f : nm;        // (only -inf so far: every term is exp(-inf))
+            float part4[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int v4 = b4 + k * (int)blockDim.x;
+                const float xs[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+                part4[k] = v4 < e4 ? (expf(xs[0] - ref) + expf(xs[1] - ref)) + (expf(xs[2] - ref) + expf(xs[3] - ref)) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int v = 4 * v4 + u;
+                    if (v4 < e4 && v != mask_id && (xs[u] > mxe || (xs[u] == mxe && v < arg))) { mxe = xs[u]; arg = v; }
+                }
+            }
+            sum = sum * expf(mx - ref) + ((part4[0] + part4[1]) + (part4[2] + part4[3]));
+            mx = nm;
         }
     } else {
         for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
@@ -1383,23 +1399,33 @@ __global__ void conf_partial_kernel(const float* logits, const int* m_count, int
     }
 }
 
+// One warp per row (one lane per chunk): a thread that walked its row's chunks spent 9 us on dependent loads.
+constexpr int CONF_FINAL_THREADS = 128;
 __global__ void conf_final_kernel(const ConfPart* part, const int* m_count, int rows, int chunks,
                                   int* yhat, float* conf) {
     KERNEL_PROLOGUE(12);   // conf_final_kernel
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, r = blockIdx.x * (CONF_FINAL_THREADS / 32) + (threadIdx.x >> 5);
     if (r >= rows || (m_count && r >= *m_count)) return;
-    const ConfPart* p = part + (size_t)r * chunks;
-    float mx = -INFINITY, mxe = -INFINITY;
+    const ConfPart* p = part + (size_t)r * chunks;      // (caller scratch: four-byte aligned)
+    float mx = -INFINITY, sum = 0.f, mxe = -INFINITY;
     int arg = 0x7fffffff;
-    for (int c = 0; c < chunks; ++c) {
-        mx = fmaxf(mx, p[c].mx_all);
-        if (p[c].mx_ex > mxe || (p[c].mx_ex == mxe && p[c].arg_ex < arg)) { mxe = p[c].mx_ex; arg = p[c].arg_ex; }
+    for (int c = lane; c < chunks; c += 32) {
+        const ConfPart q = p[c];
+        const float nm = fmaxf(mx, q.mx_all);
+        if (sum > 0.f) sum *= expf(mx - nm);
+        if (q.sum > 0.f) sum += q.sum * expf(q.mx_all - nm);
+        mx = nm;
+        if (q.mx_ex > mxe || (q.mx_ex == mxe && q.arg_ex < arg)) { mxe = q.mx_ex; arg = q.arg_ex; }
     }
-    float sum = 0.f;
-    for (int c = 0; c < chunks; ++c)
-        if (p[c].sum > 0.f) sum += p[c].sum * expf(p[c].mx_all - mx);
-    yhat[r] = arg;
-    conf[r] = expf(mxe - mx) / sum;
+    const float all = warp_max(mx);
+    sum = warp_sum(sum > 0.f ? sum * expf(mx - all) : 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, mxe, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, arg, o);
+        if (ov > mxe || (ov == mxe && oi < arg)) { mxe = ov; arg = oi; }
+    }
+    if (lane == 0) { yhat[r] = arg; conf[r] = expf(mxe - all) / sum; }
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1139,7 +1139,7 @@ struct Path {
             Scope sc(c, POLESTAR_PROF_CONFIDENCE, (double)bs * B * m.vocab * 4, 0, 3);
             CK(launch_k(conf_partial_kernel, dim3(CONF_CHUNKS, Mh), dim3(256), 0, st, b.logits, b.head_count, Mh, m.vocab, m.mask_id,
                                                                       CONF_CHUNKS, b.conf_part));
-            CK(launch_k(conf_final_kernel, dim3((Mh + 127) / 128), dim3(128), 0, st, b.conf_part, b.head_count, Mh, CONF_CHUNKS, b.yhat, b.conf));
+            CK(launch_k(conf_final_kernel, dim3((Mh + 3) / 4), dim3(CONF_FINAL_THREADS), 0, st, b.conf_part, b.head_count, Mh, CONF_CHUNKS, b.yhat, b.conf));
             CK(launch_k(delta_kernel, dim3(bs), dim3(256), 0, st, sd, b.kl, act_off, m.n_heads, b.delta));
             CK(cudaGetLastError());
         }
@@ -1788,6 +1788,12 @@ static bool conf_logits_aligned(const float* logits, int vocab) {
     return (((uintptr_t)logits) & ((vocab & 3) == 0 ? 15 : 3)) == 0;
 }
 
+static int launch_confidence(const float* logits, int rows, int vocab, int mask_id, int* yhat, float* conf, ConfPart* part, cudaStream_t st) {
+    CK(launch_k(conf_partial_kernel, dim3(CONF_CHUNKS, rows), dim3(256), 0, st, logits, (const int*)nullptr, rows, vocab, mask_id, CONF_CHUNKS, part));
+    CK(launch_k(conf_final_kernel, dim3((rows + 3) / 4), dim3(CONF_FINAL_THREADS), 0, st, (const ConfPart*)part, (const int*)nullptr, rows, CONF_CHUNKS, yhat, conf));
+    return POLESTAR_OK;
+}
+
 extern "C" int polestar_k_confidence(const float* logits, int32_t rows, int32_t vocab, int32_t mask_id, int32_t* yhat,
                                      float* conf, void* scratch, size_t scratch_bytes, void* stream) {
     if (rows < 0 || vocab <= 0) return POLESTAR_E_INVAL;
@@ -1796,10 +1802,7 @@ extern "C" int polestar_k_confidence(const float* logits, int32_t rows, int32_t 
     if (!conf_logits_aligned(logits, vocab)) return POLESTAR_E_INVAL;
     if (scratch_bytes < (size_t)rows * CONF_CHUNKS * sizeof(ConfPart)) return POLESTAR_E_NOSPACE;
     cudaStream_t st = (cudaStream_t)stream;
-    conf_partial_kernel<<<dim3(CONF_CHUNKS, rows), 256, 0, st>>>(logits, nullptr, rows, vocab, mask_id, CONF_CHUNKS, (ConfPart*)scratch);
-    conf_final_kernel<<<(rows + 127) / 128, 128, 0, st>>>((const ConfPart*)scratch, nullptr, rows, CONF_CHUNKS, yhat, conf);
-    CK(cudaGetLastError());
-    return POLESTAR_OK;
+    return launch_confidence(logits, rows, vocab, mask_id, yhat, conf, (ConfPart*)scratch, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1843,8 +1846,5 @@ extern "C" int polestar_k_confidence_noalloc(const float* logits, int32_t rows, 
     cudaStream_t st = (cudaStream_t)stream;
     // every partial the second kernel reads is written by the first one in this call, so nothing of the
     // previous call's contents has to be cleared
-    conf_partial_kernel<<<dim3(CONF_CHUNKS, rows), 256, 0, st>>>(logits, nullptr, rows, vocab, mask_id, CONF_CHUNKS, scratch);
-    conf_final_kernel<<<(rows + 127) / 128, 128, 0, st>>>(scratch, nullptr, rows, CONF_CHUNKS, yhat, conf);
-    CK(cudaGetLastError());
-    return POLESTAR_OK;
+    return launch_confidence(logits, rows, vocab, mask_id, yhat, conf, scratch, st);
 }

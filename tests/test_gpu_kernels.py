@@ -269,6 +269,27 @@ def test_confidence_matches_oracle(rows, V):
     assert np.allclose(conf.cpu().numpy(), rc, rtol=1e-4, atol=1e-7)
 
 
+@pytest.mark.parametrize("rows,V", [(5, 516), (3, 2052), (9, 131072), (2, 16384), (130, 1030)])
+def test_confidence_edges(rows, V):
+    # chunks shorter than a batch of loads, empty chunks, row counts that do not fill a block; rows that are -inf but for a
+    # few entries; scratch at a four-byte boundary
+    logits = rnd((rows, V), 12, 3.0)
+    mask_id = 3
+    logits[0] = float("-inf")
+    logits[0, V - 1], logits[0, V // 2] = 1.0, 0.5
+    logits[1, : V // 2 + 5] = float("-inf")
+    yhat = torch.zeros(rows, dtype=torch.int32, device="cuda")
+    conf = torch.zeros(rows, device="cuda")
+    scratch = torch.empty(rows * 512 + 4, dtype=torch.uint8, device="cuda")[4:]
+    Bd.polestar_k_confidence(logits.cuda(), mask_id, yhat, conf, scratch)
+    x = logits.double()
+    x[:, mask_id] = float("-inf")
+    best, arg = x.max(dim=1)
+    want = torch.exp(best - torch.logsumexp(logits.double(), dim=1))
+    assert torch.equal(yhat.cpu().long(), arg)
+    assert torch.allclose(conf.cpu().double(), want, rtol=2e-5, atol=0)          # fp32 sums of V terms, exponentials to 2 ulp
+
+
 # ------------------------------------------------------------------ empty inputs
 def test_empty_inputs_are_noops():
     dev = "cuda"
