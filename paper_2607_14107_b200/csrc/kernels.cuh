@@ -186,8 +186,21 @@ __device__ __forceinline__ void prep_qkv_row(const StepDesc& sd, int r, const Ro
                 const int c4 = threadIdx.x + u * blockDim.x;
                 const bool in = c4 < n4;
                 if (u * (int)blockDim.x >= n4) continue;         // (the whole block is past the row)
-                // members in ascending window order for every column (deterministic), four at a time: all loads of a
-                // group are issued before the first of them is used
+                // members in ascending window order for every column (deterministic): all loads of a group are issued before
+                // the first of them is used, sixteen of a plain cache's (a refresh step with eight proxies at the 8B widths: 5833 -> 5669
+                // us), four of a quantised one's
+                if (!ct.hq) {
+                    for (int t = 0; t < nb; t += 16) {
+                        float4 v[16];
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            v[k] = (t + k < nb && in) ? __ldcg(reinterpret_cast<const float4*>(s_src[t + k]) + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            if (t + k < nb) { acc[u].x += v[k].x; acc[u].y += v[k].y; acc[u].z += v[k].z; acc[u].w += v[k].w; }
+                    }
+                    continue;
+                }
                 for (int t = 0; t < nb; t += 4) {
                     float4 v[4];
                     unsigned cd[4], sb[4];
