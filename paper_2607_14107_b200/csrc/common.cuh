@@ -201,7 +201,7 @@ enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_DOWN = 3, EPI_LOGITS = 4,
 // Everything an epilogue may need; unused members are null.
 struct EpiArgs {
     const Row* rows;          // descriptors of the GEMM's rows (QKV) / of the forward (DOWN)
-    const int* list;          // DOWN: compacted row -> forward row
+    const int* list;          // DOWN, RESID: compacted row -> forward row (null: the same)
     const int* m_count;       // device-side row count (null: use the host bound)
     const unsigned char* kvflag;  // QKV: write k,v of this row into the cache
     const float2* rope;       // [N][head_dim/2] (cos, sin)
@@ -376,7 +376,7 @@ __device__ __forceinline__ void epilogue_pair(const EpiArgs& e, int m, int n, fl
             store_pair<T>((T*)e.vc + ((size_t)seq * Npos + pos) * dkv + (n - dq - dkv), v0, v1);
         }
     } else if (EPI == EPI_RESID) {
-        const size_t o = (size_t)m * e.ld_out + n;
+        const size_t o = (size_t)(e.list ? __ldg(e.list + m) : m) * e.ld_out + n;
         const float2 r = __ldg(reinterpret_cast<const float2*>(e.resid + o));
         *reinterpret_cast<float2*>(e.out_f32 + o) = make_float2(r.x + v0, r.y + v1);
     } else if (EPI == EPI_SWIGLU) {
@@ -499,7 +499,7 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int n, const
             store16<T>((T*)e.vc + ((size_t)seq * Npos + pos) * dkv + (n - dq - dkv), v);
         }
     } else if (EPI == EPI_RESID) {
-        const size_t o = (size_t)m * e.ld_out + n;
+        const size_t o = (size_t)(e.list ? __ldg(e.list + m) : m) * e.ld_out + n;
         float r[16];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -543,7 +543,7 @@ __device__ __forceinline__ void epilogue16(const EpiArgs& e, int m, int n, const
 template <typename T, int EPI>
 __device__ __forceinline__ void epilogue4(const EpiArgs& e, int m, int n, float4 v) {
     if (EPI == EPI_RESID) {
-        const size_t o = (size_t)m * e.ld_out + n;
+        const size_t o = (size_t)(e.list ? __ldg(e.list + m) : m) * e.ld_out + n;
         const float4 c = __ldg(reinterpret_cast<const float4*>(e.resid + o));
         const float4 r = make_float4(c.x + v.x, c.y + v.y, c.z + v.z, c.w + v.w);
         *reinterpret_cast<float4*>(e.out_f32 + o) = r;
@@ -573,7 +573,7 @@ __device__ __forceinline__ void epilogue_prefetch(const EpiArgs& e, int m, int n
         if (rw.y >= 0 && n < (e.n_heads + e.n_kv) * e.head_dim)
             prefetch_l1(e.rope + (size_t)rw.y * (e.head_dim / 2) + ((n % e.head_dim) >> 1));
     } else if (EPI == EPI_RESID) {
-        prefetch_l1(e.resid + (size_t)m * e.ld_out + n);
+        prefetch_l1(e.resid + (size_t)(e.list ? __ldg(e.list + m) : m) * e.ld_out + n);
         if (e.fold_a) prefetch_l1(e.fold_gain + n);
     } else if (EPI == EPI_DOWN) {
         const int r = e.list ? __ldg(e.list + m) : m;

@@ -609,7 +609,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             } else if ((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate) {
                 // partial segment of a projection whose output rows are the residual rows: add it onto them in L2
                 bool row_ok = live;
-                float* dst = e.out_f32 + (size_t)m * e.ld_out + n0;
+                float* dst = e.out_f32 + (size_t)((EPI == EPI_RESID && live && e.list) ? __ldcg(e.list + m) : m) * e.ld_out + n0;
                 if (EPI == EPI_DOWN && live) {
                     const int r0 = e.list ? __ldcg(e.list + m) : m;
                     const int4 rw = __ldg(reinterpret_cast<const int4*>(e.rows) + r0);       // {seq, pos, widx, aidx}

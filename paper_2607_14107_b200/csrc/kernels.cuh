@@ -388,6 +388,24 @@ __global__ void prep_rows_kernel(const float* x, const int* list, const int* m_c
     prep_rows_row<T>(blockIdx.x, x, list, m_count, gain, eps, d, a_out, red, rows, packet, W_max);
 }
 
+// Rows of a compacted list, gathered: dst row i <- src row list[i] (`bytes` a multiple of 16, rows 16-byte aligned).  Bound by
+// the copy; four 16-byte loads in flight per thread.
+__global__ void __launch_bounds__(128) gather_rows_kernel(const char* src, const int* list, const int* m_count, int bytes, char* dst) {
+    KERNEL_PROLOGUE(6);   // gather_rows_kernel
+    const int i = blockIdx.x;
+    if (i >= __ldcg(m_count)) return;
+    const uint4* s = reinterpret_cast<const uint4*>(src + (size_t)__ldcg(list + i) * bytes);
+    uint4* d = reinterpret_cast<uint4*>(dst + (size_t)i * bytes);
+    const int n = bytes >> 4;
+    for (int c = threadIdx.x; c < n; c += 4 * 128) {
+        uint4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) if (c + 128 * k < n) v[k] = __ldcg(s + c + 128 * k);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) if (c + 128 * k < n) d[c + 128 * k] = v[k];
+    }
+}
+
 // LM-head input rows: entry i < n_act reads x[act_rows...]; later entries read packet rows.
 struct HeadSrc { int kind; int index; };  // kind 0: x row `index`; 1: packet row `index` (= seq*W_max+w)
 template <typename T>
