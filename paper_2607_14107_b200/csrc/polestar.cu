@@ -1685,8 +1685,7 @@ extern "C" int polestar_k_select(const float* drift, int32_t batch, int32_t W, i
         return POLESTAR_OK;
     }
     if (!drift || !idx) return POLESTAR_E_INVAL;
-    select_kernel<<<batch, SEL_THREADS, 0, (cudaStream_t)stream>>>(drift, W, mode, k, thresh, floor_, idx, count);
-    CK(cudaGetLastError());
+    CK(launch_k(select_kernel, dim3(batch), dim3(SEL_THREADS), 0, (cudaStream_t)stream, drift, W, mode, k, thresh, floor_, idx, count));
     return POLESTAR_OK;
 }
 
