@@ -381,8 +381,8 @@ static bool attention_stream_applies(const AttnArgs& a) {
     return a.head_dim == ast::DH && a.N > 0 && (a.n_heads * a.head_dim) % 64 == 0 && (a.n_kv * a.head_dim) % 64 == 0;
 }
 // Which of the two tensor-core kernels: the streaming one as soon as its grid (row tiles x heads x sequences) fills a
-// good part of the GPU -- block entries, batches, long sequences (measured: 512 x 512 keys 43 us against 80 us,
-// 2048 x 2048 keys 0.6 ms against 1.4 ms) -- or the keys exceed what a cluster of key ranges covers; the cluster
+// good part of the GPU -- block entries, batches, long sequences (measured: 512 x 512 keys 28 us against 80 us,
+// 2048 x 2048 keys 0.29 ms against 1.4 ms) -- or the keys exceed what a cluster of key ranges covers; the cluster
 // kernel for the small steps of one short sequence, where spreading the keys over SMs wins (128 x 512: 20 us against 37 us).
 static bool attention_prefers_stream(const AttnArgs& a) {
     const int batch = a.batch > 0 ? a.batch : 1;
