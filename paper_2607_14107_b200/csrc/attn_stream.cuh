@@ -76,6 +76,12 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
                  ::"l"(map), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
+// "Tile j of a quarter is written": one barrier per staging tile, so each serves every second key tile.  With one barrier
+// for both, a warp that is a tile ahead (the old rows of tile j + 1 were requested before tile j was worked on) would arrive
+// in place of a slower one, and tile j would be stored without the slower warp's columns.
+__host__ __device__ constexpr int written_bar(int j) { return j & 1; }
+__host__ __device__ constexpr uint32_t written_parity(int j) { return (j >> 1) & 1; }
+
 struct Args {
     AttnArgs a;
     int maps;               // bit 0: map_p describes a.pprev, bit 1: map_r describes a.aprev (else null rows or unaligned: plain path)
@@ -88,7 +94,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                         const __grid_constant__ CUtensorMap map_p, const __grid_constant__ CUtensorMap map_r, Args g) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars[4 + 2 * NS + 4 + 8 + 4];
+    __shared__ uint64_t bars[4 + 2 * NS + 4 + 8 + 8];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     __shared__ float* prev_sh[ROWS];
@@ -119,14 +125,14 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
     auto bar_sfree = [&](int s) { return smem_u32(&bars[6 + 2 * NS + s]); };
     // staging tiles, per lane quarter (32 rows, the four warps that share them): "X_b may be worked on", "the warps are done with it"
     auto bar_x = [&](int b, int q) { return smem_u32(&bars[8 + 2 * NS + 4 * b + q]); };
-    auto bar_w = [&](int q) { return smem_u32(&bars[16 + 2 * NS + q]); };
+    auto bar_w = [&](int j, int q) { return smem_u32(&bars[16 + 2 * NS + 4 * written_bar(j) + q]); };
     auto x_s = [&](int b) { return smem_base + (uint32_t)NS * TILE_BYTES + (uint32_t)b * X_BYTES; };
 
     if (threadIdx.x == 0) {
         mbar_init(bar_q, 16); mbar_init(bar_o, 1); mbar_init(bar_pfull, 16); mbar_init(bar_pfree, 1);
         for (int s = 0; s < NS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_free(s), 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(bar_sfull(s), 1); mbar_init(bar_sfree(s), 16); }
-        for (int q = 0; q < 4; ++q) { mbar_init(bar_x(0, q), 32); mbar_init(bar_x(1, q), 32); mbar_init(bar_w(q), 4); }
+        for (int q = 0; q < 4; ++q) { mbar_init(bar_x(0, q), 32); mbar_init(bar_x(1, q), 32); mbar_init(bar_w(0, q), 4); mbar_init(bar_w(1, q), 4); }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -493,9 +499,9 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 // the quarter's rows are complete once its four warps have passed here (an mbarrier, not a named barrier:
                 // its wait is bounded like every other)
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_w(quarter));
+                if (lane == 0) mbar_arrive(bar_w(j, quarter));
                 if (cq == 0) {
-                    ok = mbar_wait(bar_w(quarter), (uint32_t)j & 1u, abort_flag) && ok && !*abort_flag;
+                    ok = mbar_wait(bar_w(j, quarter), written_parity(j), abort_flag) && ok && !*abort_flag;
                     ok = __all_sync(0xffffffffu, ok) != 0;
                     if (!ok) break;
                     const int keys = min(KEYS, a.N - j * KEYS);

@@ -290,6 +290,16 @@ def test_c1b_streaming_attention_kernel(monkeypatch, kw):
     assert seen["refresh"] > 3 and seen["entry_window"] >= 0
 
 
+@pytest.mark.parametrize("prompt_len", [600, 601])          # 601: rows of 673 floats, which no bulk copy takes
+def test_c1b_streaming_attention_stored_row_forms(monkeypatch, prompt_len):
+    # refresh steps of 24 + 72 rows over six key tiles: the first 32 rows hold the active block's and the window's stored
+    # rows (row copies in the last layer, a partly recorded quarter in the others), the other quarters tensor boxes
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", "9")
+    seen = run_forced("c1b", 8, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=2, prompt_len=prompt_len, gen_len=72, block=24,
+                      max_steps=24)
+    assert seen["refresh"] > 3
+
+
 def test_c1b_tall_gemm_tiles(monkeypatch):
     # 256-token CTA tiles (two MMAs per k step on one weight tile) for every projection of more than 129 rows: block
     # entries of a batch (ragged: 3 x 146 and 3 x 90 rows), refresh steps (3 x 72 rows), whole and split tiles
