@@ -235,8 +235,8 @@ struct SkArgs {
     int M, N_out, K, stages;
     int tiles_f, tiles_t;
     float* partial;     // [2 * gridDim.x][BLOCK_T][BLOCK_F] fp32
-    int* tile_counter;  // arrivals [tile] and, done_offset further on, finished shares [tile]; zero before
-                        // launch, zero again after
+    int* tile_counter;  // arrivals [split tile] and, done_offset further on, finished shares [split tile]; zero before launch,
+                        // zero again after.  Split tiles count from sk_whole_tiles(...) * G on (times two CTAs of a pair)
     int done_offset;
     int* status;        // set to 1 on a wait time-out
     int w_stream;       // 1: every weight byte is read once by this launch: load it with the evict_first L2 policy
@@ -276,6 +276,13 @@ __device__ __forceinline__ void tile_ft(int tile, int tiles_f, int tiles_t, int&
     const int tc = min(RASTER_T, tiles_t - chunk * RASTER_T);
     f = local / tc;
     t = chunk * RASTER_T + (local - f * tc);
+}
+
+// Tiles that every one of G scheduling units takes whole.  The split (stream-K) part is the remainder r = tiles mod G when
+// that leaves at most ~8 units per tile, else G + r tiles: fewer than 2 G in any case, so the counters of split tiles do not
+// bound the size of a projection.
+__host__ __device__ constexpr int sk_whole_tiles(int tiles, int G) {
+    return tiles < G ? 0 : ((tiles % G == 0 || tiles % G * 8 >= G) ? tiles / G : tiles / G - 1);
 }
 
 // Number of partial tile segments in CTA c's unit range (0, 1 or 2): what it has to publish and then help reduce.
@@ -326,7 +333,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     __shared__ uint32_t tmem_base_sh;
     __shared__ int abort_sh;
     __shared__ int last_sh;
-    __shared__ int fx_par[2][8];          // per partial tile of this CTA: tile, c_lo, nseg, before, mine, w_all, tile_f, tile_t
+    __shared__ int fx_par[2][8];          // per partial tile of this CTA: split tile, c_lo, nseg, before, mine, w_all, tile_f, tile_t
     __shared__ int fx_n;
     __shared__ volatile int fx_ready;
 
@@ -347,9 +354,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // [u_begin, u_end) per CTA, whose partial tiles are reduced in the fix-up pass.  U, u_begin, u_end and the
     // arithmetic derived from them count units of this stream-K part; its tiles have ids tile_base + u / kb_total.
     const int tiles_all = g.tiles_f * g.tiles_t;
-    // (the stream-K part is the remainder r = tiles mod G when that leaves at most ~8 CTAs per tile, else G + r tiles)
-    const int rem = tiles_all % G;
-    const int dp = (tiles_all < G) ? 0 : ((rem == 0 || rem * 8 >= G) ? tiles_all / G : tiles_all / G - 1);
+    const int dp = sk_whole_tiles(tiles_all, G);
     const int tile_base = dp * G;
     const long long U = (long long)(tiles_all - tile_base) * kb_total;
     const long long u_begin = sk_begin(U, G, cta), u_end = sk_begin(U, G, cta + 1);
@@ -409,7 +414,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 const int nseg = c_hi - c_lo + 1;
                 const int w_lo = sk_partial_segments(U, G, c_lo, kb_total) == 2 ? 1 : 2;
                 const int w_hi = (nseg > 1 && sk_partial_segments(U, G, c_hi, kb_total) == 2) ? 1 : 2;
-                fx_par[f][0] = tile_base + tile; fx_par[f][1] = c_lo; fx_par[f][2] = nseg;
+                fx_par[f][0] = tile; fx_par[f][1] = c_lo; fx_par[f][2] = nseg;
                 fx_par[f][3] = (cta == c_lo) ? 0 : w_lo + 2 * (cta - c_lo - 1);
                 fx_par[f][4] = (cta == c_lo) ? w_lo : (cta == c_hi ? w_hi : 2);
                 fx_par[f][5] = (nseg == 1) ? w_lo : w_lo + w_hi + 2 * (nseg - 2);
@@ -664,7 +669,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (!whole && !((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate)) {
                 __threadfence();
                 asm volatile("bar.sync 1, %0;" ::"r"(128 * groups) : "memory");
-                if (threadIdx.x == 64) atomicAdd(&g.tile_counter[tile * CG + rank], 1);
+                if (threadIdx.x == 64) atomicAdd(&g.tile_counter[(tile - tile_base) * CG + rank], 1);
             }
             ++seg;
         }

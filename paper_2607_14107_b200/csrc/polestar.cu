@@ -299,12 +299,12 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
         // the pair is the scheduling unit: G counts pairs here, the launch has twice as many CTAs
         sk_grid(ws, M, N_out, K, &U, &G, BT, ws.pairs);
         while (G > 1 && ((size_t)4 * G * tc::BLOCK_T * tc::BLOCK_F * 4 + 16384 + 65536 > ws.partial_bytes)) --G;
-        if (2 * tiles_f * tiles_t + 2 > ws.n_counters / 2) return POLESTAR_E_INVAL;
     } else {
         sk_grid(ws, M, N_out, K, &U, &G, BT, ws.sms);
         while (G > 1 && ((size_t)2 * G * BT * tc::BLOCK_F * 4 + 16384 + 65536 > ws.partial_bytes)) --G;
-        if (tiles_f * tiles_t > ws.n_counters / 2) return POLESTAR_E_INVAL;
     }
+    // (always holds: fewer than 2 G tiles are split)
+    if ((tiles_f * tiles_t - tc::sk_whole_tiles(tiles_f * tiles_t, (int)G) * (int)G) * (pair ? 2 : 1) > ws.n_counters / 2) return POLESTAR_E_INVAL;
     tc::SkArgs g;
     g.M = M; g.N_out = N_out; g.K = K; g.tiles_f = tiles_f; g.tiles_t = tiles_t;
     // Three stages (145 KB) for the weight-bound steps: measured +2 % tokens/s over four (the HBM stream needs no more in
@@ -504,7 +504,7 @@ static int launch_gemm_chain(MapCache& maps, const GemmWs& ws, const ChainSpec* 
     return POLESTAR_OK;
 }
 
-static const int GEMM_COUNTERS = 1 << 17;     // arrivals + finished shares for up to 65536 output tiles
+static const int GEMM_COUNTERS = 1 << 17;     // arrivals + finished shares of split tiles (a launch has fewer than two per SM) + the grid-wide counters
 
 struct polestar_ctx {
     polestar_model m;
@@ -1736,11 +1736,12 @@ extern "C" int polestar_k_refresh(const void* h, const int32_t* idx, const int32
     ws.partial = (float*)(sc + off_part); ws.partial_bytes = GEMM_PARTIAL_BYTES;
     const int M = batch * max_rows;
     const int dq = n_heads * head_dim, dkv = n_kv * head_dim;
-    // The scratch is caller memory with unknown contents: the split-K tile counters must start at zero.  Only the
-    // counters of this GEMM's output tiles (arrivals, then finished shares) are used, so only those are cleared.
-    const long long tiles = (long long)((dq + 2 * dkv + tc::BLOCK_F - 1) / tc::BLOCK_F) * ((M + tc::BLOCK_T - 1) / tc::BLOCK_T);
-    // (CTA pairs count per 128-row half of their 256-row tiles: up to one more half per feature tile)
-    const int n_cnt = (int)std::min<long long>(GEMM_COUNTERS, 2 * (tiles + (dq + 2 * dkv) / tc::BLOCK_F + 2));
+    // The scratch is caller memory with unknown contents: the split tiles' counters (arrivals, then finished shares) must start
+    // at zero.  Only as many as this GEMM can use are cleared: fewer than two per SM (sk_whole_tiles; a pair tile has one for
+    // each of its 128-row halves), and no more than it has 128-row tiles, the empty second half of a pair tile included.
+    const long long tiles_f = (dq + 2 * dkv + tc::BLOCK_F - 1) / tc::BLOCK_F;
+    const long long tiles = tiles_f * ((M + tc::BLOCK_T - 1) / tc::BLOCK_T + 1);
+    const int n_cnt = (int)(2 * std::min<long long>(tiles, 2LL * di.sm_count));
     ws.counters = (int*)(sc + off_cnt); ws.n_counters = n_cnt; ws.status = (int*)(sc + off_status);
     const int half = head_dim / 2;
     // Two launches with programmatic stream serialization (the projection starts while the gather drains).  The gather

@@ -345,6 +345,24 @@ def test_c1b_gemm_cta_pairs(monkeypatch):
     assert seen["refresh"] > 3 and seen["entry_window"] > 0
 
 
+def test_block_entry_of_a_large_batch_with_a_wide_feed_forward_network():
+    # 64 sequences x 1024 positions x 2 * 18944 features: 37 888 pair tiles in the gate/up projection of the block entry
+    m, p = I.config("c1b")
+    m = dataclasses.replace(m, n_layers=1, d_ffn=18944)
+    p = dataclasses.replace(p, batch=64, prompt_len=960, gen_len=64, block=32, max_steps=32)
+    packed, prompt = Bd.pack_weights(m, I.make_weights(m)), I.make_prompt(m, p).numpy()
+    whole = Bd.Polestar(m, packed, p, prompt)
+    logits = whole.read(Bd.READ_LOGITS)
+    for s in (0, 31, 63):
+        one = Bd.Polestar(m, packed, dataclasses.replace(p, batch=1), prompt[s:s + 1])
+        close(logits[s], one.read(Bd.READ_LOGITS)[0], TOL[m.dtype], f"sequence {s}")
+        one.destroy()
+    whole.commit()
+    whole.step()
+    whole.commit()
+    whole.destroy()
+
+
 def test_c1b_bf16_simt_gemm_path():
     run_forced("c1b", 6, tau_upd=-1, flags=I.FLAG_DEFAULT | Bd.FLAG_SIMT_GEMM)
 

@@ -209,6 +209,33 @@ def test_refresh_chain_on_cta_pairs(monkeypatch, P, d, nh, nkv, k, batch):
     check_refresh_chain(P, d, nh, nkv, k, batch)
 
 
+def test_refresh_of_more_tiles_than_any_counter_array():
+    # 589 824 rows x 4096 columns: 36 864 pair tiles.  Only the split tiles of a projection are counted, so its size has no
+    # limit; one sequence of the batch on its own (4096 tiles) gives the same rows (fp32 sums in another order: one bf16 step)
+    P, batch, d, nh, nkv, dh = 65536, 9, 512, 28, 2, 128
+    g = torch.Generator(device="cuda").manual_seed(3)
+    h = torch.empty((batch, P, d), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    w = torch.empty(((nh + 2 * nkv) * dh, d), dtype=torch.bfloat16, device="cuda").normal_(0, 0.05, generator=g)
+    norm = torch.ones(d, device="cuda")
+
+    def refresh(hs):
+        n = hs.shape[0]
+        kc, vc, q = (torch.zeros((n, P, x * dh), dtype=torch.bfloat16, device="cuda") for x in (nkv, nkv, nh))
+        idx = torch.arange(P, dtype=torch.int32, device="cuda").repeat(n, 1)
+        cnt = torch.full((n,), P, dtype=torch.int32, device="cuda")
+        scratch = torch.empty(Bd.polestar_k_refresh_scratch_bytes(n, P, d, nh, nkv, dh) + 1024, dtype=torch.uint8, device="cuda")
+        scratch = scratch[(-scratch.data_ptr()) % 1024:]
+        Bd.polestar_k_refresh(hs, idx, cnt, w, norm, kc, vc, q, P, nh, nkv, dh, 1e-5, 1e4, scratch)
+        assert Bd.polestar_k_refresh_status(scratch, n, P, d, dh) == Bd.OK
+        return kc, vc, q
+
+    whole = refresh(h)
+    for s in (0, 4, 8):
+        for a, b in zip(whole, refresh(h[s:s + 1].contiguous())):
+            assert torch.allclose(a[s].float(), b[0].float(), atol=1e-5, rtol=2 ** -7)
+            assert b.abs().max() > 1
+
+
 def check_refresh_chain(P, d, nh, nkv, k, batch):
     dh = 128
     big = d >= 2048
