@@ -279,10 +279,12 @@ __device__ __forceinline__ void tile_ft(int tile, int tiles_f, int tiles_t, int&
 }
 
 // Tiles that every one of G scheduling units takes whole.  The split (stream-K) part is the remainder r = tiles mod G when
-// that leaves at most ~8 units per tile, else G + r tiles: fewer than 2 G in any case, so the counters of split tiles do not
-// bound the size of a projection.
-__host__ __device__ constexpr int sk_whole_tiles(int tiles, int G) {
-    return tiles < G ? 0 : ((tiles % G == 0 || tiles % G * 8 >= G) ? tiles / G : tiles / G - 1);
+// that leaves at most ~8 units per tile and every unit at least one k block (the arrival counts of split tiles take all
+// units between a tile's first and last contributor for contributors), else G + r tiles: fewer than 2 G in any case, so the
+// counters of split tiles do not bound the size of a projection.
+__host__ __device__ constexpr int sk_whole_tiles(int tiles, int G, int kb_total) {
+    const int r = tiles % G;
+    return tiles < G ? 0 : ((r == 0 || (r * 8 >= G && (long long)r * kb_total >= G)) ? tiles / G : tiles / G - 1);
 }
 
 // Number of partial tile segments in CTA c's unit range (0, 1 or 2): what it has to publish and then help reduce.
@@ -354,7 +356,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // [u_begin, u_end) per CTA, whose partial tiles are reduced in the fix-up pass.  U, u_begin, u_end and the
     // arithmetic derived from them count units of this stream-K part; its tiles have ids tile_base + u / kb_total.
     const int tiles_all = g.tiles_f * g.tiles_t;
-    const int dp = sk_whole_tiles(tiles_all, G);
+    const int dp = sk_whole_tiles(tiles_all, G, kb_total);
     const int tile_base = dp * G;
     const long long U = (long long)(tiles_all - tile_base) * kb_total;
     const long long u_begin = sk_begin(U, G, cta), u_end = sk_begin(U, G, cta + 1);

@@ -304,7 +304,7 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
         while (G > 1 && ((size_t)2 * G * BT * tc::BLOCK_F * 4 + 16384 + 65536 > ws.partial_bytes)) --G;
     }
     // (always holds: fewer than 2 G tiles are split)
-    if ((tiles_f * tiles_t - tc::sk_whole_tiles(tiles_f * tiles_t, (int)G) * (int)G) * (pair ? 2 : 1) > ws.n_counters / 2) return POLESTAR_E_INVAL;
+    if ((tiles_f * tiles_t - tc::sk_whole_tiles(tiles_f * tiles_t, (int)G, K / 64) * (int)G) * (pair ? 2 : 1) > ws.n_counters / 2) return POLESTAR_E_INVAL;
     tc::SkArgs g;
     g.M = M; g.N_out = N_out; g.K = K; g.tiles_f = tiles_f; g.tiles_t = tiles_t;
     // Three stages (145 KB) for the weight-bound steps: measured +2 % tokens/s over four (the HBM stream needs no more in

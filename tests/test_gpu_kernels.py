@@ -209,6 +209,15 @@ def test_refresh_chain_on_cta_pairs(monkeypatch, P, d, nh, nkv, k, batch):
     check_refresh_chain(P, d, nh, nkv, k, batch)
 
 
+@pytest.mark.parametrize("pair_rows,k", [(0, 2752), (1 << 30, 2688)])
+def test_refresh_chain_few_k_blocks_in_the_split_tiles(monkeypatch, pair_rows, k):
+    # more tiles than scheduling units, with a remainder of few tiles of two k blocks each (86 tiles on 74 CTA pairs, 168 on
+    # 148 CTAs): the split part must still give every unit a k block
+    monkeypatch.setenv("POLESTAR_GEMM_PAIR_ROWS", str(pair_rows))
+    Bd.polestar_reload_env()
+    check_refresh_chain(k, 128, 2, 1, k, 4)
+
+
 def test_refresh_of_more_tiles_than_any_counter_array():
     # 589 824 rows x 4096 columns: 36 864 pair tiles.  Only the split tiles of a projection are counted, so its size has no
     # limit; one sequence of the batch on its own (4096 tiles) gives the same rows (fp32 sums in another order: one bf16 step)
