@@ -1404,7 +1404,8 @@ __global__ void conf_partial_kernel(const float* logits, const int* m_count, int
         for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
             const float x = l[v];
             const float nm = fmaxf(mx, x);
-            sum = sum * expf(mx - nm) + expf(x - nm);
+            const float ref = nm == -INFINITY ? 0.f : nm;        // (as above)
+            sum = sum * expf(mx - ref) + expf(x - ref);
             mx = nm;
             if (v != mask_id && (x > mxe || (x == mxe && v < arg))) { mxe = x; arg = v; }
         }

@@ -305,10 +305,10 @@ def test_confidence_matches_oracle(rows, V):
     assert np.allclose(conf.cpu().numpy(), rc, rtol=1e-4, atol=1e-7)
 
 
-@pytest.mark.parametrize("rows,V", [(5, 516), (3, 2052), (9, 131072), (2, 16384), (130, 1030)])
+@pytest.mark.parametrize("rows,V", [(5, 516), (3, 2052), (9, 131072), (2, 16384), (130, 1030), (3, 50258)])
 def test_confidence_edges(rows, V):
     # chunks shorter than a batch of loads, empty chunks, row counts that do not fill a block; rows that are -inf but for a
-    # few entries; scratch at a four-byte boundary
+    # few entries (50258: several entries per thread of a row that is not read in 16-byte loads); scratch at a four-byte boundary
     logits = rnd((rows, V), 12, 3.0)
     mask_id = 3
     logits[0] = float("-inf")
