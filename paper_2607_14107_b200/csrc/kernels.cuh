@@ -431,7 +431,12 @@ template <typename T>
 __global__ void prep_refresh_kernel(const T* h, const int* idx, const int* counts, int max_rows, int P,
                                     const float* gain, float eps, int d, T* a_out, float2* rope_tab, int half, double theta,
                                     int* counters, int n_counters, int* status) {
-    KERNEL_PROLOGUE(6);   // prep_refresh_kernel
+    // The projection behind this launch requests weights before its own dependency wait, so it may start only when whatever
+    // ran before this launch (the caller's kernel that wrote those weights, for one) is complete: wait, then trigger.  What
+    // that costs: the weight stream no longer starts under the selection in front of the refresh.
+    pdl_wait();
+    pdl_trigger();
+    trace_stamp(6);   // prep_refresh_kernel
     __shared__ float red[33];
     const int m = blockIdx.x;
     const int s = m / max_rows, i = m - s * max_rows;

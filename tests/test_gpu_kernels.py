@@ -288,6 +288,49 @@ def check_refresh_chain(P, d, nh, nkv, k, batch):
         assert torch.equal(kc_h[s][rest], kc0_h[s][rest]) and torch.equal(vc_h[s][rest], vc0_h[s][rest])
 
 
+LATE_WRITER = r"""
+extern "C" __global__ void late_writer(unsigned short* dst, const unsigned short* src, int n) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // dependents may start now ...
+    const long long t0 = clock64();
+    while (clock64() - t0 < 400000) { }                                  // ... about 0.2 ms before anything is written
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+"""
+
+
+@pytest.mark.parametrize("select", [False, True])
+@pytest.mark.parametrize("k", [37, 200, 256])          # one-CTA tiles, CTA pairs, every position (rotary table in a launch of its own)
+def test_refresh_sees_weights_written_by_the_kernel_before_it(k, select):
+    # stream order: the weights come from a kernel of the caller that lets its dependents start before it has written them
+    P, d, nh, nkv, dh = 256, 512, 4, 4, 128
+    late_writer = torch.cuda._compile_kernel(LATE_WRITER, "late_writer")
+    h, drift = I.make_refresh_inputs(1, P, d)
+    h, drift = h.cuda(), drift.cuda()
+    m = I.ModelCfg(1, d, nh, nkv, dh, 2 * d, 1024, I.DTYPE_BF16, 1e-5, 500000.0)
+    packed = Bd.pack_weights(m, I.make_weights(m, seed=5))
+    final, norm = packed["wqkv"][0], packed["norm1"][0]
+    scratch = torch.empty(Bd.polestar_k_refresh_scratch_bytes(1, k, d, nh, nkv, dh) + 1024, dtype=torch.uint8, device="cuda")
+    scratch = scratch[(-scratch.data_ptr()) % 1024:]
+    idx = torch.arange(k, dtype=torch.int32, device="cuda")[None].contiguous()
+    cnt = torch.full((1,), k, dtype=torch.int32, device="cuda")
+    sel_idx, sel_cnt = torch.zeros((1, P), dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def refresh(w, late):
+        kc, vc = (torch.zeros((1, P, nkv * dh), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        torch.cuda.synchronize()
+        if late:
+            late_writer(grid=(8, 1, 1), block=(256, 1, 1), args=[w, final, w.numel()])
+        if select:
+            Bd.polestar_k_select(drift, I.SELECT_TOPK_COUNT, k, 0.0, 0.0, sel_idx, sel_cnt)
+        Bd.polestar_k_refresh(h, idx, cnt, w, norm, kc, vc, None, k, nh, nkv, dh, m.rms_eps, m.rope_theta, scratch)
+        assert Bd.polestar_k_refresh_status(scratch, 1, k, d, dh) == Bd.OK
+        return kc, vc
+
+    want = refresh(final, False)
+    for a, b in zip(refresh(torch.zeros_like(final), True), want):
+        assert b.abs().max() > 0.1 and torch.allclose(a.float(), b.float(), atol=1e-5, rtol=2 ** -7)      # fp32 sums in another order
+
+
 # ------------------------------------------------------------------ confidence (a6, first half)
 @pytest.mark.parametrize("rows,V", [(32, 126464), (7, 1024), (1, 50)])
 def test_confidence_matches_oracle(rows, V):
