@@ -63,6 +63,7 @@ struct AttnMmaArgs {
     AttnArgs a;
     int rows_per_seq;   // forward rows per sequence (stand-alone: n_rows)
     int tiles_per_seq;
+    int vec;            // stored rows are read and written in 8-byte pieces (row length and bases allow it)
 };
 
 __global__ void __launch_bounds__(AT_WARPS * 32) attention_mma_kernel(AttnMmaArgs g) {
@@ -547,7 +548,7 @@ __global__ void __launch_bounds__(NW * 32) attention_sp_kernel(AttnMmaArgs g) {
     const float lse_lo = lse_sh[r_lo], lse_hi = lse_sh[r_hi];
     float* prev_lo = prev_sh[r_lo];
     float* prev_hi = prev_sh[r_hi];
-    const bool vec = (a.N & 1) == 0;
+    const bool vec = g.vec != 0;
 
     // ---- logp, KL, stored rows, P V ----------------------------------------------------------------
     float o[16][4];
@@ -943,7 +944,7 @@ __global__ void __launch_bounds__(BG_WARPS * 32) attention_big_kernel(AttnMmaArg
 
         // ---- pass 2: logp, KL, stored rows, P V ----------------------------------------------------------
         const bool with_v = a.out != nullptr;
-        const bool vec = (a.N & 1) == 0;
+        const bool vec = g.vec != 0;
         load_tile(0, with_v);
         if (n_tiles > 1) load_tile(1, with_v);
         if (n_tiles > 2) load_tile(2, with_v);
@@ -1059,6 +1060,7 @@ static cudaError_t attention_mma_set_attributes() {
 static cudaError_t launch_attention_mma(const AttnArgs& a, cudaStream_t st, int sm_count, int mode) {
     AttnMmaArgs g;
     g.a = a;
+    g.vec = stored_rows_in_pieces(a, 2) ? 1 : 0;
     const int batch = a.batch > 0 ? a.batch : 1;
     g.rows_per_seq = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
     g.tiles_per_seq = (g.rows_per_seq + AT_BM - 1) / AT_BM;

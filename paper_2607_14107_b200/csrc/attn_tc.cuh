@@ -129,6 +129,7 @@ struct Args {
     int tiles_per_seq;      // 128-row tiles per sequence
     int kt;                 // S tiles (128 keys) per CTA: 1 or 2
     int cl;                 // CTAs per cluster = key ranges per (row tile, head)
+    int vec;                // stored rows are read and written in 16-byte pieces (row length and bases allow it)
     int* status;            // set to 1 when a bounded wait gave up (null: nowhere to report)
 };
 
@@ -322,7 +323,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         // only what a lane does with its row depends on that row
         const bool warp_valid = __any_sync(0xffffffffu, valid) != 0;
         const bool use_old = prev != nullptr && a.record_kl != 0;
-        const bool vec = (a.N & 3) == 0;
+        const bool vec = g.vec != 0;
         // the stored row of the first key tile and (owner only) the stored log-sum-exp are read now, long before
         // they are needed: their latency hides behind the wait for S
         float old[64];

@@ -844,6 +844,10 @@ struct AttnArgs {
                                // written; all other K/V rows were complete before this forward was launched
     // stand-alone form: rows == null, row r belongs to sequence 0 and records into pprev[r]
 };
+// Whether every stored row can be read and written in pieces of `floats` (a power of two) floats.
+static inline bool stored_rows_in_pieces(const AttnArgs& a, int floats) {
+    return a.N % floats == 0 && (((uintptr_t)a.pprev | (uintptr_t)a.aprev) & (uintptr_t)(4 * floats - 1)) == 0;
+}
 
 template <typename T>
 __global__ void attention_simt_kernel(AttnArgs a) {

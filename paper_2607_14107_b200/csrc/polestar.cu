@@ -362,6 +362,7 @@ static int launch_attention_tc(MapCache& maps, const AttnArgs& a, cudaStream_t s
     const int tiles_k = (a.N + atc::KEYS - 1) / atc::KEYS;
     g.kt = tiles_k > atc::MAX_CL ? 2 : 1;
     g.cl = (tiles_k + g.kt - 1) / g.kt;
+    g.vec = stored_rows_in_pieces(a, 4) ? 1 : 0;
     g.status = status;
     const int dq = a.n_heads * a.head_dim, dkv = a.n_kv * a.head_dim;
     const int kv_batch = a.rows ? batch : 1;
@@ -407,7 +408,7 @@ static int launch_attention_stream(MapCache& maps, const AttnArgs& a, cudaStream
     // stored rows as tensor boxes where their layout allows (16-byte row pitch); the kernel decides per 32 rows
     const CUtensorMap *mp = mk, *mr = mk;
     g.maps = 0;
-    if (a.N % 4 == 0 && !(((uintptr_t)a.pprev | (uintptr_t)a.aprev) & 15)) {
+    if (stored_rows_in_pieces(a, 4)) {
         const uint64_t p_rows = a.rows ? (uint64_t)batch * (uint64_t)(a.cluster_K > 0 ? a.cluster_K : a.W_max) : (uint64_t)a.n_rows;
         if (a.pprev && (mp = maps.get_rows(a.pprev, p_rows, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 1;
         if (a.rows && a.aprev && (mr = maps.get_rows(a.aprev, (uint64_t)batch * a.B, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 2;
@@ -1629,18 +1630,16 @@ extern "C" int polestar_k_attention(const void* q, const void* k, const void* v,
     if (rc) return rc;
     const Switches sw = stand_alone_switches();
     if (dtype == POLESTAR_BF16 && head_dim == 128 && !sw.attn_simt) {
-        if (attention_stream_applies(a) && (sw.attn_kernel == 9 || (sw.attn_kernel == 0 && attention_prefers_stream(a))) &&
-            !((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v)) & 15)) {
-            MapCache maps;
-            maps.l2promo = sw.l2promo;
+        // Accesses: q, k and v 16 bytes in every kernel; the output 16 bytes in the streaming kernel, 8 in the cluster kernel,
+        // 4 in the warp-level ones.  (Stored rows of any alignment: each kernel falls back to single floats.)
+        const uintptr_t in = (uintptr_t)q | (uintptr_t)k | (uintptr_t)v, o = (uintptr_t)out;
+        if ((in & 15) || (o & 3)) return POLESTAR_E_INVAL;
+        MapCache maps;                     // the tensor maps of this call
+        maps.l2promo = sw.l2promo;
+        if (attention_stream_applies(a) && (sw.attn_kernel == 9 || (sw.attn_kernel == 0 && attention_prefers_stream(a))) && !(o & 15))
             return launch_attention_stream(maps, a, st, nullptr);
-        }
-        if ((sw.attn_kernel == 0 || sw.attn_kernel == 8) && attention_tc_applies(a) &&
-            !((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v)) & 15)) {
-            MapCache maps;                 // the three tensor maps of this call
-            maps.l2promo = sw.l2promo;
+        if ((sw.attn_kernel == 0 || sw.attn_kernel == 8) && attention_tc_applies(a) && !(o & 7))
             return launch_attention_tc(maps, a, st, nullptr);
-        }
         CK(launch_attention_mma(a, st, di.sm_count, sw.attn_kernel));
         return POLESTAR_OK;
     }

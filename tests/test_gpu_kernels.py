@@ -67,16 +67,47 @@ def test_attention_kernel_variants(monkeypatch, variant, R, N, nh, nkv):
     check_attention(torch.bfloat16, R, N, nh, nkv, 128)
 
 
-def check_attention(dtype, R, N, nh, nkv, dh):
+@pytest.mark.parametrize("prev_off,out_off", [(1, 0), (2, 8), (3, 4), (0, 2)])      # in elements: 4 / 8 / 12 bytes, 16 / 8 / 4 bytes
+@pytest.mark.parametrize("variant,R,N,nh,nkv", [
+    (9, 70, 404, 2, 1),            # streaming: several key tiles, a ragged second row tile
+    (8, 37, 500, 2, 1), (8, 20, 1028, 2, 2),       # one and two key tiles per CTA of the cluster kernel
+    (0, 128, 512, 2, 2),
+    (1, 20, 100, 2, 1), (2, 37, 200, 2, 1), (3, 37, 200, 2, 1), (5, 70, 300, 2, 1), (6, 21, 300, 2, 1),
+])
+def test_attention_alignment(monkeypatch, variant, R, N, nh, nkv, prev_off, out_off):
+    # stored rows at any float, outputs at any pair of elements: the result of aligned buffers' tolerance, nothing refused
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", str(variant))
+    Bd.polestar_reload_env()
+    check_attention(torch.bfloat16, R, N, nh, nkv, 128, prev_off, out_off)
+
+
+def test_attention_refuses_misaligned_operands():
+    # every bf16 kernel reads q, k and v in 16-byte pieces and writes the output in pairs
+    buf = torch.zeros(4 * 256 + 8, dtype=torch.bfloat16, device="cuda")
+    t, odd = buf[:1024].view(4, 256), buf[4:1028].view(4, 256)
+    for q, k, v, out in [(odd, t, t, t), (t, odd, t, t), (t, t, odd, t), (t, t, t, buf[1:1025].view(4, 256))]:
+        with pytest.raises(Bd.PolestarError) as e:
+            Bd.polestar_k_attention(q, k, v, None, None, None, out, 2, 2, 128)
+        assert e.value.code == Bd.E_INVAL
+
+
+def shifted(t, off):
+    """The same values `off` elements behind an allocation's start."""
+    buf = torch.zeros(t.numel() + off, dtype=t.dtype, device="cuda")
+    buf[off:].copy_(t.reshape(-1))
+    return buf[off:].view(t.shape)
+
+
+def check_attention(dtype, R, N, nh, nkv, dh, prev_off=0, out_off=0):
     q = rnd((R, nh * dh), 1, 1.0, dtype).cuda()
     k = rnd((N, nkv * dh), 2, 1.0, dtype).cuda()
     v = rnd((N, nkv * dh), 3, 1.0, dtype).cuda()
     prev_s = rnd((R, nh, N), 4, 1.0).double()
     prev = (prev_s - torch.logsumexp(prev_s, -1, keepdim=True)).float()
-    prev_dev = prev.clone().cuda()
+    prev_dev = shifted(prev, prev_off)
     lse_dev = torch.zeros((R, nh), device="cuda")          # stored pair (row, lse): log-probability = row - lse
     kl = torch.full((R, nh), -1.0, device="cuda")
-    out = torch.zeros((R, nh * dh), dtype=dtype, device="cuda")
+    out = shifted(torch.zeros((R, nh * dh), dtype=dtype), out_off)
     Bd.polestar_k_attention(q, k, v, prev_dev, lse_dev, kl, out, nh, nkv, dh)
     torch.cuda.synchronize()
     qn, kn, vn = bf16_np(q).reshape(R, nh, dh), bf16_np(k).reshape(N, nkv, dh), bf16_np(v).reshape(N, nkv, dh)
@@ -94,7 +125,7 @@ def check_attention(dtype, R, N, nh, nkv, dh):
     Bd.polestar_k_attention(q, k, v, prev_dev, lse_dev, kl2, None, nh, nkv, dh)
     torch.cuda.synchronize()
     assert np.abs(kl2.cpu().numpy()).max() < 1e-5
-    if dtype == torch.bfloat16:
+    if dtype == torch.bfloat16 and out_off % 8 == 0:      # (an output's alignment may choose another kernel than no output does)
         assert (kl2 == 0).all()            # unchanged rows: exactly zero drift (same bits in, same bits out)
     assert (kl.cpu().numpy() > -1e-4).all()
     # Pinsker bound of Appendix B, Prop. 2 with the current value rows
