@@ -853,10 +853,10 @@ struct Path {
         int rc;
 
         const double esd = (double)es;
-        const double Mlive = sparse ? (double)bs * (B + std::min(sd.W, (int)(p.select_mode == POLESTAR_SELECT_TOPK_FRAC
-                                                       ? floorf(p.select_frac * (float)sd.W + 0.5f)
-                                                       : (p.select_mode == POLESTAR_SELECT_TOPK_COUNT ? p.select_k : sd.W))))
-                                    : (double)M;
+        // what a top-k selection takes at most of a sequence's window (the kernels' k and the row bound below are this number)
+        const int sel_k = p.select_mode == POLESTAR_SELECT_TOPK_FRAC ? (int)floorf(p.select_frac * (float)sd.W + 0.5f) : p.select_k;
+        const bool sel_topk = p.select_mode == POLESTAR_SELECT_TOPK_FRAC || p.select_mode == POLESTAR_SELECT_TOPK_COUNT;
+        const double Mlive = sparse ? (double)bs * (B + std::min(sd.W, sel_topk ? sel_k : sd.W)) : (double)M;
         {
             Scope sc(c, POLESTAR_PROF_STAGE, (double)M * d * (esd + 4), 0, 2);
             CK(launch_k(build_rows_kernel, dim3((M + 255) / 256), dim3(256), 0, st, sd, b.rows));
@@ -980,7 +980,7 @@ struct Path {
                 s.forced_idx = b.forced_idx + (size_t)l * bs * Wm; s.forced_cnt = b.forced_cnt + (size_t)l * bs;
                 s.list = b.list; s.list_count = b.list_count; s.stats = b.stats; s.n_heads = m.n_heads;
                 s.mode = p.select_mode;
-                s.k = p.select_mode == POLESTAR_SELECT_TOPK_FRAC ? (int)floorf(p.select_frac * (float)sd.W + 0.5f) : p.select_k;
+                s.k = sel_k;
                 s.W_max = Wm; s.thresh = p.select_thresh; s.floor_ = p.drift_floor;
                 s.ct = ct; s.cluster_k = p.cluster_k;
                 if (sel_in_gemm) { sf.on = 1; sf.sd = sd; sf.a = s; }
@@ -996,11 +996,9 @@ struct Path {
             // Dream shape, 512 rows of which 224 are live: 519 -> 452 ms.
             // Thresholds, cluster members and imposed selections can reach every window row.
             int M2 = M;
-            if (sparse && Kp == 0 && !c->forced_select &&
-                (p.select_mode == POLESTAR_SELECT_TOPK_FRAC || p.select_mode == POLESTAR_SELECT_TOPK_COUNT)) {
-                const int k = p.select_mode == POLESTAR_SELECT_TOPK_FRAC ? (int)floorf(p.select_frac * (float)sd.W + 0.5f) : p.select_k;
+            if (sparse && Kp == 0 && !c->forced_select && sel_topk) {
                 M2 = bs * B;
-                for (int s = 0; s < bs; ++s) if (sd.refresh.v[s]) M2 += std::min(std::max(k, 0), sd.W);
+                for (int s = 0; s < bs; ++s) if (sd.refresh.v[s]) M2 += std::min(std::max(sel_k, 0), sd.W);
             }
             // O projection -> RMSNorm -> gate/up -> down as one persistent kernel when the step is small enough
             bool chained = false;

@@ -66,8 +66,19 @@ def impose_codes(gpu, ora, p, m):
             gpu.force_hcodes(l, mask, codes, scales)
 
 
-def run_forced(name, n_steps, std=0.02, force_labels=True, **kw):
-    """The CUDA path replays the oracle's refresh sets and commits; every step's numbers are compared."""
+def own_selection(gpu, m, p):
+    """The CUDA path's selected window rows of the last step, per sequence and layer."""
+    sel = [[] for _ in range(p.batch)]
+    for l in range(m.n_layers):
+        cnt, idx = gpu.read(Bd.READ_SEL_COUNT, l), gpu.read(Bd.READ_SEL_IDX, l)
+        for s in range(p.batch):
+            sel[s].append(idx[s, :cnt[s]].tolist())
+    return sel
+
+
+def run_forced(name, n_steps, std=0.02, force_labels=True, free_select=False, **kw):
+    """The CUDA path replays the oracle's refresh sets and commits; every step's numbers are compared.  free_select: the CUDA
+    path selects on its own (which lays the sparse forward out for the rows a selection can have) and the oracle replays that."""
     m, p, gpu, ora = setup(name, std, **kw)
     tol = TOL[m.dtype]
     L = m.n_layers
@@ -77,7 +88,13 @@ def run_forced(name, n_steps, std=0.02, force_labels=True, **kw):
     for step in range(n_steps):
         if ora.done:
             break
-        ora.step()     # oracle first, so that its refresh sets can be imposed on the CUDA step
+        if free_select and step > 0:
+            info = gpu.step()
+            if 0 < info.n_refreshing < p.batch:
+                seen["mixed"] = seen.get("mixed", 0) + 1
+            ora.step(forced_sel=own_selection(gpu, m, p))
+        else:
+            ora.step()     # oracle first, so that its refresh sets can be imposed on the CUDA step
         tr = ora.seqs[0].trace
         cluster = p.select_mode == I.SELECT_CLUSTER_TOPK
         if step > 0:
@@ -91,14 +108,15 @@ def run_forced(name, n_steps, std=0.02, force_labels=True, **kw):
                     gpu.force_labels(l, lab[:, :len(ora.seqs[0].labels[l])])
             if p.flags & I.FLAG_NVFP4_HCACHE:
                 impose_codes(gpu, ora, p, m)
-            if tr["kind"] == "within" and tr["refresh"]:
-                for l in range(L):
-                    sel = np.full((p.batch, gpu.W_max), -1, np.int32)
-                    for s in range(p.batch):
-                        sl = ora.seqs[s].trace["sel"][l]
-                        sel[s, :len(sl)] = sl
-                    gpu.force_select(l, sel)
-            info = gpu.step()
+            if not free_select:
+                if tr["kind"] == "within" and tr["refresh"]:
+                    for l in range(L):
+                        sel = np.full((p.batch, gpu.W_max), -1, np.int32)
+                        for s in range(p.batch):
+                            sl = ora.seqs[s].trace["sel"][l]
+                            sel[s, :len(sl)] = sl
+                        gpu.force_select(l, sel)
+                info = gpu.step()
             assert {0: "entry_full", 1: "entry_window", 2: "within"}[info.kind] == tr["kind"]
         if step == 0 and (p.flags & I.FLAG_NVFP4_HCACHE):
             # the first block entry ran inside polestar_init: bring its codes in line before anything reads the cache
@@ -300,10 +318,12 @@ def test_c1b_streaming_attention_stored_row_forms(monkeypatch, prompt_len):
     assert seen["refresh"] > 3
 
 
-def test_c1b_tall_gemm_tiles(monkeypatch):
-    # 256-token CTA tiles (two MMAs per k step on one weight tile) for every projection of more than 129 rows: block
-    # entries of a batch (ragged: 3 x 146 and 3 x 90 rows), refresh steps (3 x 72 rows), whole and split tiles
-    monkeypatch.setenv("POLESTAR_GEMM_TALL_ROWS", "130")
+@pytest.mark.parametrize("pair_rows", [1 << 30, 1])
+def test_c1b_gemm_tile_forms(monkeypatch, pair_rows):
+    # the form that the default rule does not take: projections of more than 128 rows as several 128-token tiles of single
+    # CTAs (devices without resident pairs), projections of up to 128 rows on CTA pairs (a pair tile's second half empty);
+    # block entries of a batch (ragged: 3 x 146 and 3 x 90 rows), refresh steps (3 x 72 rows), whole and split tiles
+    monkeypatch.setenv("POLESTAR_GEMM_PAIR_ROWS", str(pair_rows))
     seen = run_forced("c1b", 12, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=3, prompt_len=50, gen_len=96, block=24,
                       max_steps=16)
     assert seen["refresh"] > 3 and seen["entry_window"] > 0
@@ -311,7 +331,7 @@ def test_c1b_tall_gemm_tiles(monkeypatch):
 
 @pytest.mark.parametrize("pre,suf", [(3, 1), (2, 2)])
 def test_c1b_wide_windows(pre, suf):
-    # refresh steps of 160 rows (32 active + 128 window rows): every projection runs as one 256-token tile, the selection
+    # refresh steps of 160 rows (32 active + 128 window rows): every projection runs on one row of pair tiles, the selection
     # rides on the O projection
     seen = run_forced("c1b", 12, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, prompt_len=128, gen_len=128, block=32,
                       max_steps=16, win_prefix_blocks=pre, win_suffix_blocks=suf)
@@ -335,14 +355,32 @@ def test_c1b_epilogue_warp_groups(monkeypatch, groups):
     assert seen["refresh"] > 2
 
 
-def test_c1b_gemm_cta_pairs(monkeypatch):
-    # CTA pairs (tcgen05 cta_group::2: one MMA over two SMs, each loading half of the weight tile) for every projection of
-    # more than 129 rows: ragged block entries of a batch (a pair tile's second half partly or wholly empty), refresh
-    # steps, whole and split tiles, in-place L2 reductions of the O / down projections
-    monkeypatch.setenv("POLESTAR_GEMM_PAIR_ROWS", "130")
+def test_c1b_gemm_cta_pairs():
+    # CTA pairs (tcgen05 cta_group::2: one MMA over two SMs, each loading half of the weight tile), the default for every
+    # projection of more than 128 rows: ragged block entries of a batch (a pair tile's second half partly or wholly empty),
+    # refresh steps, whole and split tiles, in-place L2 reductions of the O / down projections
     seen = run_forced("c1b", 12, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=3, prompt_len=50, gen_len=96, block=24,
                       max_steps=16)
     assert seen["refresh"] > 3 and seen["entry_window"] > 0
+
+
+@pytest.mark.parametrize("kw", [
+    dict(batch=3, prompt_len=200, gen_len=128, block=64),                                   # 768 rows of which 336: O projection on the gathered rows
+    dict(batch=6, prompt_len=130, gen_len=128, block=64, tau_upd=20, tau_s=0.5),            # some sequences refresh, others do not
+    dict(batch=1, prompt_len=300, gen_len=256, block=128),                                  # 384 window rows: radix selection, 512 rows of which 224
+    dict(batch=1, prompt_len=128, gen_len=128, block=32, win_prefix_blocks=3),              # 160 rows: the selection rides on a pair launch
+    dict(batch=3, prompt_len=200, gen_len=128, block=64, select_mode=I.SELECT_TOPK_COUNT, select_k=10 ** 6),
+    dict(batch=3, prompt_len=200, gen_len=128, block=64, select_mode=I.SELECT_TOPK_COUNT, select_k=17),
+    dict(batch=3, prompt_len=200, gen_len=128, block=64, select_mode=I.SELECT_TOPK_COUNT, select_k=-3),
+    dict(batch=3, prompt_len=200, gen_len=128, block=64, select_mode=I.SELECT_THRESHOLD, select_thresh=1e-3),
+])
+def test_c1b_own_selection_matches_oracle(kw):
+    # refresh steps with the library's own selection: the sparse forward is laid out for the rows that can be selected
+    kw = {**dict(tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, max_steps=32), **kw}
+    seen = run_forced("c1b", 5, free_select=True, **kw)
+    assert seen["refresh"] >= 2, seen
+    if kw["tau_upd"] >= 0:
+        assert seen["mixed"] > 0, seen
 
 
 def test_block_entry_of_a_large_batch_with_a_wide_feed_forward_network():

@@ -20,7 +20,7 @@ from paper_2607_14107_b200 import binding as Bd
 from paper_2607_14107_b200 import inputs as I
 
 from parity import check_commit_quantities, new_stats, outside_fraction
-from test_gpu_decode import impose_codes
+from test_gpu_decode import impose_codes, own_selection
 
 pytestmark = pytest.mark.gpu
 TOL = 2e-2
@@ -100,7 +100,7 @@ def compare_step(gpu, ora, m, p, step):
             close(gpu.read(Bd.READ_HCACHE, l)[s, :W], ora.seqs[s].Hc[l], TOL, f"step {step} H l{l}", depth=l)
 
 
-def run_reduced_depth(m, p, n_within):
+def run_reduced_depth(m, p, n_within, free_select=False):
     w = I.make_weights(m, seed=0, device="cuda")
     packed = Bd.pack_weights(m, w)
     wn = I.weights_to_numpy(w)
@@ -125,7 +125,11 @@ def run_reduced_depth(m, p, n_within):
         y_before = ora.tokens().copy()
         forced_commit(gpu, ora, ora.commit(), p, m, y_before, stats)
         assert np.array_equal(gpu.tokens(), ora.tokens())
-        ora.step()
+        if free_select:                 # the library's own selection, replayed by the oracle
+            gpu.step()
+            ora.step(forced_sel=own_selection(gpu, m, p))
+        else:
+            ora.step()
         tr = ora.seqs[0].trace
         if cluster and tr["kind"] != "within":
             for l in range(m.n_layers):
@@ -135,14 +139,15 @@ def run_reduced_depth(m, p, n_within):
                 gpu.force_labels(l, lab)
         if quant:
             impose_codes(gpu, ora, p, m)
-        if tr["kind"] == "within" and tr["refresh"]:
-            for l in range(m.n_layers):
-                sel = np.full((p.batch, gpu.W_max), -1, np.int32)
-                for s in range(p.batch):
-                    sl = ora.seqs[s].trace["sel"][l]
-                    sel[s, :len(sl)] = sl
-                gpu.force_select(l, sel)
-        gpu.step()
+        if not free_select:
+            if tr["kind"] == "within" and tr["refresh"]:
+                for l in range(m.n_layers):
+                    sel = np.full((p.batch, gpu.W_max), -1, np.int32)
+                    for s in range(p.batch):
+                        sl = ora.seqs[s].trace["sel"][l]
+                        sel[s, :len(sl)] = sl
+                    gpu.force_select(l, sel)
+            gpu.step()
         compare_step(gpu, ora, m, p, step)
         kinds.append(tr["kind"] + ("_refresh" if tr["kind"] == "within" and tr["refresh"] else ""))
     gpu.destroy()
@@ -154,6 +159,15 @@ def test_c2_shape_reduced_depth_matches_oracle():
     m = I.reduced_depth(m, 2)
     p = dataclasses.replace(p, tau_upd=-1, flags=p.flags | I.FLAG_KEEP_HIDDEN)
     run_reduced_depth(m, p, n_within=1)
+
+
+def test_c2_widths_own_selection_on_a_pair_launch_matches_oracle():
+    # 32 active + 128 window rows of one sequence: projections on CTA pairs, the library's own selection inside the O projection
+    m, p = I.config("c2")
+    m = I.reduced_depth(m, 1)
+    p = dataclasses.replace(p, tau_upd=-1, win_prefix_blocks=3, flags=p.flags | I.FLAG_KEEP_HIDDEN)
+    kinds = run_reduced_depth(m, p, n_within=2, free_select=True)
+    assert kinds == ["entry_full", "within_refresh", "within_refresh"], kinds
 
 
 def test_c3_widths_gqa_batch_matches_oracle():

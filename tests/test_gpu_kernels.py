@@ -228,14 +228,16 @@ def test_refresh_chain_matches_oracle(P, d, nh, nkv, k, batch):
     check_refresh_chain(P, d, nh, nkv, k, batch)
 
 
+@pytest.mark.parametrize("pair_rows", [200, 1 << 30])
 @pytest.mark.parametrize("P,d,nh,nkv,k,batch", [
     (300, 256, 2, 2, 300, 1),          # 300 rows: the second pair tile's second half is empty
     (3400, 256, 2, 2, 3300, 4),        # more pair tiles than pairs: whole tiles round-robin + stream-K tail
     (4096, 4096, 32, 32, 410, 8),      # the micro-benchmark's shape, 3280 rows
 ])
-def test_refresh_chain_on_cta_pairs(monkeypatch, P, d, nh, nkv, k, batch):
-    # the same projection on CTA pairs (tcgen05 cta_group::2): each CTA of a pair loads half of the weight tile
-    monkeypatch.setenv("POLESTAR_GEMM_PAIR_ROWS", "200")
+def test_refresh_chain_tile_forms(monkeypatch, P, d, nh, nkv, k, batch, pair_rows):
+    # the same projection on CTA pairs (tcgen05 cta_group::2: each CTA of a pair loads half of the weight tile), and as several
+    # 128-token tiles of single CTAs (the form for devices without resident pairs)
+    monkeypatch.setenv("POLESTAR_GEMM_PAIR_ROWS", str(pair_rows))
     Bd.polestar_reload_env()           # the stand-alone calls read the switches once, not per launch
     check_refresh_chain(P, d, nh, nkv, k, batch)
 
