@@ -451,7 +451,9 @@ struct Buffers {
 
 static const int CONF_CHUNKS = 32;
 static const int FORCED_COMMIT_MAX = 512;
-static const size_t GEMM_PARTIAL_BYTES = ((size_t)80 << 20) + 16384 + 65536;   // at least 2 slots x 148 CTAs x 128 x 256 fp32
+// partial tiles, two slots of 128 x 256 fp32 per CTA (38.8 MB at 148 SMs; a device with more than 160 gets a smaller grid), and
+// behind them the time stamps of POLESTAR_TRACE builds
+static const size_t GEMM_PARTIAL_BYTES = (size_t)160 * 2 * tc::BLOCK_T * tc::BLOCK_F * 4 + 16384 + 65536;
 // One projection of a chained launch (gemm_chain.cuh): A [M, K] x W [N_out, K]^T with epilogue `epi`.
 struct ChainSpec {
     const void* A; const void* W;
