@@ -236,7 +236,7 @@ struct SkArgs {
     int tiles_f, tiles_t;
     float* partial;     // [2 * gridDim.x][BLOCK_T][BLOCK_F] fp32
     int* tile_counter;  // arrivals [split tile] and, done_offset further on, finished shares [split tile]; zero before launch,
-                        // zero again after.  Split tiles count from sk_whole_tiles(...) * G on (times two CTAs of a pair)
+                        // zero again after.  Split tiles count from sk_whole_tiles(...) * G on; both CTAs of a pair count
     int done_offset;
     int* status;        // set to 1 on a wait time-out
     int w_stream;       // 1: every weight byte is read once by this launch: load it with the evict_first L2 policy
@@ -324,8 +324,8 @@ __device__ __forceinline__ void red_add_v4(float* dst, uint32_t a, uint32_t b, u
 // (8192 x 24576 x 4096: 133 cycles per MMA without loads; with them 1.3 - 1.5 PFLOP/s at 1.4 - 1.5 GHz).  Measured against
 // two 128-row MMAs per k step on one CTA (256-token tile, no epilogue overlap; removed) and against 128-token tiles,
 // K = 4096: 256 x 12288 47 / 60 / 64 us, 512 x 24576 101 / 130 / 110 us, 896 x 24576 158 / 207 / 161 us.  The schedule
-// treats the pair as one CTA (stream-K ranges, whole tiles first); everything after the MMAs (epilogue, partial tiles,
-// reduction pass) is per CTA on its own 128 rows, with partial-tile slots and tile counters of its own.
+// treats the pair as one CTA (stream-K ranges, whole tiles first); the epilogue and the partial tiles are per CTA on its own
+// 128 rows, the reduction pass deals the live rows of the whole tile over the CTAs of all contributing pairs.
 template <typename T, int EPI, int CG = 1>
 __global__ void __launch_bounds__(FIX_THREADS, 1)
 gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_a,
@@ -671,7 +671,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (!whole && !((EPI == EPI_RESID || EPI == EPI_DOWN) && e.accumulate)) {
                 __threadfence();
                 asm volatile("bar.sync 1, %0;" ::"r"(128 * groups) : "memory");
-                if (threadIdx.x == 64) atomicAdd(&g.tile_counter[(tile - tile_base) * CG + rank], 1);
+                if (threadIdx.x == 64) atomicAdd(&g.tile_counter[tile - tile_base], 1);
             }
             ++seg;
         }
@@ -700,10 +700,11 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                     const int before = fx_par[f][3], mine = fx_par[f][4], w_all = fx_par[f][5];
                     f_tf[f] = fx_par[f][6]; f_tt[f] = fx_par[f][7];
                     const int tile_t = f_tt[f];
-                    const int n_live = max(0, min(BT, Mv - (tile_t * CG + rank) * BT));
-                    const int n_items = n_live * (BLOCK_F / 16);
-                    f_lo[f] = (n_items * before) / w_all;
-                    f_n[f] = (n_items * (before + mine)) / w_all - f_lo[f];
+                    // (a pair's share is split evenly between its CTAs, whichever half of the tile the rows are in)
+                    const int n_live = max(0, min(CG * BT, Mv - tile_t * CG * BT));
+                    const int n_items = n_live * (BLOCK_F / 16), lo = CG * before + rank * mine;
+                    f_lo[f] = (n_items * lo) / (CG * w_all);
+                    f_n[f] = (n_items * (lo + mine)) / (CG * w_all) - f_lo[f];
                 }
             }
             const int total = f_n[0] + f_n[1];
@@ -711,15 +712,14 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 // pull what the epilogue of this thread's first item reads into L1 while the tiles are still arriving
                 const int f = (int)threadIdx.x < f_n[0] ? 0 : 1;
                 const int item = f_lo[f] + (int)threadIdx.x - (f ? f_n[0] : 0);
-                const int tile = fix_tile[f];
-                epilogue_prefetch<T, EPI>(e, (f_tt[f] * CG + rank) * BT + item / (BLOCK_F / 16), f_tf[f] * BLOCK_F + (item % (BLOCK_F / 16)) * 16);
+                epilogue_prefetch<T, EPI>(e, f_tt[f] * CG * BT + item / (BLOCK_F / 16), f_tf[f] * BLOCK_F + (item % (BLOCK_F / 16)) * 16);
             }
             if (threadIdx.x == 64) {
                 // bounded wait until all contributors have published their partial tiles
                 const long long t0 = clock64();
                 int ok = 1;
                 for (int f = 0; f < n_fix && ok; ++f) {
-                    while (ld_acquire_gpu(&g.tile_counter[fix_tile[f] * CG + rank]) < f_nseg[f]) {
+                    while (ld_acquire_gpu(&g.tile_counter[fix_tile[f]]) < f_nseg[f] * CG) {
                         if (*abort_flag || clock64() - t0 > WAIT_LIMIT_CYCLES) { ok = 0; *abort_flag = 1; break; }
                         __nanosleep(64);
                     }
@@ -736,9 +736,8 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                     const int i = i4 >> 2;
                     const int f = i < f_n[0] ? 0 : 1;
                     const int item = f_lo[f] + i - (f ? f_n[0] : 0);
-                    const int tile = fix_tile[f];
                     const int c_lo = f_clo[f], nseg = f_nseg[f];
-                    const int tl = item / (BLOCK_F / 16), c0 = (item % (BLOCK_F / 16)) * 16 + (i4 & 3) * 4;
+                    const int tl = item / (BLOCK_F / 16), half = tl / BT, c0 = (item % (BLOCK_F / 16)) * 16 + (i4 & 3) * 4;
                     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
                     for (int sg0 = 0; sg0 < nseg; sg0 += 16) {
                         float4 tv[16];
@@ -747,21 +746,20 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                             const int cc = c_lo + sg0 + j;
                             const int wsl = (cc == c_lo) ? 1 : 0;
                             tv[j] = (sg0 + j < nseg)
-                                        ? __ldcg(reinterpret_cast<const float4*>(g.partial + ((size_t)(2 * (cc * CG + rank) + wsl) * BT + tl) * BLOCK_F + c0))
+                                        ? __ldcg(reinterpret_cast<const float4*>(g.partial + ((size_t)(2 * (cc * CG + half) + wsl) * BT + (tl - half * BT)) * BLOCK_F + c0))
                                         : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) { acc.x += tv[j].x; acc.y += tv[j].y; acc.z += tv[j].z; acc.w += tv[j].w; }
                     }
-                    epilogue4<T, EPI>(e, (f_tt[f] * CG + rank) * BT + tl, f_tf[f] * BLOCK_F + c0, acc);
+                    epilogue4<T, EPI>(e, f_tt[f] * CG * BT + tl, f_tf[f] * BLOCK_F + c0, acc);
                 }
             } else if (last_sh) {
                 for (int i = (int)threadIdx.x; i < total; i += FIX_THREADS) {
                     const int f = i < f_n[0] ? 0 : 1;
                     const int item = f_lo[f] + i - (f ? f_n[0] : 0);
-                    const int tile = fix_tile[f];
                     const int c_lo = f_clo[f], nseg = f_nseg[f];
-                    const int tl = item / (BLOCK_F / 16), c0 = (item % (BLOCK_F / 16)) * 16;
+                    const int tl = item / (BLOCK_F / 16), half = tl / BT, c0 = (item % (BLOCK_F / 16)) * 16;
                     float acc[16];
 #pragma unroll
                     for (int x = 0; x < 16; ++x) acc[x] = 0.f;
@@ -775,7 +773,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                                 // (only the tile's first contributor can start at or before the tile's first unit)
                                 const int wsl = (cc == c_lo) ? 1 : 0;
                                 const float4* ps = reinterpret_cast<const float4*>(
-                                    g.partial + ((size_t)(2 * (cc * CG + rank) + wsl) * BT + tl) * BLOCK_F + c0);
+                                    g.partial + ((size_t)(2 * (cc * CG + half) + wsl) * BT + (tl - half * BT)) * BLOCK_F + c0);
 #pragma unroll
                                 for (int x = 0; x < 4; ++x) tv[j][x] = __ldcg(ps + x);
                             } else {
@@ -791,7 +789,7 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                                 acc[4 * x + 2] += tv[j][x].z; acc[4 * x + 3] += tv[j][x].w;
                             }
                     }
-                    const int mm = (f_tt[f] * CG + rank) * BT + tl;
+                    const int mm = f_tt[f] * CG * BT + tl;
                     const int n0 = f_tf[f] * BLOCK_F;
                     epilogue16<T, EPI>(e, mm, n0 + c0, acc);
                 }
@@ -801,9 +799,9 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (threadIdx.x == 64 && last_sh) {
                 // the last contributor to finish its share re-arms the tile's counters for the next launch
                 for (int f = 0; f < n_fix; ++f) {
-                    const int tile = fix_tile[f] * CG + rank;
+                    const int tile = fix_tile[f];
                     const int prev = atomicAdd(&g.tile_counter[g.done_offset + tile], 1);
-                    if (prev == f_nseg[f] - 1) { g.tile_counter[tile] = 0; g.tile_counter[g.done_offset + tile] = 0; }
+                    if (prev == f_nseg[f] * CG - 1) { g.tile_counter[tile] = 0; g.tile_counter[g.done_offset + tile] = 0; }
                 }
             }
         }

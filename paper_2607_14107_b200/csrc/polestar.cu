@@ -304,7 +304,7 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
         while (G > 1 && ((size_t)2 * G * BT * tc::BLOCK_F * 4 + 16384 + 65536 > ws.partial_bytes)) --G;
     }
     // (always holds: fewer than 2 G tiles are split)
-    if ((tiles_f * tiles_t - tc::sk_whole_tiles(tiles_f * tiles_t, (int)G, K / 64) * (int)G) * (pair ? 2 : 1) > ws.n_counters / 2) return POLESTAR_E_INVAL;
+    if (tiles_f * tiles_t - tc::sk_whole_tiles(tiles_f * tiles_t, (int)G, K / 64) * (int)G > ws.n_counters / 2) return POLESTAR_E_INVAL;
     tc::SkArgs g;
     g.M = M; g.N_out = N_out; g.K = K; g.tiles_f = tiles_f; g.tiles_t = tiles_t;
     // Three stages (145 KB) for the weight-bound steps: measured +2 % tokens/s over four (the HBM stream needs no more in
@@ -1736,10 +1736,10 @@ extern "C" int polestar_k_refresh(const void* h, const int32_t* idx, const int32
     const int M = batch * max_rows;
     const int dq = n_heads * head_dim, dkv = n_kv * head_dim;
     // The scratch is caller memory with unknown contents: the split tiles' counters (arrivals, then finished shares) must start
-    // at zero.  Only as many as this GEMM can use are cleared: fewer than two per SM (sk_whole_tiles; a pair tile has one for
-    // each of its 128-row halves), and no more than it has 128-row tiles, the empty second half of a pair tile included.
+    // at zero.  Only as many as this GEMM can use are cleared: fewer than two per SM (sk_whole_tiles), and no more than it has
+    // 128-row tiles.
     const long long tiles_f = (dq + 2 * dkv + tc::BLOCK_F - 1) / tc::BLOCK_F;
-    const long long tiles = tiles_f * ((M + tc::BLOCK_T - 1) / tc::BLOCK_T + 1);
+    const long long tiles = tiles_f * ((M + tc::BLOCK_T - 1) / tc::BLOCK_T);
     const int n_cnt = (int)(2 * std::min<long long>(tiles, 2LL * di.sm_count));
     ws.counters = (int*)(sc + off_cnt); ws.n_counters = n_cnt; ws.status = (int*)(sc + off_status);
     const int half = head_dim / 2;
