@@ -276,6 +276,21 @@ static void sk_grid(const GemmWs& ws, int M, int N_out, int K, long long* U, lon
     *G = g;
 }
 
+// Whether a projection with enough rows for CTA pairs is better off on 128-row tiles of single CTAs: where those fill whole
+// waves, so that (nearly) none is split, and the 256-row pair tiles, padded to an even number of halves, neither fill theirs
+// nor make up for the padding.  A pair wave takes about 0.8 of a single one (32 KB of operands per CTA and k block instead of
+// 48), a wave that is partly filled costs its share and a reduction pass, about a quarter wave.  Gather and projection, single /
+// pair, us: K = 4096, 257 - 384 rows x 12288 36 / 46 - 50, x 24576 54 - 58 / 65 - 74, 1100 rows x 4096 38 / 55; on the other
+// side 400 x 12288 54 / 50, 640 x 12288 62 / 48, 1100 x 24576 166 / 156, 2300 x 37888 (K = 3584) 424 / 325.
+static bool single_tiles_win(const GemmWs& ws, int tiles_f, int M) {
+    const long long t1 = (long long)tiles_f * ((M + tc::BLOCK_T - 1) / tc::BLOCK_T), t2 = (long long)tiles_f * ((M + 2 * tc::BLOCK_T - 1) / (2 * tc::BLOCK_T));
+    const long long last1 = t1 % ws.sms, last2 = t2 % ws.pairs;
+    if (last1 != 0 && last1 * 10 < 9LL * ws.sms) return false;
+    const double waves1 = (double)((t1 + ws.sms - 1) / ws.sms);
+    const double waves2 = (double)t2 / ws.pairs + (last2 == 0 || last2 * 10 >= 9LL * ws.pairs ? 0.0 : 0.25);
+    return waves1 < 0.8 * waves2;
+}
+
 template <int EPI>
 static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const void* W, int M,
                           int N_out, int K, const EpiArgs& e, cudaStream_t st,
@@ -286,9 +301,10 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     // More than one token tile of 128 rows (POLESTAR_GEMM_PAIR_ROWS): CTA pairs on tiles of 256 tokens (one MMA over both SMs,
     // half a weight tile each).  Up to 256 rows that is still a single token tile: every weight byte is read once and
     // streamed with evict_first.
-    const bool pair = ws.pairs > 0 && M >= ws.sw.pair_rows;
+    const int tiles_f = N_out / tc::BLOCK_F;
+    const bool pair = ws.pairs > 0 && M >= ws.sw.pair_rows && !single_tiles_win(ws, tiles_f, M);
     const int BT = tc::BLOCK_T * (pair ? 2 : 1);           // tokens per scheduling unit's tile
-    const int tiles_f = N_out / tc::BLOCK_F, tiles_t = (M + BT - 1) / BT;
+    const int tiles_t = (M + BT - 1) / BT;
     // When a multiple of the tile count fits on >= 85 % of the SMs, the grid takes it: CTA ranges then never
     // cross a tile boundary, so every CTA has one segment (one fix-up instead of two, or none at all).
     const CUtensorMap* mw = maps.get(W, (uint64_t)N_out * (uint64_t)(K / 64), 64, pair ? tc::BLOCK_F / 2 : tc::BLOCK_F);

@@ -221,6 +221,8 @@ def test_select_zero_drift_and_nan():
     (256, 256, 2, 2, 37, 1), (512, 512, 4, 1, 128, 2), (300, 256, 2, 2, 300, 1),
     (3400, 256, 2, 2, 3300, 4),       # 13200 rows: 312 output tiles > SM count (whole tiles round-robin + stream-K tail)
     (2000, 256, 2, 2, 1700, 2),       # 3400 rows: 27 token tiles (two raster chunks), fewer tiles than SMs
+    (300, 256, 32, 32, 257, 1), (400, 256, 32, 32, 384, 1),      # 3 x 48 tiles of single CTAs, one wave, none split
+    (1200, 256, 16, 8, 1100, 1),      # 9 x 16 tiles of single CTAs (80 pair tiles would not fill two waves of 74)
     # the refresh micro-benchmark's own shape (LLaDA-8B layer: d 4096 = 64 k-blocks, 32 x 128 heads, 4096 positions)
     (4096, 4096, 32, 32, 41, 1), (4096, 4096, 32, 32, 1024, 1), (4096, 4096, 32, 32, 410, 8),
 ])
