@@ -101,13 +101,16 @@ static Switches stand_alone_switches() {
 // ------------------------------------------------------------------------------------------
 // per-device facts: SM count, dynamic shared-memory attributes of the kernels, built-in scratch
 // ------------------------------------------------------------------------------------------
-struct DevInfo { bool ready = false; int sm_count = 0; int gemm_pairs = 0; };
+// clusters of the cluster attention kernel that are resident at once, by key tiles per CTA (less one) and CTAs per cluster
+struct AttnClusters { int n[atc::MAX_KT][atc::MAX_CL + 1] = {}; };
+struct DevInfo { bool ready = false; int sm_count = 0; int gemm_pairs = 0; AttnClusters attn; };
 static const int MAX_DEVICES = 64;
 static DevInfo g_dev[MAX_DEVICES];
 static int g_last_sm_count = 0;
 
 static cudaError_t set_kernel_attributes();
 static int resident_gemm_pairs();
+static int resident_attention_clusters(int kt, int cl);
 // Facts of the CURRENT device; the first call on a device queries it and raises the shared-memory limits of
 // every kernel that needs more than the default there (function attributes are per device).
 static int device_info(DevInfo* out) {
@@ -120,6 +123,8 @@ static int device_info(DevInfo* out) {
         CK(cudaDeviceGetAttribute(&di.sm_count, cudaDevAttrMultiProcessorCount, dev));
         CK(set_kernel_attributes());
         di.gemm_pairs = resident_gemm_pairs();
+        for (int kt = 1; kt <= atc::MAX_KT; ++kt)
+            for (int cl = 1; cl <= atc::MAX_CL; ++cl) di.attn.n[kt - 1][cl] = resident_attention_clusters(kt, cl);
         di.ready = true;
     }
     g_last_sm_count = di.sm_count;
@@ -367,6 +372,11 @@ static bool attention_tc_applies(const AttnArgs& a) {
     return a.head_dim == atc::DH && a.N <= atc::MAX_N && a.N > 0 && (a.n_heads * a.head_dim) % 64 == 0 &&
            (a.n_kv * a.head_dim) % 64 == 0;
 }
+static void attention_tc_split(int N, int* kt, int* cl) {      // key tiles per CTA, CTAs per cluster
+    const int tiles = (N + atc::KEYS - 1) / atc::KEYS;
+    *kt = tiles > atc::MAX_CL ? 2 : 1;
+    *cl = (tiles + *kt - 1) / *kt;
+}
 static int launch_attention_tc(MapCache& maps, const AttnArgs& a, cudaStream_t st, int* status) {
     if (a.n_rows <= 0) return POLESTAR_OK;
     atc::Args g;
@@ -375,9 +385,7 @@ static int launch_attention_tc(MapCache& maps, const AttnArgs& a, cudaStream_t s
     const int batch = a.batch > 0 ? a.batch : 1;
     g.rows_per_seq = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
     g.tiles_per_seq = (g.rows_per_seq + atc::ROWS - 1) / atc::ROWS;
-    const int tiles_k = (a.N + atc::KEYS - 1) / atc::KEYS;
-    g.kt = tiles_k > atc::MAX_CL ? 2 : 1;
-    g.cl = (tiles_k + g.kt - 1) / g.kt;
+    attention_tc_split(a.N, &g.kt, &g.cl);
     g.vec = stored_rows_in_pieces(a, 4) ? 1 : 0;
     g.status = status;
     const int dq = a.n_heads * a.head_dim, dkv = a.n_kv * a.head_dim;
@@ -397,15 +405,28 @@ static int launch_attention_tc(MapCache& maps, const AttnArgs& a, cudaStream_t s
 static bool attention_stream_applies(const AttnArgs& a) {
     return a.head_dim == ast::DH && a.N > 0 && (a.n_heads * a.head_dim) % 64 == 0 && (a.n_kv * a.head_dim) % 64 == 0;
 }
-// Which of the two tensor-core kernels: the streaming one as soon as its grid (row tiles x heads x sequences) fills a
-// good part of the GPU -- block entries, batches, long sequences (measured: 512 x 512 keys 28 us against 80 us,
-// 2048 x 2048 keys 0.29 ms against 1.4 ms) -- or the keys exceed what a cluster of key ranges covers; the cluster
-// kernel for the small steps of one short sequence, where spreading the keys over SMs wins (128 x 512: 20 us against 37 us).
-static bool attention_prefers_stream(const AttnArgs& a) {
+// Which of the two tensor-core kernels.  The streaming one as soon as its grid (row tiles x heads x sequences) fills a good
+// part of the GPU -- block entries, batches (with drift, us, cluster / streaming: 256 rows x 512 keys x 32 heads 40 / 25, 512 x
+// 512 x 32 77 / 27) -- or the keys exceed what a cluster of key ranges covers.  Below that the cluster kernel, which spreads
+// the keys of a (row tile, head) over SMs, while all its clusters are resident at once: 128 x 512 x 32 21 / 24, 96 x 512 x 32
+// 19 / 23, 128 x 1200 x 8 39 / 48, 128 x 2000 x 8 41 / 73.  With more clusters than that its time is waves x one wave (13.5 +
+// 0.055 a row us with drift, 12.5 + 0.033 without; two key tiles per CTA 16.5 + 0.18 and 16.5 + 0.02), the streaming kernel's is
+// proportional to the key tiles (10 + 4 each, 8 + 2 without drift): 128 x 512 x 36 39 / 26, 128 x 1024 x 32 62 / 41, without drift
+// 48 / 25, but 40 x 1024 x 16 31 / 39, 32 x 1300 x 32 43 / 48.  (Rows that the streaming kernel can not move in 16-byte pieces stay.)
+static bool attention_prefers_stream(const AttnArgs& a, const AttnClusters& resident) {
     const int batch = a.batch > 0 ? a.batch : 1;
     const int rps = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
-    const long long ctas = (long long)((rps + ast::ROWS - 1) / ast::ROWS) * batch * a.n_heads;
-    return ctas >= 64 || a.N > atc::MAX_N;
+    const long long tiles = (long long)((rps + ast::ROWS - 1) / ast::ROWS) * batch * a.n_heads;
+    if (tiles >= 64 || a.N > atc::MAX_N) return true;
+    int kt, cl;
+    attention_tc_split(a.N, &kt, &cl);
+    const long long at_once = std::max(resident.n[kt - 1][cl], 1);
+    if (tiles <= at_once) return false;
+    const bool drift = a.pprev || a.aprev;
+    if (drift && !stored_rows_in_pieces(a, 4)) return false;
+    const double rows = std::min(rps, ast::ROWS), key_tiles = (a.N + ast::KEYS - 1) / ast::KEYS;
+    const double wave = drift ? (kt == 1 ? 13.5 + 0.055 * rows : 16.5 + 0.18 * rows) : (kt == 1 ? 12.5 + 0.033 * rows : 16.5 + 0.02 * rows);
+    return (double)((tiles + at_once - 1) / at_once) * wave > (drift ? 10 + 4 * key_tiles : 8 + 2 * key_tiles);
 }
 static int launch_attention_stream(MapCache& maps, const AttnArgs& a, cudaStream_t st, int* status) {
     if (a.n_rows <= 0) return POLESTAR_OK;
@@ -540,6 +561,7 @@ struct polestar_ctx {
     int es;          // element size of the model dtype
     int device = 0;  // CUDA device the context was created on
     int sms = 148;
+    AttnClusters attn_clusters;
     Switches sw;
     int N, B, W_max, n_blocks, M_max, rows_lm;
     // controller
@@ -770,6 +792,20 @@ static int resident_gemm_pairs() {
     return n;
 }
 
+static int resident_attention_clusters(int kt, int cl) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(cl); cfg.blockDim = dim3(atc::THREADS);
+    cfg.dynamicSmemBytes = atc::smem_bytes(kt);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, atc::attention_tc_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n;
+}
+
 static cudaError_t set_kernel_attributes() {
     cudaError_t e;
     const int gemm_smem = 4 * (int)tc::STAGE_BYTES + 1024;    // four stages of 48 KB + alignment slack
@@ -829,16 +865,17 @@ struct Path {
             // different forms (scores + log-sum-exp / log-probabilities)
             // Launches that record or compare stored rows all go to the tensor-core kernel.  A launch that touches
             // no stored row (the layers below the last one of a step without refresh) may take either family: for a
-            // single block of rows the warp-level kernel's shorter dependency chain wins (11 us against 16 us per
+            // single block of rows the warp-level kernel's shorter dependency chain wins (10 us against 15 us per
             // layer at the 8B shape), everywhere else the tensor-core kernel does.
             const bool records = a.pprev != nullptr || a.aprev != nullptr;
             // Beyond 1024 keys the warp-level family has a 64-row kernel: it wins where (sequences x heads) fill the GPU (a
-            // batch of long sequences, 64 rows each: 85 us against 111 us for the streaming kernel, whose 128-row tiles are half empty).
+            // batch of long sequences, 64 rows each: 8 x 2048 keys x 32 heads 73 us against 88 us for the streaming kernel, whose
+            // 128-row tiles are half empty).
             const bool fills = (long long)(a.batch > 0 ? a.batch : 1) * a.n_heads >= c->sms;
             const bool few_rows = !records && a.rows_per_seq <= 64 && c->sw.attn_kernel == 0 &&
                                   (a.N <= 1024 || (a.rows_per_seq >= 48 && fills));
             if (attention_stream_applies(a) && !few_rows &&
-                (c->sw.attn_kernel == 9 || (c->sw.attn_kernel == 0 && attention_prefers_stream(a))))
+                (c->sw.attn_kernel == 9 || (c->sw.attn_kernel == 0 && attention_prefers_stream(a, c->attn_clusters))))
                 return launch_attention_stream(c->maps, a, c->st, c->b.status);
             if ((c->sw.attn_kernel == 0 || c->sw.attn_kernel == 8) && attention_tc_applies(a) && !few_rows)
                 return launch_attention_tc(c->maps, a, c->st, c->b.status);
@@ -1368,7 +1405,7 @@ extern "C" int polestar_init(polestar_ctx** out, const polestar_model* m, const 
         g_sw = c->sw; g_sw_loaded = true;
         g_use_pdl = c->sw.pdl != 0;
     }
-    c->sms = di.sm_count;
+    c->sms = di.sm_count; c->attn_clusters = di.attn;
     c->maps.l2promo = c->sw.l2promo;
     cudaGetDevice(&c->device);
     for (int l = 0; l < m->n_layers; ++l) {
@@ -1652,7 +1689,7 @@ extern "C" int polestar_k_attention(const void* q, const void* k, const void* v,
         if ((in & 15) || (o & 3)) return POLESTAR_E_INVAL;
         MapCache maps;                     // the tensor maps of this call
         maps.l2promo = sw.l2promo;
-        if (attention_stream_applies(a) && (sw.attn_kernel == 9 || (sw.attn_kernel == 0 && attention_prefers_stream(a))) && !(o & 15))
+        if (attention_stream_applies(a) && (sw.attn_kernel == 9 || (sw.attn_kernel == 0 && attention_prefers_stream(a, di.attn))) && !(o & 15))
             return launch_attention_stream(maps, a, st, nullptr);
         if ((sw.attn_kernel == 0 || sw.attn_kernel == 8) && attention_tc_applies(a) && !(o & 7))
             return launch_attention_tc(maps, a, st, nullptr);

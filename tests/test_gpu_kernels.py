@@ -43,6 +43,8 @@ def test_attention_drift_matches_oracle(dtype, R, N, nh, nkv, dh):
     (6, 32, 512, 4, 4), (6, 21, 300, 4, 2), (6, 5, 37, 2, 2),        # keys split over a cluster of two CTAs
     (7, 32, 1000, 2, 1), (7, 16, 512, 2, 2),
     (0, 32, 512, 2, 2),            # automatic choice for one block of rows
+    (0, 100, 640, 32, 4),          # ... where the cluster kernel's clusters are not all resident at once: streaming kernel,
+    (0, 40, 1028, 16, 16), (0, 20, 1021, 32, 32),       # cluster kernel in two waves (few rows; rows of no whole 16 bytes)
     # tensor-core kernel (tcgen05, S and O in tensor memory, key ranges over a cluster)
     (8, 128, 512, 2, 2),           # one full row tile, four key ranges
     (8, 32, 512, 4, 4),            # a block of active rows
