@@ -1364,8 +1364,11 @@ __global__ void build_head_list_kernel(StepDesc sd, const int* y, int mask_id, c
 // ---------------------------------------------------------------------------------------
 struct ConfPart { float mx_all; float sum; float mx_ex; int arg_ex; };
 
-__global__ void conf_partial_kernel(const float* logits, const int* m_count, int rows, int V, int mask_id,
-                                    int chunks, ConfPart* part) {
+// A block is a chain of a few microseconds (load, running maximum, three block reductions): what counts is how many are
+// resident.  Eight per SM with one 16-byte load in flight per thread (30 registers) against four loads in flight and four
+// blocks (63 registers), us: 32 rows x 126464 11 / 11, 64 x 50258 15 / 22, 512 x 126464 80 / 98, 512 x 2000 36 / 70.
+__global__ void __launch_bounds__(256, 8) conf_partial_kernel(const float* logits, const int* m_count, int rows, int V, int mask_id,
+                                                              int chunks, ConfPart* part) {
     KERNEL_PROLOGUE(11);   // conf_partial_kernel
     __shared__ float red[33];
     __shared__ float bv[32];
@@ -1381,33 +1384,18 @@ __global__ void conf_partial_kernel(const float* logits, const int* m_count, int
     int arg = 0x7fffffff;
     if ((V & 3) == 0) {
         const float4* l4 = reinterpret_cast<const float4*>(l);
-        // four loads in flight, one rescaling per sixteen values (entries past the chunk are -inf: exp 0, never the maximum)
-        const int e4 = v1 >> 2;
-        for (int b4 = (v0 >> 2) + threadIdx.x; b4 < e4; b4 += 4 * blockDim.x) {
-            float4 x[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int v4 = b4 + k * (int)blockDim.x;
-                x[k] = v4 < e4 ? __ldg(l4 + v4) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            }
-            float nm = mx;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) nm = fmaxf(nm, fmaxf(fmaxf(x[k].x, x[k].y), fmaxf(x[k].z, x[k].w)));
+        for (int v4 = (v0 >> 2) + threadIdx.x; v4 < (v1 >> 2); v4 += blockDim.x) {
+            const float4 x = __ldg(l4 + v4);
+            const float xs[4] = {x.x, x.y, x.z, x.w};
+            const float nm = fmaxf(mx, fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)));
             const float ref = nm == -INFINITY ? 0.f : nm;        // (only -inf so far: every term is exp(-inf))
-            float part4[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int v4 = b4 + k * (int)blockDim.x;
-                const float xs[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
-                part4[k] = v4 < e4 ? (expf(xs[0] - ref) + expf(xs[1] - ref)) + (expf(xs[2] - ref) + expf(xs[3] - ref)) : 0.f;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int v = 4 * v4 + u;
-                    if (v4 < e4 && v != mask_id && (xs[u] > mxe || (xs[u] == mxe && v < arg))) { mxe = xs[u]; arg = v; }
-                }
-            }
-            sum = sum * expf(mx - ref) + ((part4[0] + part4[1]) + (part4[2] + part4[3]));
+            sum = sum * expf(mx - ref) + ((expf(xs[0] - ref) + expf(xs[1] - ref)) + (expf(xs[2] - ref) + expf(xs[3] - ref)));
             mx = nm;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int v = 4 * v4 + u;
+                if (v != mask_id && (xs[u] > mxe || (xs[u] == mxe && v < arg))) { mxe = xs[u]; arg = v; }
+            }
         }
     } else {
         for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
