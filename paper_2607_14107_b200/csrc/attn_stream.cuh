@@ -310,9 +310,10 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         // j / 2 of bar_x(b, quarter): the quarter's 32 first threads arrive on it once the store of tile j - 2 has read X_b,
         // together with the bytes of the old rows of tile j when there are any: tile j + 1 is on its way while tile j is
         // worked on.  2048 rows x 2048 keys x 32 heads, rows read and written: one staging tile and row copies 434 us, two
-        // 381, boxes 293 (without any stored rows: 159); 256 x 2048: 102 / 94 / 74.  Rows whose length is not a multiple of four floats (no 16-byte alignment) go the plain way:
-        // every thread reads and writes its own row segment.
+        // 381, boxes 293 (without any stored rows: 159); 256 x 2048: 102 / 94 / 74.  Rows that no bulk copy takes
+        // (length or base no multiple of 16 bytes) go through the same tiles, a warp at a time (patch_load below).
         const bool use_x = vec && warp_prev;                     // (the same in the four warps of a quarter, like everything here)
+        const bool patch = !vec && warp_prev;
         const bool boxes = use_x && box_map_sh[quarter] >= 0;
         const CUtensorMap* const map_x = box_map_sh[quarter] == 1 ? &map_r : &map_p;
         auto x_quarter = [&](int b) { return x_s(b) + (uint32_t)quarter * XQ_BYTES; };
@@ -335,6 +336,21 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             }
         };
         if (use_x && cq == 0) { x_ready(0); if (n > 1) x_ready(1); }
+        // Each warp keeps its own [32 rows][32 keys] patch of the staging tiles, filled two tiles ahead by four-byte asynchronous
+        // copies and written back a row of the warp's 32 keys at a time: whole sectors, no waiting for other warps.  Every thread
+        // reading and writing its own row touched 32 lines per instruction (403 keys, 200 rows x 32 heads: 137 us, now 35; 2047 keys,
+        // 256 rows x 8 heads: 616, 114), and its 32 registers of old scores made the other forms spill.
+        auto patch_s = [&](int j, int r) { return x_quarter(j & 1) + (uint32_t)r * XPITCH + (uint32_t)cq * 128u + (uint32_t)lane * 4u; };
+        auto patch_load = [&](int j) {
+            const int k = j * KEYS + cq * 32 + lane;
+            if (a.record_kl && k < a.N)
+                for (int r = 0; r < 32; ++r) {
+                    const float* src = prev_sh[quarter * 32 + r];
+                    if (src) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(patch_s(j, r)), "l"(src + k) : "memory");
+                }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (patch) { patch_load(0); if (n > 1) patch_load(1); }
 
         // ---- pass 1: running (maximum, sum) of this thread's columns (four independent chains each: two or four warps
         // per scheduler cannot hide one long dependent chain) ----
@@ -413,11 +429,6 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             const int t = n + j, b = t & 1;
             const int kb = j * KEYS + cq * 32;
             const bool edge = kb + 32 > a.N;
-            float oldv[32];              // plain path: the lane's own row segment
-            if (!vec && use_old) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) oldv[i] = (kb + i < a.N) ? __ldcg(prev + kb + i) : 0.f;
-            }
             ok = mbar_wait(bar_sfull(b), (uint32_t)(t >> 1) & 1u, abort_flag) && ok && !*abort_flag;
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
@@ -465,6 +476,26 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_pfull);
             // ---- the tensor core has what it needs; now the stored row of this tile
+            // old scores out of the staging tile, drift sum, new scores into their place
+            auto new_rows = [&](uint32_t x) {
+                if (!warp_valid) return;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    float o0, o1, o2, o3;
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o0), "=f"(o1), "=f"(o2), "=f"(o3) : "r"(x + (((uint32_t)c ^ x_swz) << 4)) : "memory");
+                    float sn[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)       // (rounded products, never fused into the subtraction below: an unchanged row gives exactly zero)
+                        sn[i] = __fmul_rn(__fmul_rn(__uint_as_float(r[c >> 2][4 * (c & 3) + i]), scale2), LN2_F);
+                    if (use_old) {
+                        const float od[4] = {o0, o1, o2, o3};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (pr[4 * c + i] > 0.f) A4[i] = fmaf(pr[4 * c + i], sn[i] - od[i], A4[i]);      // (p = 0: also the masked entries)
+                    }
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(x + (((uint32_t)c ^ x_swz) << 4)), "f"(sn[0]), "f"(sn[1]), "f"(sn[2]), "f"(sn[3]) : "memory");
+                }
+            };
             if (use_x) {
                 const int xb = j & 1;
                 if (cq == 0 && j > 0) {
@@ -476,25 +507,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                 ok = mbar_wait(bar_x(xb, quarter), (uint32_t)(j >> 1) & 1u, abort_flag) && ok && !*abort_flag;
                 ok = __all_sync(0xffffffffu, ok) != 0;
                 if (!ok) break;
-                const uint32_t x = x_quarter(xb) + x_seg;
-                if (warp_valid) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float o0, o1, o2, o3;
-                        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o0), "=f"(o1), "=f"(o2), "=f"(o3) : "r"(x + (((uint32_t)c ^ x_swz) << 4)) : "memory");
-                        float sn[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)       // (rounded products, never fused into the subtraction below: an unchanged row gives exactly zero)
-                            sn[i] = __fmul_rn(__fmul_rn(__uint_as_float(r[c >> 2][4 * (c & 3) + i]), scale2), LN2_F);
-                        if (use_old) {
-                            const float od[4] = {o0, o1, o2, o3};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                if (pr[4 * c + i] > 0.f) A4[i] = fmaf(pr[4 * c + i], sn[i] - od[i], A4[i]);      // (p = 0: also the masked entries)
-                        }
-                        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(x + (((uint32_t)c ^ x_swz) << 4)), "f"(sn[0]), "f"(sn[1]), "f"(sn[2]), "f"(sn[3]) : "memory");
-                    }
-                }
+                new_rows(x_quarter(xb) + x_seg);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the bulk store reads what was just written
                 // the quarter's rows are complete once its four warps have passed here (an mbarrier, not a named barrier:
                 // its wait is bounded like every other)
@@ -516,16 +529,26 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                 }
-            } else if (warp_valid && prev && valid) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const float sn = __fmul_rn(__fmul_rn(__uint_as_float(r[i >> 4][i & 15]), scale2), LN2_F);
-                    if (use_old && pr[i] > 0.f) A4[i & 3] = fmaf(pr[i], sn - oldv[i], A4[i & 3]);
-                    if (kb + i < a.N) __stcg(prev + kb + i, sn);
-                }
+            } else if (patch) {
+                if (j + 1 < n) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncwarp();                    // the patch has landed for every lane
+                new_rows(x_quarter(j & 1) + x_seg);
+                __syncwarp();                    // ... and holds the new rows: out, a row of the warp's keys at a time
+                const int k = kb + lane;
+                if (k < a.N)
+                    for (int rr = 0; rr < 32; ++rr) {
+                        float* dst = prev_sh[quarter * 32 + rr];
+                        float v;
+                        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(patch_s(j, rr)) : "memory");
+                        if (dst) __stcg(dst + k, v);
+                    }
+                __syncwarp();
+                if (j + 2 < n) patch_load(j + 2);
             }
         }
         if (use_x && cq == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // the last stores have left
+        if (patch) asm volatile("cp.async.wait_all;" ::: "memory");         // (a wait that gave up left copies in flight)
 
         // ---- output rows and drift ----
         const float A = (A4[0] + A4[1]) + (A4[2] + A4[3]);
