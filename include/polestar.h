@@ -313,7 +313,9 @@ int polestar_reload_env(void);
  *   row_prev_dev float [R][n_heads][N], lse_prev_dev float [R][n_heads], both in/out (both NULL: no KL,
  *   nothing stored)
  *   kl_dev float [R][n_heads] (NULL allowed iff row_prev_dev NULL), out_dev [R][n_heads*head_dim]
- *   model dtype (NULL: skipped). */
+ *   model dtype (NULL: skipped).
+ * bf16 with head_dim 128: q, k and v 16-byte, out 4-byte aligned (E_INVAL otherwise; fastest with out and row_prev
+ * 16-byte aligned and N % 4 == 0). */
 int polestar_k_attention(const void *q_dev, const void *k_dev, const void *v_dev,
                          float *row_prev_dev, float *lse_prev_dev, float *kl_dev, void *out_dev,
                          int32_t R, int32_t N, int32_t n_heads, int32_t n_kv_heads,
