@@ -310,7 +310,7 @@ attention_stream_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_
         // j / 2 of bar_x(b, quarter): the quarter's 32 first threads arrive on it once the store of tile j - 2 has read X_b,
         // together with the bytes of the old rows of tile j when there are any: tile j + 1 is on its way while tile j is
         // worked on.  2048 rows x 2048 keys x 32 heads, rows read and written: one staging tile and row copies 434 us, two
-        // 381, boxes 293 (without any stored rows: 159); 256 x 2048: 102 / 94 / 74.  Rows that no bulk copy takes
+        // 381, boxes 293, now 281 (without any stored rows: 157); 256 x 2048: 102 / 94 / 74.  Rows that no bulk copy takes
         // (length or base no multiple of 16 bytes) go through the same tiles, a warp at a time (patch_load below).
         const bool use_x = vec && warp_prev;                     // (the same in the four warps of a quarter, like everything here)
         const bool patch = !vec && warp_prev;

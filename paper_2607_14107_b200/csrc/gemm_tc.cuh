@@ -316,14 +316,15 @@ __device__ __forceinline__ void red_add_v4(float* dst, uint32_t a, uint32_t b, u
                  "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
 }
 
-// CG = 2 (launched as clusters of two CTAs; every projection of more than 128 rows): a CTA pair works on a tile of 256
+// CG = 2 (launched as clusters of two CTAs; more than 128 rows, but see single_tiles_win): a CTA pair works on a tile of 256
 // tokens x 256 features.  Each CTA loads its 128 tokens and HALF of the weight tile (128 features), the even CTA issues one
 // MMA for both tensor cores (tcgen05.mma.cta_group::2, M = 256), and each CTA ends up with its 128 tokens x 256 features in
 // its own tensor memory: 32 KB of operands per CTA and k block instead of 48, so six stages fit, and the two accumulators
 // keep the epilogue overlapped with the next segment's MMAs.  Bound by the tensor pipe, at full load by the power limit
 // (8192 x 24576 x 4096: 133 cycles per MMA without loads; with them 1.3 - 1.5 PFLOP/s at 1.4 - 1.5 GHz).  Measured against
-// two 128-row MMAs per k step on one CTA (256-token tile, no epilogue overlap; removed) and against 128-token tiles,
-// K = 4096: 256 x 12288 47 / 60 / 64 us, 512 x 24576 101 / 130 / 110 us, 896 x 24576 158 / 207 / 161 us.  The schedule
+// two 128-row MMAs per k step on one CTA (256-token tile, no epilogue overlap; removed) and against 128-token tiles (gather and
+// projection),
+// K = 4096: 256 x 12288 33 / 38 / 47 us, 896 x 24576 129 / 146 / 134 us, 4096 x 24576 450 / 573 / 547 us.  The schedule
 // treats the pair as one CTA (stream-K ranges, whole tiles first); the epilogue and the partial tiles are per CTA on its own
 // 128 rows, the reduction pass deals the live rows of the whole tile over the CTAs of all contributing pairs.
 template <typename T, int EPI, int CG = 1>
