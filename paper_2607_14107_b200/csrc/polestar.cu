@@ -1798,11 +1798,18 @@ extern "C" int polestar_k_refresh(const void* h, const int32_t* idx, const int32
     const int half = head_dim / 2;
     // Two launches with programmatic stream serialization (the projection starts while the gather drains).  The gather
     // kernel also clears the counters and the status word (read back by polestar_k_refresh_status) and writes the rotary
-    // entries of the selected positions; only a refresh of (nearly) every position fills the whole table instead.
-    const bool table = M >= P;
-    if (table) CK(launch_k(rope_table_kernel, dim3((P * half + 255) / 256), dim3(256), 0, st, rope, P, half, (double)rope_theta));
-    CK(launch_k(prep_refresh_kernel<__nv_bfloat16>, dim3(M), dim3(256), 0, st, (const __nv_bfloat16*)h, idx, counts, max_rows, P, norm,
-                rms_eps, d, a_buf, table ? (float2*)nullptr : rope, half, (double)rope_theta, ws.counters, n_cnt, ws.status));
+    // entries of the selected positions, or the whole table where (nearly) every position is refreshed.  Its rotary blocks
+    // have at most one SM's worth of threads each, a few positions per thread.
+    const bool rope_all = M >= P;
+    const int side = std::max(1, REFRESH_THREADS / std::max(half, 1));           // positions a block works on side by side
+    const int rope_blocks = std::min(((rope_all ? P : M) + side - 1) / side, 2 * di.sm_count);
+    const bool by_warp = M >= REFRESH_WARP_ROWS && d <= 8 * 32 * REFRESH_VPT;
+    const int vec = d % 8 == 0 && (((uintptr_t)h | (uintptr_t)norm) & 15) == 0 && d <= 8 * (by_warp ? 32 : REFRESH_THREADS) * REFRESH_VPT;
+    const int rows_per_block = by_warp ? REFRESH_THREADS / 32 : 1;
+    const dim3 grid(rope_blocks + (M + rows_per_block - 1) / rows_per_block);
+    auto kern = by_warp ? prep_refresh_kernel<32> : prep_refresh_kernel<REFRESH_THREADS>;
+    CK(launch_k(kern, grid, dim3(REFRESH_THREADS), 0, st, (const __nv_bfloat16*)h, idx, counts, batch, max_rows, P, norm, rms_eps, d, vec,
+                a_buf, rope, rope_blocks, rope_all ? 1 : 0, half, (double)rope_theta, ws.counters, n_cnt, ws.status));
     CK(cudaGetLastError());
     EpiArgs e;
     memset(&e, 0, sizeof(e));

@@ -255,6 +255,14 @@ def test_refresh_chain_few_k_blocks_in_the_split_tiles(monkeypatch, pair_rows, k
     check_refresh_chain(k, 128, 2, 1, k, 4)
 
 
+@pytest.mark.parametrize("k,P,d,shift", [(1023, 1100, 256, 0), (1024, 1100, 256, 0), (1031, 1031, 4160, 0), (37, 64, 8256, 0),
+                                         (37, 64, 256, 2), (1031, 1100, 256, 2)])
+def test_refresh_row_staging_forms(k, P, d, shift):
+    # a block per row, a warp per row (a last block that is not full, rows longer than a warp holds), gains at a four-byte
+    # boundary; the rotary entries of the selected positions and of all of them
+    check_refresh_chain(P, d, 2, 2, k, 1, norm_shift=shift)
+
+
 def test_refresh_of_more_tiles_than_any_counter_array():
     # 589 824 rows x 4096 columns: 36 864 pair tiles.  Only the split tiles of a projection are counted, so its size has no
     # limit; one sequence of the batch on its own (4096 tiles) gives the same rows (fp32 sums in another order: one bf16 step)
@@ -282,7 +290,7 @@ def test_refresh_of_more_tiles_than_any_counter_array():
             assert b.abs().max() > 1
 
 
-def check_refresh_chain(P, d, nh, nkv, k, batch):
+def check_refresh_chain(P, d, nh, nkv, k, batch, norm_shift=0):
     dh = 128
     big = d >= 2048
     dev = "cuda" if big else "cpu"                      # large inputs are generated on the device (same values)
@@ -302,7 +310,7 @@ def check_refresh_chain(P, d, nh, nkv, k, batch):
     q_out = torch.zeros((batch, k, nh * dh), dtype=torch.bfloat16, device="cuda")
     scratch = torch.empty(Bd.polestar_k_refresh_scratch_bytes(batch, k, d, nh, nkv, dh) + 1024, dtype=torch.uint8, device="cuda")
     off = (-scratch.data_ptr()) % 1024
-    Bd.polestar_k_refresh(h.cuda(), idx, cnt, packed["wqkv"][0], packed["norm1"][0], kc, vc, q_out, k, nh, nkv, dh,
+    Bd.polestar_k_refresh(h.cuda(), idx, cnt, packed["wqkv"][0], shifted(packed["norm1"][0], norm_shift), kc, vc, q_out, k, nh, nkv, dh,
                           m.rms_eps, m.rope_theta, scratch[off:])
     assert Bd.polestar_k_refresh_status(scratch[off:], batch, k, d, dh) == Bd.OK      # synchronises
     assert cnt.cpu().tolist() == [k] * batch
