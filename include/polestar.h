@@ -373,23 +373,17 @@ int polestar_k_nvfp4_residual(const float *x_dev, const float *ref_dev, int32_t 
 
 /* Confidence of logits rows (Eq. 1; Sec. 2 sampler set): per row, y_hat = argmax over v != mask_id
  * (lowest id on ties), conf = softmax(logits)[y_hat].  logits_dev float [rows][vocab], 16-byte aligned
- * when vocab % 4 == 0 (E_INVAL otherwise); scratch_dev: >= rows * 512 bytes of device memory. */
+ * when vocab % 4 == 0 (E_INVAL otherwise); scratch_dev: >= rows * 512 bytes of device memory (checked, not used). */
 int polestar_k_confidence(const float *logits_dev, int32_t rows, int32_t vocab, int32_t mask_id,
                           int32_t *yhat_dev, float *conf_dev, void *scratch_dev, size_t scratch_bytes,
                           void *cuda_stream);
 
 /* Same result as polestar_k_confidence for callers that cannot provide or allocate device scratch
  * (a server whose memory pool owns every byte of the GPU, a loop that must not hit cudaMalloc's
- * device-wide synchronisation, a plug-in interface that passes inputs and outputs only).  The
- * partial results live in a 512 KB array that is part of the library image on every GPU using it.
+ * device-wide synchronisation, a plug-in interface that passes inputs and outputs only).
  * The paper has no counterpart: this is a packaging variant of the confidence kernel.
  *   - rows <= POLESTAR_NOALLOC_MAX_ROWS, otherwise POLESTAR_E_NOSPACE (use polestar_k_confidence).
- *   - Calls no allocation routine.  The first call on each device looks up the array's device
- *     address (cudaGetSymbolAddress, with the caller's current device); make that first call
- *     outside any stream capture.
- *   - All calls on a device share the one array: calls that may overlap on the GPU (different
- *     streams without ordering) race on it and must be serialised by the caller.  Nothing in the
- *     array has to be cleared between calls; it simply keeps the last call's partial results. */
+ *   - Calls no allocation routine and keeps nothing between calls: calls on different streams are independent. */
 #define POLESTAR_NOALLOC_MAX_ROWS 1024
 int polestar_k_confidence_noalloc(const float *logits_dev, int32_t rows, int32_t vocab, int32_t mask_id,
                                   int32_t *yhat_dev, float *conf_dev, void *cuda_stream);

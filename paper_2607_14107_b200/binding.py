@@ -458,8 +458,7 @@ NOALLOC_MAX_ROWS = 1024
 
 
 def polestar_k_confidence_noalloc(logits, mask_id, yhat, conf):
-    """Confidence of logits rows using the library's built-in scratch (no allocation, rows <= 1024).
-    For callers that cannot hand over scratch memory; concurrent calls on one device must be serialised."""
+    """Confidence of logits rows without any scratch memory (rows <= 1024)."""
     rows, V = logits.shape
     _check(load().polestar_k_confidence_noalloc(_ptr(logits), rows, V, mask_id, _ptr(yhat), _ptr(conf),
                                                 C.c_void_p(_stream())))

@@ -367,6 +367,21 @@ static int norm_threads(int rows, int d) {
     return (rows >= 256 && d <= 4 * NORM_VPT * 128) ? 128 : NORM_THREADS;
 }
 
+// Confidence of `rows` logits rows (of *m_count of them, when given).
+static cudaError_t launch_confidence(const float* logits, const int* m_count, int rows, int vocab, int mask_id, int* yhat, float* conf,
+                                     cudaStream_t st, int sms) {
+    // Threads per row: at least a batch of loads each, as long as all rows together do not exceed what the GPU holds at once
+    // (1776 threads per SM); in CTAs of 128 to 512, up to eight of them.  us at 4096 / 2048 / 1024 / 512 threads per row: 32 x 126464
+    // 7.4 / 9.9 / 13.7 / 19, 512 x 126464 100 / 63 / 57 / 53, 64 x 50258 9.1 / 7.3 / 8.8 / 12; 512 x 2000 128 4.4, 512 7.1.
+    const long long most = std::min<long long>(vocab / 16, 1776LL * sms / rows);
+    int per_row = 128;
+    while (per_row < CONF_CL * CONF_MAX_THREADS && 2 * per_row <= most) per_row *= 2;
+    const int cl = std::min(CONF_CL, std::max(1, per_row / 256)), threads = per_row / cl;
+    const dim3 grid((unsigned)rows * cl);
+    if (cl > 1) return launch_k_cluster(confidence_kernel, grid, dim3(threads), 0, st, (unsigned)cl, logits, m_count, vocab, mask_id, cl, yhat, conf);
+    return launch_k(confidence_kernel, grid, dim3(threads), 0, st, logits, m_count, vocab, mask_id, cl, yhat, conf);
+}
+
 // Attention + drift on tensor cores (attn_tc.cuh): bf16, head_dim 128, at most atc::MAX_N keys.
 static bool attention_tc_applies(const AttnArgs& a) {
     return a.head_dim == atc::DH && a.N <= atc::MAX_N && a.N > 0 && (a.n_heads * a.head_dim) % 64 == 0 &&
@@ -482,11 +497,10 @@ struct Buffers {
     unsigned char* fmask; unsigned char* fq; unsigned char* fs;                                                  // imposed codes (checking only)
     // scratch
     Row* rows; unsigned char* kvflag; float* x; float* x1; float* packet; char* a_buf; char* q_buf; char* o_buf;
-    char* g_buf; float* kl; int* list; long long* fold_ss; HeadSrc* head_list; char* a_head; float* logits; ConfPart* conf_part;
+    char* g_buf; float* kl; int* list; long long* fold_ss; HeadSrc* head_list; char* a_head; float* logits;
     float* gemm_partial; int* gemm_counters;
 };
 
-static const int CONF_CHUNKS = 32;
 static const int FORCED_COMMIT_MAX = 512;
 // partial tiles, two slots of 128 x 256 fp32 per CTA (38.8 MB at 148 SMs; a device with more than 160 gets a smaller grid), and
 // behind them the time stamps of POLESTAR_TRACE builds
@@ -736,7 +750,6 @@ static size_t make_plan(const polestar_model* m, const polestar_params* p, Buffe
     TAKE(head_list, HeadSrc, rows_lm);
     TAKE(a_head, char, rows_lm * d * es);
     TAKE(logits, float, rows_lm * V);
-    TAKE(conf_part, ConfPart, rows_lm * CONF_CHUNKS);
     TAKE(gemm_partial, float, GEMM_PARTIAL_BYTES / 4);
     TAKE(gemm_counters, int, GEMM_COUNTERS);
 #undef TAKE
@@ -1202,10 +1215,8 @@ struct Path {
             if ((rc = gemm<EPI_LOGITS>(c, b.a_head, c->lm_head, Mh, m.vocab, d, e))) return rc;
         }
         {
-            Scope sc(c, POLESTAR_PROF_CONFIDENCE, (double)bs * B * m.vocab * 4, 0, 3);
-            CK(launch_k(conf_partial_kernel, dim3(CONF_CHUNKS, Mh), dim3(256), 0, st, b.logits, b.head_count, Mh, m.vocab, m.mask_id,
-                                                                      CONF_CHUNKS, b.conf_part));
-            CK(launch_k(conf_final_kernel, dim3((Mh + 3) / 4), dim3(CONF_FINAL_THREADS), 0, st, b.conf_part, b.head_count, Mh, CONF_CHUNKS, b.yhat, b.conf));
+            Scope sc(c, POLESTAR_PROF_CONFIDENCE, (double)bs * B * m.vocab * 4, 0, 2);
+            CK(launch_confidence(b.logits, b.head_count, Mh, m.vocab, m.mask_id, b.yhat, b.conf, st, c->sms));
             CK(launch_k(delta_kernel, dim3(bs), dim3(256), 0, st, sd, b.kl, act_off, m.n_heads, b.delta));
             CK(cudaGetLastError());
         }
@@ -1859,63 +1870,33 @@ static bool conf_logits_aligned(const float* logits, int vocab) {
     return (((uintptr_t)logits) & ((vocab & 3) == 0 ? 15 : 3)) == 0;
 }
 
-static int launch_confidence(const float* logits, int rows, int vocab, int mask_id, int* yhat, float* conf, ConfPart* part, cudaStream_t st) {
-    CK(launch_k(conf_partial_kernel, dim3(CONF_CHUNKS, rows), dim3(256), 0, st, logits, (const int*)nullptr, rows, vocab, mask_id, CONF_CHUNKS, part));
-    CK(launch_k(conf_final_kernel, dim3((rows + 3) / 4), dim3(CONF_FINAL_THREADS), 0, st, (const ConfPart*)part, (const int*)nullptr, rows, CONF_CHUNKS, yhat, conf));
-    return POLESTAR_OK;
-}
-
 extern "C" int polestar_k_confidence(const float* logits, int32_t rows, int32_t vocab, int32_t mask_id, int32_t* yhat,
                                      float* conf, void* scratch, size_t scratch_bytes, void* stream) {
     if (rows < 0 || vocab <= 0) return POLESTAR_E_INVAL;
     if (rows == 0) return POLESTAR_OK;           // no rows: nothing to do (the pointers may be null)
     if (!logits || !yhat || !conf || !scratch) return POLESTAR_E_INVAL;
     if (!conf_logits_aligned(logits, vocab)) return POLESTAR_E_INVAL;
-    if (scratch_bytes < (size_t)rows * CONF_CHUNKS * sizeof(ConfPart)) return POLESTAR_E_NOSPACE;
-    cudaStream_t st = (cudaStream_t)stream;
-    return launch_confidence(logits, rows, vocab, mask_id, yhat, conf, (ConfPart*)scratch, st);
+    if (scratch_bytes < (size_t)rows * 512) return POLESTAR_E_NOSPACE;      // (the interface's size; the kernel needs none of it)
+    DevInfo di;
+    int rc = device_info(&di);
+    if (rc) return rc;
+    CK(launch_confidence(logits, nullptr, rows, vocab, mask_id, yhat, conf, (cudaStream_t)stream, di.sm_count));
+    return POLESTAR_OK;
 }
 
-// ------------------------------------------------------------------------------------------
-// Confidence without any caller-provided or allocated scratch
-// ------------------------------------------------------------------------------------------
-// Some callers have no way to obtain device scratch at call time: a serving process that handed
-// its whole memory budget to a KV-cache pool at start-up, a latency-critical loop in which
-// cudaMalloc's implicit device synchronisation is not acceptable, or a plug-in that is only
-// given input and output buffers.  For them the per-chunk partial results of the confidence
-// kernel live in a fixed array inside the library image (every GPU that loads the library
-// carries these 512 KB until the process exits).
-static __device__ __align__(256) ConfPart g_conf_scratch[POLESTAR_NOALLOC_MAX_ROWS * CONF_CHUNKS];
-
-// On the host, `g_conf_scratch` is only a handle of the symbol, not a device address: the real
-// address differs per device and has to be looked up once per device with that device current.
-static ConfPart* conf_scratch_ptr(int* err) {
-    static ConfPart* ptrs[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || dev < 0 || dev >= 64) { last_cuda_error = e; *err = POLESTAR_E_CUDA; return nullptr; }
-    if (!ptrs[dev]) {
-        void* p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_conf_scratch);
-        if (e != cudaSuccess || !p) { last_cuda_error = e; *err = POLESTAR_E_CUDA; return nullptr; }
-        ptrs[dev] = (ConfPart*)p;
-    }
-    *err = POLESTAR_OK;
-    return ptrs[dev];
-}
-
+// The same for callers that have no way to obtain device scratch at call time: a serving process that handed its whole memory
+// budget to a KV-cache pool at start-up, a latency-critical loop in which cudaMalloc's implicit device synchronisation is not
+// acceptable, or a plug-in that is only given input and output buffers.
 extern "C" int polestar_k_confidence_noalloc(const float* logits, int32_t rows, int32_t vocab, int32_t mask_id,
                                              int32_t* yhat, float* conf, void* stream) {
     if (rows < 0 || vocab <= 0) return POLESTAR_E_INVAL;
     if (rows == 0) return POLESTAR_OK;           // no rows: nothing to do (the pointers may be null)
     if (!logits || !yhat || !conf) return POLESTAR_E_INVAL;
     if (!conf_logits_aligned(logits, vocab)) return POLESTAR_E_INVAL;
-    if (rows > POLESTAR_NOALLOC_MAX_ROWS) return POLESTAR_E_NOSPACE;    // beyond the built-in scratch: use polestar_k_confidence
-    int err = POLESTAR_OK;
-    ConfPart* scratch = conf_scratch_ptr(&err);
-    if (!scratch) return err;
-    cudaStream_t st = (cudaStream_t)stream;
-    // every partial the second kernel reads is written by the first one in this call, so nothing of the
-    // previous call's contents has to be cleared
-    return launch_confidence(logits, rows, vocab, mask_id, yhat, conf, scratch, st);
+    if (rows > POLESTAR_NOALLOC_MAX_ROWS) return POLESTAR_E_NOSPACE;    // the interface's limit: use polestar_k_confidence
+    DevInfo di;
+    int rc = device_info(&di);
+    if (rc) return rc;
+    CK(launch_confidence(logits, nullptr, rows, vocab, mask_id, yhat, conf, (cudaStream_t)stream, di.sm_count));
+    return POLESTAR_OK;
 }

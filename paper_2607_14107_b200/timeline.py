@@ -18,7 +18,7 @@ import os
 import numpy as np
 
 NAMES = {1: "build_rows", 2: "embed", 3: "prep_qkv", 4: "prep_rows", 5: "prep_head", 6: "gather_rows", 7: "attention/select",
-         10: "head_list", 11: "conf_partial", 12: "conf_final", 13: "commit", 14: "delta", 15: "keep_hidden",
+         10: "head_list", 11: "confidence", 13: "commit", 14: "delta", 15: "keep_hidden",
          100: "gemm_qkv", 101: "gemm_o", 102: "gemm_gate_up", 103: "gemm_down", 104: "gemm_lm_head",
          200: "gemm_qkv:cta0_done", 201: "gemm_o:cta0_done", 202: "gemm_gate_up:cta0_done",
          203: "gemm_down:cta0_done", 204: "gemm_lm_head:cta0_done",

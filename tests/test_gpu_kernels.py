@@ -414,6 +414,28 @@ def test_confidence_edges(rows, V):
     assert torch.allclose(conf.cpu().double(), want, rtol=2e-5, atol=0)          # fp32 sums of V terms, exponentials to 2 ulp
 
 
+@pytest.mark.parametrize("rows,V", [(1, 2), (3, 7), (4, 4097), (5, 4099), (40, 16390), (600, 258), (1, 152065)])
+def test_confidence_rows_at_any_alignment(rows, V):
+    # rows that start at every offset from a 16-byte boundary, fewer elements than threads, each number of CTAs per row
+    logits = rnd((rows, V), 13, 3.0)
+    mask_id = V // 2
+    logits[0, 0] = logits[0, V - 1] = 30.0               # tie between the elements in front of and behind the 16-byte pieces
+    if rows > 2:
+        logits[1] = torch.finfo(torch.float32).min       # masked with the type's lowest value but for one entry, and throughout
+        logits[1, V - 2] = 1.0
+        logits[2] = torch.finfo(torch.float32).min
+    yhat = torch.zeros(rows, dtype=torch.int32, device="cuda")
+    conf = torch.zeros(rows, device="cuda")
+    Bd.polestar_k_confidence(logits.cuda(), mask_id, yhat, conf, torch.empty(rows * 512, dtype=torch.uint8, device="cuda"))
+    x = logits.double()
+    x[:, mask_id] = float("-inf")
+    best = x.max(dim=1).values
+    arg = (x == best[:, None]).int().argmax(dim=1)       # lowest id on ties
+    want = torch.softmax(logits.double(), dim=1)[torch.arange(rows), arg]
+    assert torch.equal(yhat.cpu().long(), arg)
+    assert torch.allclose(conf.cpu().double(), want, rtol=2e-5, atol=0)          # as above
+
+
 # ------------------------------------------------------------------ empty inputs
 def test_empty_inputs_are_noops():
     dev = "cuda"
