@@ -908,6 +908,7 @@ struct AttnArgs {
     float scale;
     int cluster_K;             // > 0: centroid proxies: pprev / pprev_lse hold [batch][cluster_K] proxy rows per head and
                                // window rows are not recorded
+    int rec_lo, rec_hi;        // rows [lo, hi) of every sequence hold all the recorded ones (hi 0: any row may be recorded)
     int dirty_lo, dirty_hi;    // key positions [lo, hi) of every sequence that the kernel running just before may have
                                // written; all other K/V rows were complete before this forward was launched
     // stand-alone form: rows == null, row r belongs to sequence 0 and records into pprev[r]

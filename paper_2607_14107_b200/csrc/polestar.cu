@@ -21,6 +21,7 @@
 #include "gemm_tc.cuh"
 #include "attn_tc.cuh"
 #include "attn_stream.cuh"
+#include "attn_flash.cuh"
 #include "gemm_chain.cuh"
 #include "kernels.cuh"
 
@@ -420,7 +421,74 @@ static int launch_attention_tc(MapCache& maps, const AttnArgs& a, cudaStream_t s
 static bool attention_stream_applies(const AttnArgs& a) {
     return a.head_dim == ast::DH && a.N > 0 && (a.n_heads * a.head_dim) % 64 == 0 && (a.n_kv * a.head_dim) % 64 == 0;
 }
-// Which of the two tensor-core kernels.  The streaming one as soon as its grid (row tiles x heads x sequences) fills a good
+// Stored rows as tensor boxes where their layout allows (16-byte row pitch; the kernels decide per 32 rows): bit 0: *mp describes
+// a.pprev, bit 1: *mr describes a.aprev (else untouched).
+static int stored_row_maps(MapCache& maps, const AttnArgs& a, int batch, const CUtensorMap** mp, const CUtensorMap** mr) {
+    if (!stored_rows_in_pieces(a, 4)) return 0;
+    int have = 0;
+    const uint64_t p_rows = a.rows ? (uint64_t)batch * (uint64_t)(a.cluster_K > 0 ? a.cluster_K : a.W_max) : (uint64_t)a.n_rows;
+    const CUtensorMap* m;
+    if (a.pprev && (m = maps.get_rows(a.pprev, p_rows, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) { *mp = m; have |= 1; }
+    if (a.rows && a.aprev && (m = maps.get_rows(a.aprev, (uint64_t)batch * a.B, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) { *mr = m; have |= 2; }
+    return have;
+}
+static int launch_attention_stream(MapCache& maps, const AttnArgs& a, cudaStream_t st, int* status) {
+    if (a.n_rows <= 0) return POLESTAR_OK;
+    ast::Args g;
+    memset(&g, 0, sizeof(g));
+    g.a = a;
+    const int batch = a.batch > 0 ? a.batch : 1;
+    g.rows_per_seq = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
+    g.tiles_per_seq = (g.rows_per_seq + ast::ROWS - 1) / ast::ROWS;
+    g.status = status;
+    const int dkv = a.n_kv * a.head_dim;
+    const int kv_batch = a.rows ? batch : 1;
+    const CUtensorMap* mk = maps.get3(a.kc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
+    const CUtensorMap* mv = maps.get3(a.vc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
+    if (!mk || !mv) return POLESTAR_E_CUDA;
+    const CUtensorMap *mp = mk, *mr = mk;
+    g.maps = stored_row_maps(maps, a, batch, &mp, &mr);
+    dim3 grid((unsigned)(g.tiles_per_seq * batch), (unsigned)a.n_heads);
+    CK(launch_k(ast::attention_stream_kernel, grid, dim3(ast::THREADS), ast::smem_bytes(), st, *mk, *mv, *mp, *mr, g));
+    return POLESTAR_OK;
+}
+
+// The two-stream form (attn_flash.cuh): any number of keys.
+static bool attention_flash_applies(const AttnArgs& a) { return attention_stream_applies(a); }
+struct FlashPlan { afl::FlashPart part[2]; int rec, stride, batch; long long waves_rec, steps_rec, waves, steps; };
+static FlashPlan flash_plan(const AttnArgs& a, int sms) {
+    FlashPlan p;
+    memset(&p, 0, sizeof(p));
+    p.batch = a.batch > 0 ? a.batch : 1;
+    p.stride = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
+    p.rec = a.pprev || a.aprev;
+    const int hpg = a.n_heads / a.n_kv;
+    const long long n = (a.N + afl::KEYS - 1) / afl::KEYS, per = (long long)p.batch * a.n_kv;
+    auto tiles_of = [&](int rows) { return (rows * hpg + afl::ROWS - 1) / afl::ROWS; };
+    // Recorded rows cost several times what the others do, so they get CTAs of their own where that makes fewer tiles with recorded
+    // rows (in the pipeline, us: block entry of 8 x 2048 rows, 192 of each sequence recorded, 1162 -> 991 a layer, 3 x 841 154 -> 133,
+    // refresh step of 8 x 192 rows, 128 recorded, 241 -> 222).
+    int lo = 0, hi = p.stride;
+    if (p.rec && a.rec_hi > a.rec_lo && tiles_of(a.rec_hi - a.rec_lo) < tiles_of(p.stride)) { lo = a.rec_lo; hi = a.rec_hi; }
+    const int n_rec = p.rec ? hi - lo : 0;
+    afl::FlashPart& r = p.part[0];
+    r.rows = n_rec; r.skip = lo; r.vrows = n_rec * hpg; r.key_split = 1; r.tiles = tiles_of(n_rec);
+    p.waves_rec = (r.tiles * per + sms - 1) / sms;
+    p.steps_rec = (n + 1) / 2;
+    afl::FlashPart& o = p.part[1];
+    o.rows = p.stride - n_rec; o.skip_at = n_rec ? lo : o.rows; o.skip = n_rec; o.vrows = o.rows * hpg;
+    // A row split takes the keys in n steps of two row tiles, a key split in n / 2 steps of one: whichever makes fewer steps per
+    // SM (2048 x 2048 x 32 heads 82 / 95 us, 512 x 512 x 32 18 / 11), at the same number the row split, which loads each K/V tile for
+    // both.  (A part with recorded rows has no room for two q tiles beside its patches.)
+    const int tiles = tiles_of(o.rows);
+    const long long row_waves = ((tiles + 1) / 2 * per + sms - 1) / sms, key_waves = (tiles * per + sms - 1) / sms;
+    o.key_split = (tiles == 1 || key_waves * ((n + 1) / 2) < row_waves * n) ? 1 : 0;
+    o.tiles = o.key_split ? tiles : (tiles + 1) / 2;
+    p.waves = o.key_split ? key_waves : row_waves;
+    p.steps = o.key_split ? (n + 1) / 2 : n;
+    return p;
+}
+// Which of the two kernels that normalise the probabilities before they round them.  The streaming one as soon as its grid (row tiles x heads x sequences) fills a good
 // part of the GPU -- block entries, batches (with drift, us, cluster / streaming: 256 rows x 512 keys x 32 heads 40 / 25, 512 x
 // 512 x 32 77 / 27) -- or the keys exceed what a cluster of key ranges covers.  Below that the cluster kernel, which spreads
 // the keys of a (row tile, head) over SMs, while all its clusters are resident at once: 128 x 512 x 32 21 / 24, 96 x 512 x 32
@@ -443,32 +511,57 @@ static bool attention_prefers_stream(const AttnArgs& a, const AttnClusters& resi
     const double wave = drift ? (kt == 1 ? 13.5 + 0.055 * rows : 16.5 + 0.18 * rows) : (kt == 1 ? 12.5 + 0.033 * rows : 16.5 + 0.02 * rows);
     return (double)((tiles + at_once - 1) / at_once) * wave > (drift ? 10 + 4 * key_tiles : 8 + 2 * key_tiles);
 }
-static int launch_attention_stream(MapCache& maps, const AttnArgs& a, cudaStream_t st, int* status) {
+// Which tensor-core kernel: the two-stream one, but for
+//  - forwards over up to 512 keys: they stay with the two kernels that round the NORMALISED probabilities to bf16, as a plain
+//    implementation does.  The two-stream kernel's roundings are as fine (relative error of the output rows against 64 bits, 128 x
+//    512 x 32 2.13e-3 / 2.35e-3, 300 x 2000 x 8 2.29e-3 / 2.35e-3, scores of spread 9 1.74e-3 / 2.11e-3) but fall elsewhere, and over the
+//    layers of an 8B-width model that difference takes the margin to a forward that rounds like a plain one: 6.8 % instead of
+//    3.5 % of the hidden values beyond 2e-2 after two layers at 160 keys.  At these sizes it would save 1 - 4 us a layer;
+//  - a single key tile, which leaves one of its streams idle: the streaming kernel (us, two-stream / streaming: 32 rows x 96 keys
+//    x 32 heads with stored rows 9.5 / 7.9, 28 heads on 4 11.4 / 8.3, without 12.2 / 7.0);
+//  - few (row tile, head) pairs with many keys, where the cluster kernel spreads the keys over SMs: by their estimated times, fitted
+//    to 32 / 32, 28 / 4, 8 / 8 and 4 / 1 heads, 1 - 900 rows, 96 - 2048 keys.  Two-stream: waves x (start + steps of two key tiles); cluster: waves of
+//    resident clusters x (start + its rows' share of the stored rows; `kt` key tiles per CTA).  us, two-stream / cluster with stored
+//    rows: 8 heads, 128 x 2000 49 / 35, 128 x 1200 32 / 34, 4 heads on 1, 64 x 2048 49 / 23, 28 on 4, 32 x 512 18 / 14, 128 x 1024 30 / 41,
+//    32 / 32 heads 128 x 512 18 / 19, 1 x 1501 (rows of no whole 16 bytes) 53 / 39, 64 x 1501 58 / 105.
+enum AttnForm { ATTN_FLASH, ATTN_STREAM, ATTN_CLUSTER };
+static AttnForm attention_form(const AttnArgs& a, const AttnClusters& resident, int sms) {
+    if (a.rows && a.N <= 512) return attention_prefers_stream(a, resident) ? ATTN_STREAM : ATTN_CLUSTER;
+    if (a.N <= ast::KEYS) return ATTN_STREAM;
+    if (!attention_tc_applies(a)) return ATTN_FLASH;
+    const FlashPlan f = flash_plan(a, sms);
+    int kt, cl;
+    attention_tc_split(a.N, &kt, &cl);
+    const long long at_once = std::max(resident.n[kt - 1][cl], 1);
+    const long long tiles = (long long)((f.stride + ast::ROWS - 1) / ast::ROWS) * f.batch * a.n_heads;
+    const double rows = std::min(f.stride, ast::ROWS);
+    const bool pieces = stored_rows_in_pieces(a, 4);
+    // (a step of two key tiles: boxes; warps whose rows span two heads; rows of no whole 16 bytes)
+    const double step = !pieces ? 9.0 : (f.stride % 32 && a.n_heads > a.n_kv ? 8.0 : 5.9);
+    const double flash = (double)f.waves_rec * (5.5 + step * (double)f.steps_rec) + (double)f.waves * (5.0 + 2.0 * (double)f.steps);
+    const double wave = !f.rec ? (kt == 1 ? 12.5 + 0.033 * rows : 16.5 + 0.02 * rows)
+                               : (kt == 1 ? 13.0 + (pieces ? 0.05 : 0.4) * rows : 17.5 + (pieces ? 0.15 : 0.55) * rows);
+    return (double)((tiles + at_once - 1) / at_once) * wave < flash ? ATTN_CLUSTER : ATTN_FLASH;
+}
+static int launch_attention_flash(MapCache& maps, const AttnArgs& a, cudaStream_t st, int* status, int sms) {
     if (a.n_rows <= 0) return POLESTAR_OK;
-    ast::Args g;
-    memset(&g, 0, sizeof(g));
-    g.a = a;
-    const int batch = a.batch > 0 ? a.batch : 1;
-    g.rows_per_seq = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
-    g.tiles_per_seq = (g.rows_per_seq + ast::ROWS - 1) / ast::ROWS;
-    g.status = status;
-    const int dkv = a.n_kv * a.head_dim;
-    const int kv_batch = a.rows ? batch : 1;
+    const FlashPlan fs = flash_plan(a, sms);
+    afl::FlashArgs f;
+    memset(&f, 0, sizeof(f));
+    f.a = a;
+    f.stride = fs.stride;
+    f.rec_ctas = fs.part[0].tiles * fs.batch;
+    f.part[0] = fs.part[0]; f.part[1] = fs.part[1];
+    f.status = status;
+    const int dkv = a.n_kv * a.head_dim, kv_batch = a.rows ? fs.batch : 1;
     const CUtensorMap* mk = maps.get3(a.kc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
     const CUtensorMap* mv = maps.get3(a.vc, (uint64_t)kv_batch, (uint64_t)a.N, (uint64_t)dkv);
     if (!mk || !mv) return POLESTAR_E_CUDA;
-    // stored rows as tensor boxes where their layout allows (16-byte row pitch); the kernel decides per 32 rows
     const CUtensorMap *mp = mk, *mr = mk;
-    g.maps = 0;
-    if (stored_rows_in_pieces(a, 4)) {
-        const uint64_t p_rows = a.rows ? (uint64_t)batch * (uint64_t)(a.cluster_K > 0 ? a.cluster_K : a.W_max) : (uint64_t)a.n_rows;
-        if (a.pprev && (mp = maps.get_rows(a.pprev, p_rows, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 1;
-        if (a.rows && a.aprev && (mr = maps.get_rows(a.aprev, (uint64_t)batch * a.B, (uint64_t)a.n_heads, (uint64_t)a.N)) != nullptr) g.maps |= 2;
-        if (!mp) mp = mk;
-        if (!mr) mr = mk;
-    }
-    dim3 grid((unsigned)(g.tiles_per_seq * batch), (unsigned)a.n_heads);
-    CK(launch_k(ast::attention_stream_kernel, grid, dim3(ast::THREADS), ast::smem_bytes(), st, *mk, *mv, *mp, *mr, g));
+    f.maps = stored_row_maps(maps, a, fs.batch, &mp, &mr);
+    const dim3 grid((unsigned)(f.rec_ctas + f.part[1].tiles * fs.batch), (unsigned)a.n_kv);
+    CK(launch_k(fs.rec ? afl::attention_flash_kernel<true> : afl::attention_flash_kernel<false>, grid, dim3(afl::FL_THREADS),
+                afl::flash_smem_bytes(fs.rec != 0), st, *mk, *mv, *mp, *mr, f));
     return POLESTAR_OK;
 }
 
@@ -844,6 +937,8 @@ static cudaError_t set_kernel_attributes() {
     PS_ATTR(gemm_f32_kernel<EPI_LOGITS>, LAT_SMEM);
     PS_ATTR(kmeans_kernel, KM_SMEM_BYTES);
     PS_ATTR(ast::attention_stream_kernel, (int)ast::smem_bytes());
+    PS_ATTR(afl::attention_flash_kernel<true>, (int)afl::flash_smem_bytes(true));
+    PS_ATTR(afl::attention_flash_kernel<false>, (int)afl::flash_smem_bytes(false));
     PS_ATTR(attention_simt_kernel<float>, (int)SIMT_ATTN_SMEM_MAX);
     PS_ATTR(attention_simt_kernel<__nv_bfloat16>, (int)SIMT_ATTN_SMEM_MAX);
 #undef PS_ATTR
@@ -874,26 +969,25 @@ struct Path {
 
     static int attention(polestar_ctx* c, const AttnArgs& a) {
         if (is_bf16 && c->m.head_dim == 128 && !c->sw.attn_simt) {
-            // one kernel family per context (decided by the shape alone): the families keep stored rows in
-            // different forms (scores + log-sum-exp / log-probabilities)
-            // Launches that record or compare stored rows all go to the tensor-core kernel.  A launch that touches
-            // no stored row (the layers below the last one of a step without refresh) may take either family: for a
-            // single block of rows the warp-level kernel's shorter dependency chain wins (10 us against 15 us per
-            // layer at the 8B shape), everywhere else the tensor-core kernel does.
+            // The families keep stored rows in different forms (scores + log-sum-exp / log-probabilities), so launches that
+            // record or compare stored rows all go to the tensor-core kernels.  A launch that touches none (the layers below
+            // the last one of a step without refresh) may take either family: for a single block of rows the warp-level
+            // kernel's shorter dependency chain wins while its (sequence, head) pairs fill less than half of the GPU and a cluster of
+            // two covers the keys.  In the pipeline, 32 rows, us, warp-level / two-stream: 32 heads x 512 keys 9.4 / 12.1, x 1024 13.5 / 16.1, two
+            // sequences 10.5 / 12.3, four 18.7 / 13.1; 28 heads on 4, 1024 keys, four sequences 39.9 / 21.3.
             const bool records = a.pprev != nullptr || a.aprev != nullptr;
-            // Beyond 1024 keys the warp-level family has a 64-row kernel: it wins where (sequences x heads) fill the GPU (a
-            // batch of long sequences, 64 rows each: 8 x 2048 keys x 32 heads 73 us against 88 us for the streaming kernel, whose
-            // 128-row tiles are half empty).
-            const bool fills = (long long)(a.batch > 0 ? a.batch : 1) * a.n_heads >= c->sms;
-            const bool few_rows = !records && a.rows_per_seq <= 64 && c->sw.attn_kernel == 0 &&
-                                  (a.N <= 1024 || (a.rows_per_seq >= 48 && fills));
-            if (attention_stream_applies(a) && !few_rows &&
-                (c->sw.attn_kernel == 9 || (c->sw.attn_kernel == 0 && attention_prefers_stream(a, c->attn_clusters))))
-                return launch_attention_stream(c->maps, a, c->st, c->b.status);
-            if ((c->sw.attn_kernel == 0 || c->sw.attn_kernel == 8) && attention_tc_applies(a) && !few_rows)
+            const long long pairs = (long long)(a.batch > 0 ? a.batch : 1) * a.n_heads;
+            const bool few_rows = !records && a.rows_per_seq <= 64 && c->sw.attn_kernel == 0 && a.N <= 1024 && 2 * pairs <= c->sms;
+            const int forced = c->sw.attn_kernel;
+            if (attention_flash_applies(a) && !few_rows && (forced == 0 || forced >= 9)) {
+                const AttnForm form = forced == 0 ? attention_form(a, c->attn_clusters, c->sms) : (forced == 9 ? ATTN_STREAM : ATTN_FLASH);
+                if (form == ATTN_FLASH) return launch_attention_flash(c->maps, a, c->st, c->b.status, c->sms);
+                if (form == ATTN_STREAM) return launch_attention_stream(c->maps, a, c->st, c->b.status);
+            }
+            if ((forced == 0 || forced == 8) && attention_tc_applies(a) && !few_rows)
                 return launch_attention_tc(c->maps, a, c->st, c->b.status);
             if (a.cluster_K > 0 && (a.pprev || a.aprev)) goto simt;      // the warp-level kernels do not know proxy rows
-            CK(launch_attention_mma(a, c->st, c->sms, c->sw.attn_kernel));
+            CK(launch_attention_mma(a, c->st, c->sms, forced));
             return POLESTAR_OK;
         }
     simt:
@@ -1022,6 +1116,15 @@ struct Path {
                 a.kl = b.kl; a.N = N; a.n_heads = m.n_heads; a.n_kv = m.n_kv_heads; a.head_dim = m.head_dim;
                 a.W_max = Wm; a.B = B; a.record_kl = sd.record_kl; a.rows_per_seq = sd.rows_per_seq; a.batch = bs;
                 a.scale = 1.0f / sqrtf((float)m.head_dim);
+                // rows that may be recorded: the window rows, among which an entry step has the active block, or the proxy rows;
+                // and in the last layer the active rows
+                if (within) { a.rec_lo = last ? 0 : B; a.rec_hi = B + sd.W; }
+                else { a.rec_lo = sd.pre_start - sd.e0; a.rec_hi = sd.suf_start + (sd.W - sd.n_pre) - sd.e0; }
+                a.rec_hi = std::min(a.rec_hi, sd.rows_per_seq);
+                if (a.cluster_K > 0) {
+                    if (!last) a.rec_lo = sd.rows_per_seq - sd.K;
+                    a.rec_hi = sd.rows_per_seq;
+                }
                 // positions whose K/V this layer's QKV projection writes: the forwarded rows of an entry step; the
                 // active block and, on refresh steps, the patched window rows of a within-block step
                 if (!within) { a.dirty_lo = sd.e0; a.dirty_hi = sd.e0 + sd.rows_per_seq; }
@@ -1700,9 +1803,13 @@ extern "C" int polestar_k_attention(const void* q, const void* k, const void* v,
         if ((in & 15) || (o & 3)) return POLESTAR_E_INVAL;
         MapCache maps;                     // the tensor maps of this call
         maps.l2promo = sw.l2promo;
-        if (attention_stream_applies(a) && (sw.attn_kernel == 9 || (sw.attn_kernel == 0 && attention_prefers_stream(a, di.attn))) && !(o & 15))
-            return launch_attention_stream(maps, a, st, nullptr);
-        if ((sw.attn_kernel == 0 || sw.attn_kernel == 8) && attention_tc_applies(a) && !(o & 7))
+        const int forced = sw.attn_kernel;
+        if (attention_flash_applies(a) && (forced == 0 || forced >= 9) && !(o & 15)) {
+            const AttnForm form = forced == 0 ? attention_form(a, di.attn, di.sm_count) : (forced == 9 ? ATTN_STREAM : ATTN_FLASH);
+            if (form == ATTN_FLASH) return launch_attention_flash(maps, a, st, nullptr, di.sm_count);
+            if (form == ATTN_STREAM) return launch_attention_stream(maps, a, st, nullptr);
+        }
+        if ((forced == 0 || forced == 8) && attention_tc_applies(a) && !(o & 7))
             return launch_attention_tc(maps, a, st, nullptr);
         CK(launch_attention_mma(a, st, di.sm_count, sw.attn_kernel));
         return POLESTAR_OK;

@@ -62,6 +62,12 @@ def test_attention_drift_matches_oracle(dtype, R, N, nh, nkv, dh):
     (9, 200, 2048, 8, 8),          # the long-sequence shape
     (9, 64, 402, 2, 1),            # key count not a multiple of four
     (9, 70, 3000, 2, 2),           # more keys than the cluster kernel takes
+    # two streams per CTA, one pass: the keys of a row tile split (few row tiles) ...
+    (10, 5, 37, 2, 2), (10, 1, 129, 2, 1),         # one key tile: the second stream has none; a tile of one key
+    (10, 128, 512, 2, 2), (10, 37, 200, 4, 2),     # ragged rows and keys; grouped heads in one row tile, 32-row groups across heads
+    (10, 150, 1100, 2, 1), (10, 64, 402, 4, 1), (10, 64, 512, 8, 1), (10, 70, 3000, 2, 2),
+    # ... and a row tile each (more row tiles than SMs): an odd and an even number of them, one and several key tiles
+    (10, 300, 300, 64, 64), (10, 129, 100, 100, 100), (10, 400, 402, 50, 25), (10, 256, 640, 80, 80),
 ])
 def test_attention_kernel_variants(monkeypatch, variant, R, N, nh, nkv):
     monkeypatch.setenv("POLESTAR_ATTN_KERNEL", str(variant))
@@ -72,6 +78,7 @@ def test_attention_kernel_variants(monkeypatch, variant, R, N, nh, nkv):
 @pytest.mark.parametrize("prev_off,out_off", [(1, 0), (2, 8), (3, 4), (0, 2)])      # in elements: 4 / 8 / 12 bytes, 16 / 8 / 4 bytes
 @pytest.mark.parametrize("variant,R,N,nh,nkv", [
     (9, 70, 404, 2, 1),            # streaming: several key tiles, a ragged second row tile
+    (10, 70, 404, 2, 1),           # two streams: the same (no boxes: pieces of 16 or 4 bytes)
     (8, 37, 500, 2, 1), (8, 20, 1028, 2, 2),       # one and two key tiles per CTA of the cluster kernel
     (0, 128, 512, 2, 2),
     (1, 20, 100, 2, 1), (2, 37, 200, 2, 1), (3, 37, 200, 2, 1), (5, 70, 300, 2, 1), (6, 21, 300, 2, 1),
@@ -153,7 +160,9 @@ def test_attention_without_recording():
 
 
 @pytest.mark.parametrize("variant,R,N,nh,nkv", [(5, 150, 1100, 2, 1), (5, 64, 2048, 4, 4), (5, 5, 37, 2, 2), (0, 300, 2048, 8, 2),
-                                                (9, 150, 1100, 2, 1), (9, 300, 2048, 8, 2), (9, 5, 37, 2, 2), (9, 130, 3000, 2, 2)])
+                                                (9, 150, 1100, 2, 1), (9, 300, 2048, 8, 2), (9, 5, 37, 2, 2), (9, 130, 3000, 2, 2),
+                                                # two streams: keys split; a row tile each (an odd and an even number of row tiles)
+                                                (10, 150, 1100, 2, 1), (10, 5, 37, 2, 2), (10, 257, 300, 80, 80), (10, 256, 520, 80, 80), (10, 60, 384, 160, 20)])
 def test_attention_many_rows_single_pass(monkeypatch, variant, R, N, nh, nkv):
     # without stored rows the 64-row-tile kernel makes one pass with a running maximum (probabilities are rounded
     # to bf16 before the final normalisation): same tolerance against the oracle; the streaming kernel (9) normalises
