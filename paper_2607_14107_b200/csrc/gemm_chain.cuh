@@ -174,11 +174,11 @@ gemm_chain_kernel(const __grid_constant__ ChainMaps maps, const __grid_constant_
         fx_ready = 1;
     }
     if (sf.on && cta == 0 && warp >= 6 && warp < 14) {
-        __shared__ float sel_dsh[SEL_SMALL_W];
-        __shared__ int sel_flags[SEL_SMALL_W];
+        __shared__ __align__(16) float sel_dsh[SEL_SMALL_W];
+        __shared__ int sel_cnts[8];
         __syncwarp();
         pdl_wait();
-        step_select_inline(sf.sd, sf.a, (int)threadIdx.x - THREADS, 256, 2, sel_dsh, sel_flags);
+        step_select_inline(sf.sd, sf.a, (int)threadIdx.x - THREADS, 256, 2, sel_dsh, sel_cnts);
     }
 
     // running counters of the roles (they continue across the projections of the chain)

@@ -431,11 +431,11 @@ gemm_sk_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
     if constexpr (EPI == EPI_RESID) {
         if (sf.on && blockIdx.x == 0 && warp >= 6 && warp < 14) {
-            __shared__ float sel_dsh[SEL_SMALL_W];
-            __shared__ int sel_flags[SEL_SMALL_W];
+            __shared__ __align__(16) float sel_dsh[SEL_SMALL_W];
+            __shared__ int sel_cnts[8];
             __syncwarp();
             pdl_wait();                                  // the per-head drift comes from the attention kernel
-            step_select_inline(sf.sd, sf.a, (int)threadIdx.x - THREADS, 256, 2, sel_dsh, sel_flags);
+            step_select_inline(sf.sd, sf.a, (int)threadIdx.x - THREADS, 256, 2, sel_dsh, sel_cnts);
         }
     }
 

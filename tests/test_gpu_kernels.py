@@ -195,7 +195,8 @@ def test_hidden_delta(dtype, rows, d):
 
 
 # ------------------------------------------------------------------ select + compaction (a2)
-@pytest.mark.parametrize("W,batch", [(96, 1), (64, 3), (192, 8), (4096, 2), (1, 1), (1000, 1)])
+@pytest.mark.parametrize("W,batch", [(96, 1), (64, 3), (192, 8), (4096, 2), (1, 1), (1000, 1),
+                                     (255, 2), (256, 1), (257, 3), (4093, 2), (31, 2)])       # either form's last size, rows off 16 bytes
 def test_select_matches_bruteforce(W, batch):
     g = torch.Generator().manual_seed(W * 31 + batch)
     z = torch.randn(batch, W, generator=g)
