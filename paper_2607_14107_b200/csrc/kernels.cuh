@@ -787,6 +787,8 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 // 64 x 64 tiles leave most SMs idle and every 16-wide K slice is a round trip to L2.  Here the operands of three
 // 64-wide K slices are in flight at once (cp.async ring; the weights' share of it before the dependency wait), each
 // warp multiplies eight k of a slice, and the eight partial tiles are added in warp order through shared memory.
+// Where the output tiles leave most SMs idle and K is long, the slices are split over a cluster of up to eight CTAs (gridDim.z), which
+// push their tiles into the first one's shared memory; it adds them in rank order.
 // Rows / columns beyond the matrix and k beyond K arrive as zeros.  Needs K % 4 == 0 and 16-byte aligned operands.
 // Measured against 64 x 64 tiles (rows x columns x K): 32 x 768 x 256 5.6 / 29 us, 32 x 256 x 1024 11 / 109 us,
 // 128 x 2048 x 256 11 / 31 us, 512 x 2048 x 256 29 / 37 us, 4096 x 4096 x 1024 1160 / 1522 us: faster at every size, so the
@@ -807,11 +809,13 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
     extern __shared__ __align__(16) float lat_sm[];
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int m0 = blockIdx.y * LAT_TM, n0 = blockIdx.x * LAT_TN;
-    const int slices = (K + LAT_KC - 1) / LAT_KC;
+    // this CTA's slices of K
+    const int slices_all = (K + LAT_KC - 1) / LAT_KC, cl = gridDim.z, rank = blockIdx.z;
+    const int s_begin = slices_all * rank / cl, slices = slices_all * (rank + 1) / cl - s_begin;
     // thread t copies 16 bytes of A (row t / 16, k chunk t % 16) and twice 16 bytes of W (rows t / 16 and t / 16 + 16)
     const int cr = t >> 4, ck = (t & 15) * 4;
     auto load_w = [&](int s) {
-        const int k = s * LAT_KC + ck;
+        const int k = (s_begin + s) * LAT_KC + ck;
         float* st = lat_sm + (s % LAT_STAGES) * STAGE + LAT_TM * LAT_LD;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -821,7 +825,7 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
         }
     };
     auto load_a = [&](int s) {
-        const int k = s * LAT_KC + ck;
+        const int k = (s_begin + s) * LAT_KC + ck;
         const bool ok = m0 + cr < M && k < K;
         cp_async16_zfill(lat_sm + (s % LAT_STAGES) * STAGE + cr * LAT_LD + ck, ok ? A + (size_t)(m0 + cr) * K + k : A, ok);
     };
@@ -830,7 +834,7 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
     pdl_wait();
     trace_stamp(7);
     const int Mv = e.m_count ? min(M, *e.m_count) : M;
-    if (m0 >= Mv) {
+    if (m0 >= Mv) {                             // (the whole cluster)
         asm volatile("cp.async.wait_all;" ::: "memory");
         return;
     }
@@ -871,6 +875,7 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    if (cl > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // this CTA's ring is free
     float* red = lat_sm + warp * (LAT_TM * LAT_TN);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -883,6 +888,19 @@ __global__ void __launch_bounds__(256) gemm_f32_kernel(const float* __restrict__
     for (int w = 0; w < 8; ++w) {
         const float2 v = *reinterpret_cast<const float2*>(lat_sm + w * (LAT_TM * LAT_TN) + t * 2);
         sum.x += v.x; sum.y += v.y;
+    }
+    if (cl > 1) {
+        // the other CTAs' tiles, behind the partial tiles in the first CTA's ring
+        static_assert((8 + 7) * LAT_TM * LAT_TN <= LAT_STAGES * STAGE, "and so do the cluster's tiles");
+        float2* const peer = reinterpret_cast<float2*>(lat_sm + 8 * LAT_TM * LAT_TN) + t;
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank > 0) {
+            const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(peer + (rank - 1) * 256), 0);
+            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(sum.x), "f"(sum.y) : "memory");
+        }
+        cluster_sync_all();
+        if (rank > 0) return;
+        for (int c = 1; c < cl; ++c) { const float2 v = peer[(c - 1) * 256]; sum.x += v.x; sum.y += v.y; }
     }
     if (m < Mv && n + 1 < Nout) epilogue_pair<float, EPI>(e, m, n, sum.x, sum.y);
 }
@@ -918,13 +936,18 @@ static inline bool stored_rows_in_pieces(const AttnArgs& a, int floats) {
     return a.N % floats == 0 && (((uintptr_t)a.pprev | (uintptr_t)a.aprev) & (uintptr_t)(4 * floats - 1)) == 0;
 }
 
+// One CTA of four warps per (row, head): a chain of dependent loads at the sizes of these models, so the keys are split over the
+// warps and everything a thread needs of K (16-byte pieces of its keys, sixteen in flight) and V (its columns of 32 keys) is
+// requested at once.  Parts are put together in warp order.  fp32, 4 heads of 64, 128 keys, in the pipeline, us,
+// against a warp per (row, head): 32 rows 14.4 -> 7.5, 128 rows with stored rows 19.6 - 33 -> 12.
+constexpr int SIMT_WARPS = 4;
+__host__ __device__ constexpr size_t simt_attn_smem(int N, int dh) { return ((size_t)N + SIMT_WARPS * dh + 2 * SIMT_WARPS) * sizeof(float); }
 template <typename T>
-__global__ void attention_simt_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(SIMT_WARPS * 32) attention_simt_kernel(AttnArgs a) {
     KERNEL_PROLOGUE(8);   // attention_simt_kernel
     extern __shared__ float sm[];
-    const int wpb = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = blockIdx.x * wpb + wid, h = blockIdx.y;
-    if (r >= a.n_rows) return;
+    const int t = threadIdx.x, wid = t >> 5, lane = t & 31;
+    const int r = blockIdx.x, h = blockIdx.y;
     int seq = 0;
     float* prev = nullptr;
     if (a.rows) {
@@ -940,31 +963,42 @@ __global__ void attention_simt_kernel(AttnArgs a) {
     } else if (a.pprev) {
         prev = a.pprev + ((size_t)r * a.n_heads + h) * a.N;
     }
-    float* sc = sm + (size_t)wid * a.N;
     const int dh = a.head_dim, g = (h * a.n_kv) / a.n_heads;
+    float* const sc = sm;                              // scores, then probabilities
+    float* const part = sm + a.N;                      // [warp][dh] partial output rows
+    float* const red = part + SIMT_WARPS * dh;         // [2][warp]
     const int dq = a.n_heads * dh, dkv = a.n_kv * dh;
     const T* q = (const T*)a.q + (size_t)r * dq + h * dh;
     const T* K = (const T*)a.kc + (size_t)seq * a.N * dkv + g * dh;
     const T* V = (const T*)a.vc + (size_t)seq * a.N * dkv + g * dh;
+    // one value of every warp, combined in warp order
+    auto combine = [&](float v, int slot, auto op) {
+        if (lane == 0) red[slot * SIMT_WARPS + wid] = v;
+        __syncthreads();
+        float x = red[slot * SIMT_WARPS];
+#pragma unroll
+        for (int w = 1; w < SIMT_WARPS; ++w) x = op(x, red[slot * SIMT_WARPS + w]);
+        return x;
+    };
     // scores
     float mx = -INFINITY;
-    // (one warp per row and head: a chain of dependent loads.  fp32 heads of 32-multiples are read in 16-byte pieces,
-    // eight in flight; the products are added in the same order)
     const bool vec = sizeof(T) == 4 && (dh & 31) == 0 && (dq & 3) == 0 && (dkv & 3) == 0 && (((uintptr_t)a.q | (uintptr_t)a.kc) & 15) == 0;
-    for (int j = lane; j < a.N; j += 32) {
+    for (int j = t; j < a.N; j += SIMT_WARPS * 32) {
         const T* kj = K + (size_t)j * dkv;
         float s = 0.f;
         if (vec) {
             const float4* k4 = reinterpret_cast<const float4*>(kj);
             const float4* q4 = reinterpret_cast<const float4*>(q);
-            for (int c = 0; c < (dh >> 2); c += 8) {
-                float4 kv[8], qv[8];
+            for (int c = 0; c < (dh >> 2); c += 16) {
+                float4 kv[16];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) { kv[i] = k4[c + i]; qv[i] = q4[c + i]; }
+                for (int i = 0; i < 16; ++i) if (c + i < (dh >> 2)) kv[i] = k4[c + i];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    s = fmaf(qv[i].x, kv[i].x, s); s = fmaf(qv[i].y, kv[i].y, s);
-                    s = fmaf(qv[i].z, kv[i].z, s); s = fmaf(qv[i].w, kv[i].w, s);
+                for (int i = 0; i < 16; ++i) {
+                    if (c + i >= (dh >> 2)) break;
+                    const float4 qv = q4[c + i];
+                    s = fmaf(qv.x, kv[i].x, s); s = fmaf(qv.y, kv[i].y, s);
+                    s = fmaf(qv.z, kv[i].z, s); s = fmaf(qv.w, kv[i].w, s);
                 }
             }
         } else {
@@ -974,13 +1008,13 @@ __global__ void attention_simt_kernel(AttnArgs a) {
         sc[j] = s;
         mx = fmaxf(mx, s);
     }
-    mx = warp_max(mx);
+    mx = combine(warp_max(mx), 0, [](float x, float y) { return fmaxf(x, y); });
     float sum = 0.f;
-    for (int j = lane; j < a.N; j += 32) sum += expf(sc[j] - mx);
-    sum = warp_sum(sum);
+    for (int j = t; j < a.N; j += SIMT_WARPS * 32) sum += expf(sc[j] - mx);
+    sum = combine(warp_sum(sum), 1, [](float x, float y) { return x + y; });
     const float lse = mx + logf(sum);
     float kl = 0.f;
-    for (int j = lane; j < a.N; j += 32) {
+    for (int j = t; j < a.N; j += SIMT_WARPS * 32) {
         const float lp = sc[j] - lse;
         const float p = expf(lp);
         if (prev) {
@@ -989,25 +1023,47 @@ __global__ void attention_simt_kernel(AttnArgs a) {
         }
         sc[j] = round_to<T>(p);
     }
-    __syncwarp();
-    if (a.kl) {
-        kl = warp_sum(kl);
-        if (lane == 0) a.kl[(size_t)r * a.n_heads + h] = (prev && a.record_kl) ? kl : 0.f;
-    }
+    kl = combine(warp_sum(kl), 0, [](float x, float y) { return x + y; });        // (also: the probabilities are complete)
+    if (a.kl && t == 0) a.kl[(size_t)r * a.n_heads + h] = (prev && a.record_kl) ? kl : 0.f;
     if (a.out) {
-        T* o = (T*)a.out + (size_t)r * dq + h * dh;
-        for (int c = lane; c < dh; c += 32) {
-            float acc = 0.f;
-            int j = 0;
-            for (; j + 16 <= a.N; j += 16) {          // sixteen rows of V in flight, added in ascending order
-                T v[16];
+        // a warp takes every fourth group of 32 keys, a lane one column or two adjacent ones
+        const bool two = sizeof(T) == 4 && (dh & 63) == 0 && (dkv & 1) == 0 && (((uintptr_t)a.vc) & 7) == 0;
+        for (int c = two ? 2 * lane : lane; c < dh; c += two ? 64 : 32) {
+            float a0 = 0.f, a1 = 0.f;
+            for (int j0 = 32 * wid; j0 < a.N; j0 += 32 * SIMT_WARPS) {
+                const T* vj = V + (size_t)j0 * dkv + c;
+                if (j0 + 32 <= a.N) {
+                    if (two) {
+                        float2 v[32];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = V[(size_t)(j + i) * dkv + c];
+                        for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(vj + (size_t)i * dkv);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) acc = fmaf(sc[j + i], to_f<T>(v[i]), acc);
+                        for (int i = 0; i < 32; ++i) { const float p = sc[j0 + i]; a0 = fmaf(p, v[i].x, a0); a1 = fmaf(p, v[i].y, a1); }
+                    } else {
+                        T v[32];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] = vj[(size_t)i * dkv];
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) a0 = fmaf(sc[j0 + i], to_f<T>(v[i]), a0);
+                    }
+                } else {
+                    for (int i = 0; j0 + i < a.N; ++i) {
+                        const float p = sc[j0 + i];
+                        a0 = fmaf(p, to_f<T>(vj[(size_t)i * dkv]), a0);
+                        if (two) a1 = fmaf(p, to_f<T>(vj[(size_t)i * dkv + 1]), a1);
+                    }
+                }
             }
-            for (; j < a.N; ++j) acc = fmaf(sc[j], to_f<T>(V[(size_t)j * dkv + c]), acc);
-            o[c] = from_f<T>(acc);
+            part[wid * dh + c] = a0;
+            if (two) part[wid * dh + c + 1] = a1;
+        }
+        __syncthreads();
+        T* o = (T*)a.out + (size_t)r * dq + h * dh;
+        for (int c = t; c < dh; c += SIMT_WARPS * 32) {
+            float x = part[c];
+#pragma unroll
+            for (int w = 1; w < SIMT_WARPS; ++w) x += part[w * dh + c];
+            o[c] = from_f<T>(x);
         }
     }
 }
@@ -1073,20 +1129,36 @@ __device__ int select_one(const float* D, int W, int mode, int k, float thresh, 
     float val[SEL_ITEMS];
     bool cand[SEL_ITEMS], sel[SEL_ITEMS];
     // items are blocked: thread t owns indices t*ITEMS .. t*ITEMS+ITEMS-1 (keeps index order in scans)
+    if (t < 256) s.hist[0][t] = 0;
+    if (t == 0) { s.ncand = 0; s.prefix = 0u; s.kleft = k; }
+    if (t * SEL_ITEMS + SEL_ITEMS <= W && ((uintptr_t)D & 15) == 0) {
+        const float4 v = *reinterpret_cast<const float4*>(D + t * SEL_ITEMS);
+        val[0] = v.x; val[1] = v.y; val[2] = v.z; val[3] = v.w;
+    } else {
 #pragma unroll
-    for (int u = 0; u < SEL_ITEMS; ++u) {
-        const int i = t * SEL_ITEMS + u;
-        const float v = i < W ? D[i] : 0.f;
-        cand[u] = (i < W) && (v > floor_);          // NaN compares false: never a candidate
-        val[u] = v;
-        key[u] = float_key(v);
-        sel[u] = false;
+        for (int u = 0; u < SEL_ITEMS; ++u) val[u] = t * SEL_ITEMS + u < W ? D[t * SEL_ITEMS + u] : 0.f;
     }
     int ncand_local = 0;
 #pragma unroll
-    for (int u = 0; u < SEL_ITEMS; ++u) ncand_local += cand[u];
-    int ncand;
-    block_excl_scan(ncand_local, s.scan, &ncand);
+    for (int u = 0; u < SEL_ITEMS; ++u) {
+        cand[u] = (t * SEL_ITEMS + u < W) && (val[u] > floor_);          // NaN compares false: never a candidate
+        key[u] = float_key(val[u]);
+        sel[u] = false;
+        ncand_local += cand[u];
+    }
+    ncand_local = __reduce_add_sync(0xffffffffu, ncand_local);
+    __syncthreads();
+    if ((t & 31) == 0 && ncand_local) atomicAdd(&s.ncand, ncand_local);
+    if (mode < 2) {
+#pragma unroll
+        for (int u = 0; u < SEL_ITEMS; ++u) {
+            const unsigned bkt = cand[u] ? key[u] >> 24 : 256u;
+            const unsigned same = __match_any_sync(0xffffffffu, bkt);
+            if (cand[u] && (t & 31) == __ffs(same) - 1) atomicAdd(&s.hist[0][bkt], __popc(same));
+        }
+    }
+    __syncthreads();
+    const int ncand = s.ncand;
     if (mode == 3) {                                  // ALL: every row
 #pragma unroll
         for (int u = 0; u < SEL_ITEMS; ++u) sel[u] = (t * SEL_ITEMS + u) < W;
@@ -1099,28 +1171,22 @@ __device__ int select_one(const float* D, int W, int mode, int k, float thresh, 
         for (int u = 0; u < SEL_ITEMS; ++u) sel[u] = cand[u];
     } else {
         // radix select, most significant byte first
-        if (t == 0) { s.prefix = 0u; s.kleft = k; }
-        __syncthreads();
         for (int pass = 0; pass < 4; ++pass) {
             const int shift = 24 - 8 * pass;
-            const unsigned himask = pass == 0 ? 0u : (0xFFFFFFFFu << (shift + 8));
-            if (t < 256) s.hist[t] = 0;
-            __syncthreads();
+            int* const hist = s.hist[pass & 1];
             const unsigned prefix = s.prefix;
+            if (pass > 0) {
+                const unsigned himask = 0xFFFFFFFFu << (shift + 8);
 #pragma unroll
-            for (int u = 0; u < SEL_ITEMS; ++u) {
-                // (one addition per distinct bucket of a warp: drift values share their leading bytes)
-                const bool in = cand[u] && (key[u] & himask) == prefix;
-                const unsigned bkt = in ? (key[u] >> shift) & 255u : 256u;
-                const unsigned same = __match_any_sync(0xffffffffu, bkt);
-                if (in && (t & 31) == __ffs(same) - 1) atomicAdd(&s.hist[bkt], __popc(same));
+                for (int u = 0; u < SEL_ITEMS; ++u)
+                    if (cand[u] && (key[u] & himask) == prefix) atomicAdd(&hist[(key[u] >> shift) & 255u], 1);
+                __syncthreads();
             }
-            __syncthreads();
             if (t < 32) {
                 // the bucket that holds the k-th candidate, from the top: lane t owns buckets 255 - 8 t ... 248 - 8 t
                 int c[8], sum = 0;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { c[j] = s.hist[255 - 8 * t - j]; sum += c[j]; }
+                for (int j = 0; j < 8; ++j) { c[j] = hist[255 - 8 * t - j]; sum += c[j]; }
                 int inc = sum;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -1137,6 +1203,8 @@ __device__ int select_one(const float* D, int W, int mode, int k, float thresh, 
                     s.kleft = left;
                     s.prefix = prefix | ((unsigned)(255 - 8 * t - j) << shift);
                 }
+            } else if (t < 288) {
+                s.hist[(pass & 1) ^ 1][t - 32] = 0;
             }
             __syncthreads();
         }
