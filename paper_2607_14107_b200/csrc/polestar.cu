@@ -374,8 +374,10 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
 // Block size of the row-wise staging kernels (one CTA per row, the row in registers): 512 threads for the few rows of a
 // decoding step (latency: every thread has one or two 16-byte loads in flight), 128 threads when a step has hundreds of
 // rows, so that several rows share an SM instead of queueing one 512-thread CTA after the other.
-static int norm_threads(int rows, int d) {
-    return (rows >= 256 && d <= 4 * NORM_VPT * 128) ? 128 : NORM_THREADS;
+// Proxy rows (the mean of a cluster's members) are one long chain each, so a step that has some stays with 512 threads longer: block
+// entry of 392 rows with eight proxies 34.6 us a launch at 128 threads, 19.2 at 512.
+static int norm_threads(int rows, int d, int proxies = 0) {
+    return (rows >= (proxies ? 1024 : 256) && d <= 4 * NORM_VPT * 128) ? 128 : NORM_THREADS;
 }
 
 // Confidence of `rows` logits rows (of *m_count of them, when given).
@@ -1083,7 +1085,7 @@ struct Path {
             if (fold && l > 0) qkv_staged = true;      // the previous down projection stored x * gain and the sums of squares
             if (!qkv_done && !qkv_staged) {      // (else: staged by the previous layer's down projection or chained kernel)
                 Scope sc(c, POLESTAR_PROF_STAGE, (double)M * d * (4 + esd), 0, 1);
-                CK(launch_k(prep_qkv_kernel<T>, dim3(M), dim3(norm_threads(M, d)), 0, st, sd, b.rows, b.x, hc, b.packet, b.patch + (size_t)l * bs * Wm,
+                CK(launch_k(prep_qkv_kernel<T>, dim3(M), dim3(norm_threads(M, d, Kp)), 0, st, sd, b.rows, b.x, hc, b.packet, b.patch + (size_t)l * bs * Wm,
                                                      c->n1[l], m.rms_eps, d, (T*)b.a_buf, b.kvflag, ct));
                 CK(cudaGetLastError());
             }
