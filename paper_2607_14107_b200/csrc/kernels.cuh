@@ -538,51 +538,103 @@ prep_refresh_kernel(const __nv_bfloat16* h, const int* idx, const int* counts, i
 // Deterministic reading: centre j starts at the unit vector of window row floor((j + 1/2) W / K); `iters` Lloyd
 // iterations (assign to the largest cosine, lowest cluster on ties; centre = normalised sum of the members' unit
 // vectors, an empty cluster keeps its centre); no more rows than clusters: every row its own cluster.
-// All sums run in a fixed order.  K <= KM_MAX_K, W <= KM_MAX_W.
+// All sums run in a fixed order.  K <= KM_MAX_K, W <= KM_MAX_W (what a configuration with proxies admits).
+// A chain of dependent phases on L2-resident rows: each keeps eight or sixteen loads per thread in flight (rows in flat member
+// order, across cluster boundaries, in the centre update) and groups the rows by ballots.  96 rows x 4096, 8 clusters, in the pipeline,
+// with
+// single floats, centres in shared memory, a chain per cluster and loops over the labels 130 us, now 82; 64 rows 96, now 56.
 // ---------------------------------------------------------------------------------------
-constexpr int KM_MAX_K = 16, KM_MAX_W = 1024, KM_THREADS = 512, KM_CL = 8, KM_SMEM_BYTES = 160 * 1024;
+constexpr int KM_MAX_K = 16, KM_MAX_W = 256, KM_THREADS = 512, KM_CL = 8, KM_SMEM_BYTES = 160 * 1024;
+constexpr float KM_TIE = 1e-6f;            // eight times the unit roundoff of a cosine's fp32 sums
 struct KmeansArgs {
     const float* x;            // entry forward: residual-stream rows of this layer [rows][d]
     int d, K, iters;
-    int chunk;                 // columns of the centres staged in shared memory at a time (multiple of 128; K * chunk floats)
+    float* invn;               // scratch [batch][W_max]: the rows' 1 / norm
     int* labels; int* zpos; int* zcnt; int* members; int* moff;      // this layer's tables (see ClusterTabs)
     const int* forced_labels;  // [batch][W_max], first entry < 0: not forced (parity replay of another clustering)
     float* z0;                 // NVFP4 residual cache: [batch][K][d] member means of the plain rows (null: not kept)
-    float* cent;               // scratch [batch][K * d + W_max]: the centres (member sums, not normalised), the rows' 1 / norm
 };
-// A cluster of KM_CL CTAs per sequence: the rows are split over the CTAs for the assignment, the columns for the
-// centre update; cluster barriers (release / acquire) separate the phases, data of other CTAs is read through L2.
+// A cluster of KM_CL CTAs per sequence.  The columns are split over the CTAs: each keeps its columns of the centres in shared
+// memory, works out its part of every (row, centre) product with four centres at a time in registers (a row's values against centres in
+// shared memory were bound by its bandwidth), and adds up its columns of the members.  The rows are split over the CTAs for the decision: a row's
+// owner receives the parts in its shared memory, adds them in rank order and sends the label to all.
+__host__ __device__ inline int km_columns(int d) { return (((d + KM_CL - 1) / KM_CL) + 3) & ~3; }                     // per CTA
+__host__ __device__ inline size_t km_smem(int d, int K, int W) { return ((size_t)K * km_columns(d) + (size_t)2 * KM_CL * ((W + KM_CL - 1) / KM_CL) * K) * sizeof(float); }
 __device__ __forceinline__ void km_cluster_sync() {
     __syncthreads();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmeans_kernel(StepDesc sd, KmeansArgs a) {
     KERNEL_PROLOGUE(18);   // kmeans_kernel
-    extern __shared__ __align__(16) float Cs[];             // [K][chunk]
-    const int KM_CHUNK = a.chunk;
+    extern __shared__ __align__(16) float Cs[];             // [K][columns of this CTA]: the centres (member sums, not normalised)
     __shared__ float invn[KM_MAX_W];
     __shared__ int lab[KM_MAX_W];
     __shared__ float inv_c[KM_MAX_K];
     __shared__ int cnt[KM_MAX_K + 1], off[KM_MAX_K + 1];
     __shared__ unsigned short ord[KM_MAX_W];                 // window rows grouped by cluster, ascending inside a cluster
+    // ... their rows of x, 1 / norm, and (last of a cluster) the cluster + 1
+    __shared__ int ord_row[KM_MAX_W];
+    __shared__ float ord_inv[KM_MAX_W];
+    __shared__ unsigned char ord_last[KM_MAX_W];
+    __shared__ int wcnt[KM_MAX_W / 32][KM_MAX_K];
+    __shared__ float c2[KM_CL][KM_MAX_K];                    // every CTA's part of |centre|^2
     const int s = blockIdx.y, rk = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = KM_THREADS / 32;
     const int W = sd.W, K = a.K, d = a.d;
-    auto row = [&](int w) { return a.x + ((size_t)s * sd.rows_per_seq + (window_pos(sd, w) - sd.e0)) * d; };
-    // lab[] -> cnt[], off[], ord[] (the whole block calls)
+    auto row_index = [&](int w) { return s * sd.rows_per_seq + (window_pos(sd, w) - sd.e0); };
+    auto row = [&](int w) { return a.x + (size_t)row_index(w) * d; };
+    // lab[] -> cnt[], off[], ord[], ord_row[] (the whole block calls): ballots of the rows' labels, a warp per 32 rows
     auto group_rows = [&]() {
         __syncthreads();
-        if (t < K) { int n = 0; for (int w = 0; w < W; ++w) n += lab[w] == t; cnt[t] = n; }
+        const int mine = t < W ? lab[t] : -1;
+        int before = 0;                                      // rows of the own cluster in front of this one in its warp
+        if (warp < KM_MAX_W / 32)
+            for (int j = 0; j < K; ++j) {
+                const unsigned b = __ballot_sync(0xffffffffu, mine == j);
+                if (lane == 0) wcnt[warp][j] = __popc(b);
+                if (mine == j) before = __popc(b & ((1u << lane) - 1u));
+            }
         __syncthreads();
-        if (t == 0) { int o = 0; for (int j = 0; j < K; ++j) { off[j] = o; o += cnt[j]; } off[K] = o; }
+        if (t < 32) {
+            int n = 0;
+            if (t < K) for (int q = 0; q < KM_MAX_W / 32; ++q) { const int c = wcnt[q][t]; wcnt[q][t] = n; n += c; }
+            int inc = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, inc, o); if (t >= o) inc += up; }
+            if (t < K) { cnt[t] = n; off[t] = inc - n; }
+            if (t == K - 1) off[K] = inc;
+        }
         __syncthreads();
-        if (t < K) { int o = off[t]; for (int w = 0; w < W; ++w) if (lab[w] == t) ord[o++] = (unsigned short)w; }
+        if (mine >= 0) {
+            const int o = off[mine] + wcnt[warp][mine] + before;
+            ord[o] = (unsigned short)t;
+            ord_row[o] = row_index(t);
+            ord_inv[o] = invn[t];
+            ord_last[o] = o + 1 == off[mine] + cnt[mine] ? mine + 1 : 0;
+        }
         __syncthreads();
     };
-    float* C = a.cent + (size_t)s * ((size_t)K * d + sd.W_max);
-    float* invn_g = C + (size_t)K * d;
+    // sums over the members of every cluster for one column, rows in flat member order: done(cluster, sum), empty clusters left out
+    auto member_sums = [&](int c, auto term, auto done) {
+        float acc = 0.f;
+        for (int i0 = 0; i0 < W; i0 += 16) {
+            float v[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = i0 + k < W ? __ldg(a.x + (size_t)ord_row[i0 + k] * d + c) : 0.f;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                if (i0 + k >= W) break;
+                acc = term(acc, v[k], i0 + k);
+                const int last = ord_last[i0 + k];
+                if (last) { done(last - 1, acc); acc = 0.f; }
+            }
+        }
+    };
+    float* invn_g = a.invn + (size_t)s * sd.W_max;
     int* labels = a.labels + (size_t)s * sd.W_max;
     const int per = (W + KM_CL - 1) / KM_CL, w_lo = min(W, rk * per), w_hi = min(W, w_lo + per);     // this CTA's rows
-    const int dper = (((d + KM_CL - 1) / KM_CL) + 3) & ~3, c_lo = min(d, rk * dper), c_hi = min(d, c_lo + dper);   // ... and columns
+    const int dper = km_columns(d), c_lo = min(d, rk * dper), c_hi = min(d, c_lo + dper), cols = c_hi - c_lo;        // ... and columns
+    float* const part = Cs + (size_t)K * dper;               // [W][K] this CTA's part of the products
+    float* const recv = part + (size_t)KM_CL * per * K;      // [CTA][per][K] the parts of this CTA's rows
     const int* forced = a.forced_labels ? a.forced_labels + (size_t)s * sd.W_max : nullptr;
     if (forced && forced[0] >= 0) {
         for (int w = w_lo + t; w < w_hi; w += KM_THREADS) labels[w] = min(max(forced[w], 0), K - 1);
@@ -591,89 +643,138 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
     } else {
         for (int w = w_lo + warp; w < w_hi; w += nw) {
             float ss = 0.f;
-            const float* h = row(w);
-            for (int c = lane; c < d; c += 32) { const float v = h[c]; ss = fmaf(v, v, ss); }
+            const float4* h4 = reinterpret_cast<const float4*>(row(w));
+            for (int q0 = lane; q0 < (d >> 2); q0 += 8 * 32) {
+                float4 v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = q0 + 32 * u < (d >> 2) ? __ldg(h4 + q0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) ss = fmaf(v[u].x, v[u].x, fmaf(v[u].y, v[u].y, fmaf(v[u].z, v[u].z, fmaf(v[u].w, v[u].w, ss))));
+            }
             ss = warp_sum(ss);
             if (lane == 0) invn_g[w] = ss > 0.f ? rsqrtf(ss) : 0.f;
         }
-        for (int j = rk; j < K; j += KM_CL) {                                  // starting centres: rows of the window
-            const int w0 = (int)(((2 * j + 1) * (long long)W) / (2 * K));       // floor((j + 1/2) W / K)
-            const float* h = row(w0);
-            for (int c = t; c < d; c += KM_THREADS) C[(size_t)j * d + c] = h[c];
+        // starting centres: rows floor((j + 1/2) W / K) of the window
+        for (int e = t; e < K * cols; e += KM_THREADS) {
+            const int j = e / cols, c = e - j * cols;
+            Cs[(size_t)j * dper + c] = row((int)(((2 * j + 1) * (long long)W) / (2 * K)))[c_lo + c];
         }
         km_cluster_sync();
         for (int w = t; w < W; w += KM_THREADS) invn[w] = __ldcg(invn_g + w);
+        const int groups = (K + 3) / 4, team = nw / groups;      // warps per group of four centres
+        const int grp = warp / team, wt = warp - grp * team;
         for (int it = 0; it < a.iters; ++it) {
-            // ---- assignment of this CTA's rows: a warp per row, the centres through shared memory in column chunks
-            for (int w_base = w_lo; w_base < w_hi || w_base == w_lo; w_base += nw) {
-                const int w = w_base + warp;
-                const bool live = w < w_hi;
-                const float* h = live ? row(w) : a.x;
-                float dot[KM_MAX_K];
+            // ---- this CTA's part of every product
+            __syncthreads();
+            if (grp < groups) {
+                for (int q_lo = 0; q_lo < cols; q_lo += 512) {
+                    float4 cv[4][4];
 #pragma unroll
-                for (int j = 0; j < KM_MAX_K; ++j) dot[j] = 0.f;
-                float n2 = 0.f;                                                 // warp j: |centre j|^2 (first round only)
-                for (int c0 = 0; c0 < d; c0 += KM_CHUNK) {
-                    const int cw = min(KM_CHUNK, d - c0);
-                    __syncthreads();
-#pragma unroll 8
-                    for (int e = t; e < K * (KM_CHUNK / 4); e += KM_THREADS) {
-                        const int j = e / (KM_CHUNK / 4), q = e - j * (KM_CHUNK / 4);
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (4 * q < cw) v = __ldcg(reinterpret_cast<const float4*>(C + (size_t)j * d + c0) + q);
-                        reinterpret_cast<float4*>(Cs + (size_t)j * KM_CHUNK)[q] = v;
-                    }
-                    __syncthreads();
-                    if (w_base == w_lo && warp < K)
-                        for (int q = lane; q < KM_CHUNK; q += 32) n2 = fmaf(Cs[warp * KM_CHUNK + q], Cs[warp * KM_CHUNK + q], n2);
-                    if (live) {
-#pragma unroll 4
-                        for (int q = lane * 4; q < cw; q += 128) {
-                            const float4 hv = *reinterpret_cast<const float4*>(h + c0 + q);
+                    for (int j = 0; j < 4; ++j)
 #pragma unroll
-                            for (int j = 0; j < KM_MAX_K; ++j) {
-                                if (j < K) {
-                                    const float4 cv = *reinterpret_cast<const float4*>(Cs + j * KM_CHUNK + q);
-                                    dot[j] = fmaf(hv.x, cv.x, fmaf(hv.y, cv.y, fmaf(hv.z, cv.z, fmaf(hv.w, cv.w, dot[j]))));
-                                }
-                            }
+                        for (int u = 0; u < 4; ++u) {
+                            const int c = q_lo + 4 * (lane + 32 * u);
+                            cv[j][u] = (4 * grp + j < K && c < cols) ? *reinterpret_cast<const float4*>(Cs + (size_t)(4 * grp + j) * dper + c) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
-                    }
-                }
-                if (w_base == w_lo) {
-                    n2 = warp_sum(n2);
-                    if (warp < K && lane == 0) inv_c[warp] = n2 > 0.f ? rsqrtf(n2) : 0.f;
-                }
-                __syncthreads();
-                if (live) {
-                    float best = -INFINITY;
-                    int bj = 0;
+                    float4 hv[2][4];                              // this row and the next one, on its way
+                    auto fetch = [&](int w, float4 (&v)[4]) {
+                        const float* h = row(min(w, W - 1)) + c_lo;
 #pragma unroll
-                    for (int j = 0; j < KM_MAX_K; ++j) {
-                        if (j < K) {
-                            const float cs = warp_sum(dot[j]) * inv_c[j] * invn[w];
-                            if (cs > best) { best = cs; bj = j; }          // (lowest cluster on ties)
+                        for (int u = 0; u < 4; ++u) {
+                            const int c = q_lo + 4 * (lane + 32 * u);
+                            v[u] = c < cols ? __ldg(reinterpret_cast<const float4*>(h + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
+                    };
+                    auto products = [&](int w, const float4 (&hv)[4]) {
+                        float dot[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            dot[j] = 0.f;
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                dot[j] = fmaf(hv[u].x, cv[j][u].x, fmaf(hv[u].y, cv[j][u].y, fmaf(hv[u].z, cv[j][u].z, fmaf(hv[u].w, cv[j][u].w, dot[j]))));
+                        }
+                        // four sums over the warp: after two exchange steps a lane carries one of them
+                        const float x0 = __shfl_xor_sync(0xffffffffu, (lane & 1) ? dot[0] : dot[1], 1), x1 = __shfl_xor_sync(0xffffffffu, (lane & 1) ? dot[2] : dot[3], 1);
+                        const float y0 = ((lane & 1) ? dot[1] : dot[0]) + x0, y1 = ((lane & 1) ? dot[3] : dot[2]) + x1;
+                        float z = ((lane & 2) ? y1 : y0) + __shfl_xor_sync(0xffffffffu, (lane & 2) ? y0 : y1, 2);
+                        z += __shfl_xor_sync(0xffffffffu, z, 4);
+                        z += __shfl_xor_sync(0xffffffffu, z, 8);
+                        z += __shfl_xor_sync(0xffffffffu, z, 16);
+                        const int j = 4 * grp + (lane & 3);                  // (lane 0: 0, 1: 1, 2: 2, 3: 3)
+                        if (lane < 4 && j < K) {
+                            float* dst = part + w * K + j;
+                            *dst = q_lo ? *dst + z : z;
+                        }
+                    };
+                    fetch(wt, hv[0]);
+                    for (int w = wt; w < W; w += 2 * team) {
+                        fetch(w + team, hv[1]);
+                        products(w, hv[0]);
+                        if (w + team >= W) break;
+                        fetch(w + 2 * team, hv[0]);
+                        products(w + team, hv[1]);
                     }
-                    if (lane == 0) labels[w] = bj;
                 }
-                if (w_hi <= w_lo) break;
+            }
+            if (warp < K) {
+                float n2 = 0.f;
+                for (int c = 4 * lane; c < cols; c += 128) {
+                    const float4 v = *reinterpret_cast<const float4*>(Cs + (size_t)warp * dper + c);
+                    n2 = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, n2))));
+                }
+                n2 = warp_sum(n2);
+                if (lane < KM_CL) {
+                    const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(&c2[rk][warp]), lane);
+                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(n2) : "memory");
+                }
+            }
+            __syncthreads();
+            for (int e = t; e < W * K; e += KM_THREADS) {
+                const int w = e / K, o = w / per;
+                const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(recv + ((size_t)rk * per + (w - o * per)) * K + (e - w * K)), o);
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(part[e]) : "memory");
+            }
+            km_cluster_sync();
+            // ---- labels of this CTA's rows, to every CTA
+            if (t < K) {
+                float n2 = 0.f;
+#pragma unroll
+                for (int r = 0; r < KM_CL; ++r) n2 += c2[r][t];
+                inv_c[t] = n2 > 0.f ? rsqrtf(n2) : 0.f;
+            }
+            __syncthreads();
+            // a half warp per row, a lane per centre
+            for (int w0 = w_lo; w0 < w_hi; w0 += KM_THREADS / 16) {
+                const int w = w0 + (t >> 4), j = t & 15;
+                float cs = -INFINITY;
+                if (w < w_hi && j < K) {
+                    float dot = 0.f;
+#pragma unroll
+                    for (int r = 0; r < KM_CL; ++r) dot += recv[((size_t)r * per + (w - w_lo)) * K + j];
+                    cs = dot * inv_c[j] * invn[w];
+                }
+                float best = cs;
+#pragma unroll
+                for (int o = 1; o < 16; o <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+                // lowest cluster on ties: cosines that differ by less than the rounding of their sums are the same (rows that agree, as
+                // masked positions do, meet centres that are sums of a different number of them)
+                const unsigned tie = __ballot_sync(0xffffffffu, cs >= best - KM_TIE);
+                const int bj = max(__ffs((tie >> (t & 16)) & 0xffffu) - 1, 0);
+                if (w < w_hi) {
+                    if (j == 0) labels[w] = bj;
+                    if (j < KM_CL) {
+                        const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(lab + w), j);
+                        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst), "r"(bj) : "memory");
+                    }
+                }
             }
             km_cluster_sync();
             if (it + 1 == a.iters) break;          // the centres of the last update are never used
             // ---- update of this CTA's columns: members added in ascending row order; an empty cluster keeps its centre
-            for (int w = t; w < W; w += KM_THREADS) lab[w] = __ldcg(labels + w);
             group_rows();
-            for (int c = c_lo + t; c < c_hi; c += KM_THREADS) {
-                for (int j = 0; j < K; ++j) {
-                    if (cnt[j] == 0) continue;
-                    float acc = 0.f;
-#pragma unroll 8
-                    for (int i = off[j]; i < off[j + 1]; ++i) { const int w = ord[i]; acc += row(w)[c] * invn[w]; }
-                    C[(size_t)j * d + c] = acc;
-                }
-            }
-            km_cluster_sync();
+            for (int c = c_lo + t; c < c_hi; c += KM_THREADS)
+                member_sums(c, [&](float acc, float v, int i) { return acc + v * ord_inv[i]; }, [&](int j, float sum) { Cs[(size_t)j * dper + c - c_lo] = sum; });
         }
     }
     km_cluster_sync();
@@ -695,12 +796,9 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
     if (a.z0) {
         // reference rows of the residual codec: the clusters' centroids as this block entry sees them (this CTA's columns)
         for (int c = c_lo + t; c < c_hi; c += KM_THREADS) {
-            for (int j = 0; j < K; ++j) {
-                float acc = 0.f;
-#pragma unroll 8
-                for (int i = off[j]; i < off[j + 1]; ++i) acc += row(ord[i])[c];
-                a.z0[((size_t)s * K + j) * d + c] = cnt[j] > 0 ? acc * (1.f / (float)cnt[j]) : 0.f;
-            }
+            for (int j = 0; j < K; ++j) if (cnt[j] == 0) a.z0[((size_t)s * K + j) * d + c] = 0.f;
+            member_sums(c, [&](float acc, float v, int) { return acc + v; },
+                        [&](int j, float sum) { a.z0[((size_t)s * K + j) * d + c] = sum * (1.f / (float)cnt[j]); });
         }
     }
 }

@@ -832,7 +832,7 @@ static size_t make_plan(const polestar_model* m, const polestar_params* p, Buffe
     TAKE(moff, int, Kp ? L * bs * (Kp + 1) : 1);
     TAKE(forced_labels, int, Kp ? L * bs * Wm : 1);
     TAKE(zbuf, float, Kp ? bs * Kp * d : 1);
-    TAKE(kcent, float, Kp ? bs * (Kp * d + Wm) : 1);
+    TAKE(kcent, float, Kp ? bs * Wm : 1);
     TAKE(hq, unsigned char, quant ? L * bs * Wm * (d / 2) : 1);
     TAKE(hs, unsigned char, quant ? L * bs * Wm * (d / 16) : 1);
     TAKE(z0, float, quant ? L * bs * Kp * d : 1);
@@ -1073,9 +1073,8 @@ struct Path {
                     ka.x = b.x; ka.d = d; ka.K = Kp; ka.iters = p.kmeans_iters;
                     ka.labels = b.labels + (size_t)l * bs * Wm; ka.zpos = b.zpos + (size_t)l * bs * Kp; ka.zcnt = b.zcnt + (size_t)l * bs * Kp;
                     ka.members = b.members + (size_t)l * bs * Wm; ka.moff = b.moff + (size_t)l * bs * (Kp + 1);
-                    ka.forced_labels = b.forced_labels + (size_t)l * bs * Wm; ka.cent = b.kcent; ka.z0 = ct.z0;
-                    ka.chunk = std::min((d + 127) & ~127, (KM_SMEM_BYTES / (Kp * 4)) & ~127);
-                    CK(launch_k(kmeans_kernel, dim3(KM_CL, bs), dim3(KM_THREADS), (size_t)Kp * ka.chunk * 4, st, sd, ka));
+                    ka.forced_labels = b.forced_labels + (size_t)l * bs * Wm; ka.invn = b.kcent; ka.z0 = ct.z0;
+                    CK(launch_k(kmeans_kernel, dim3(KM_CL, bs), dim3(KM_THREADS), km_smem(d, Kp, sd.W), st, sd, ka));
                 }
             }
             if (p.flags & POLESTAR_FLAG_KEEP_HIDDEN) {
