@@ -1,8 +1,9 @@
 // Bidirectional attention rows with drift (Eq. 3, Eq. 4) as a STREAM over the key tiles: one CTA per
 // (128 query rows, head) walks all keys twice, with the tensor core, the loads and the sixteen statistics warps
 // overlapped through rings of operand tiles and two score accumulators in tensor memory.  bf16, head_dim 128,
-// any number of keys.  For steps with many rows (block entries, long sequences, batches), where the kernel of
-// attn_tc.cuh -- one tile per CTA, key ranges combined across a cluster -- spends its time in start-up and exchange.
+// any number of keys.  For a single key tile, and in forwards over up to 512 keys for steps with many rows (block entries,
+// batches), where the kernel of attn_tc.cuh -- one tile per CTA, key ranges combined across a cluster -- spends its time in
+// start-up and exchange; beyond that the one-pass kernel of attn_flash.cuh takes over.
 //
 //   pass 1   S_t = Q K_t^T for every key tile t (tcgen05.mma into accumulator t & 1); the statistics warps read
 //            each S_t from tensor memory (lane = row, four threads per row) and keep a running maximum and sum:
