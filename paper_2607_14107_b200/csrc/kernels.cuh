@@ -133,7 +133,8 @@ __device__ __forceinline__ void zero_row(T* a, int d) {
 //   window rows of a within-block step read the hidden cache (after taking the packet row if
 //   the previous layer selected them); every other row reads the residual stream x.
 // ---------------------------------------------------------------------------------------
-template <typename T>
+// TABS false: a step without cluster tables (no proxy rows, no quantised cache), whose rows need half of the registers
+template <typename T, bool TABS = true>
 __device__ __forceinline__ void prep_qkv_row(const StepDesc& sd, int r, const Row* rows, float* x, float* hc, const float* packet,
                                              const unsigned char* patch, const float* gain, float eps, int d,
                                              T* a_out, unsigned char* kvflag, float* red, const ClusterTabs& ct) {
@@ -144,7 +145,7 @@ __device__ __forceinline__ void prep_qkv_row(const StepDesc& sd, int r, const Ro
         if (threadIdx.x == 0) kvflag[r] = 0;
         return;
     }
-    if (row_is_proxy(rw.widx)) {
+    if (TABS && row_is_proxy(rw.widx)) {
         // Proxy of a cluster = mean of its members' current hidden rows (Sec. 4.1: the centroid follows its refreshed
         // members; rebuilding the mean from the cache is that incremental update without its rounding drift).
         // Members are added in ascending window order by every thread for its own columns: deterministic.
@@ -271,7 +272,7 @@ __device__ __forceinline__ void prep_qkv_row(const StepDesc& sd, int r, const Ro
     }
     float* xr = x + (size_t)r * d;
     bool kv = true;
-    if (rw.widx >= 0 && ct.hq) {
+    if (TABS && rw.widx >= 0 && ct.hq) {
         // ---- NVFP4 residual cache: the row's codes against its cluster's block-entry centroid
         const size_t o = (size_t)rw.seq * sd.W_max + rw.widx;
         const float* ref = ct.z0 + ((size_t)rw.seq * ct.K + ct.labels[o]) * d;
@@ -350,13 +351,13 @@ __global__ void impose_codes_kernel(const unsigned char* fmask, const unsigned c
     for (int i = threadIdx.x; i < (d >> 4); i += blockDim.x) hs[o * (size_t)(d >> 4) + i] = fs[o * (size_t)(d >> 4) + i];
 }
 
-template <typename T>
+template <typename T, bool TABS>
 __global__ void prep_qkv_kernel(StepDesc sd, const Row* rows, float* x, float* hc, const float* packet,
                                 const unsigned char* patch, const float* gain, float eps, int d,
                                 T* a_out, unsigned char* kvflag, ClusterTabs ct) {
     KERNEL_PROLOGUE(3);   // prep_qkv_kernel
     __shared__ float red[33];
-    prep_qkv_row<T>(sd, blockIdx.x, rows, x, hc, packet, patch, gain, eps, d, a_out, kvflag, red, ct);
+    prep_qkv_row<T, TABS>(sd, blockIdx.x, rows, x, hc, packet, patch, gain, eps, d, a_out, kvflag, red, ct);
 }
 
 // RMSNorm of a compacted list of rows (FFN input, LM-head input).

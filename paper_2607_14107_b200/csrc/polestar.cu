@@ -371,6 +371,8 @@ static int launch_gemm_tc(MapCache& maps, const GemmWs& ws, const void* A, const
     return POLESTAR_OK;
 }
 
+// (Steps without cluster tables stage their QKV rows with a kernel of their own, 72 registers instead of 128: in the pipeline, us, 16384
+// rows 130 -> 107, 4096 rows of 3584 32 -> 25, 2523 rows 24.6 -> 18.4, 32 rows 4.7 -> 4.2.)
 // Block size of the row-wise staging kernels (one CTA per row, the row in registers): 512 threads for the few rows of a
 // decoding step (latency: every thread has one or two 16-byte loads in flight), 128 threads when a step has hundreds of
 // rows, so that several rows share an SM instead of queueing one 512-thread CTA after the other.
@@ -1084,7 +1086,7 @@ struct Path {
             if (fold && l > 0) qkv_staged = true;      // the previous down projection stored x * gain and the sums of squares
             if (!qkv_done && !qkv_staged) {      // (else: staged by the previous layer's down projection or chained kernel)
                 Scope sc(c, POLESTAR_PROF_STAGE, (double)M * d * (4 + esd), 0, 1);
-                CK(launch_k(prep_qkv_kernel<T>, dim3(M), dim3(norm_threads(M, d, Kp)), 0, st, sd, b.rows, b.x, hc, b.packet, b.patch + (size_t)l * bs * Wm,
+                CK(launch_k(Kp > 0 ? prep_qkv_kernel<T, true> : prep_qkv_kernel<T, false>, dim3(M), dim3(norm_threads(M, d, Kp)), 0, st, sd, b.rows, b.x, hc, b.packet, b.patch + (size_t)l * bs * Wm,
                                                      c->n1[l], m.rms_eps, d, (T*)b.a_buf, b.kvflag, ct));
                 CK(cudaGetLastError());
             }
