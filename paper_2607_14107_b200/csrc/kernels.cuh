@@ -760,7 +760,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                 for (int o = 1; o < 16; o <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
                 // lowest cluster on ties: cosines that differ by less than the rounding of their sums are the same (rows that agree, as
                 // masked positions do, meet centres that are sums of a different number of them)
-                const unsigned tie = __ballot_sync(0xffffffffu, cs >= best - KM_TIE);
+                const unsigned tie = __ballot_sync(0xffffffffu, j < K && cs >= best - KM_TIE);      // (no centre: a row of NaN, lowest cluster)
                 const int bj = max(__ffs((tie >> (t & 16)) & 0xffffu) - 1, 0);
                 if (w < w_hi) {
                     if (j == 0) labels[w] = bj;

@@ -248,6 +248,27 @@ def test_centroid_proxy_own_clustering_matches_oracle():
     assert seen["clusterings"] >= 2, seen
 
 
+def test_clustering_of_rows_that_are_not_numbers():
+    # a NaN embedding in the window: the row's cosines are NaN with every centre, it goes to the lowest cluster (whose
+    # centre then is NaN too, so no other row stays there); behind the first attention every row is NaN
+    m, p = I.config("c1")
+    p = dataclasses.replace(p, select_mode=I.SELECT_CLUSTER_TOPK)
+    w = I.make_weights(m, seed=0, std=0.2)
+    prompt = I.make_prompt(m, p)
+    bad = 37                                                   # (a window row that no centre starts from)
+    tok = int(prompt.numpy().reshape(-1)[bad])
+    w["embed"][tok, 5] = float("nan")
+    hit = np.nonzero(prompt.numpy().reshape(-1) == tok)[0]
+    gpu = Bd.Polestar(m, Bd.pack_weights(m, w), p, prompt.numpy())
+    W, K = gpu.W_max, p.n_clusters
+    first, second = (gpu.read(Bd.READ_LABELS, l)[0, :W] for l in range(2))
+    gpu.destroy()
+    starts = [(2 * j + 1) * W // (2 * K) for j in range(K)]
+    assert not set(hit.tolist()) & set(starts)
+    assert (first[hit] == 0).all() and (np.delete(first, hit) > 0).all() and first.max() < K
+    assert (second == 0).all()
+
+
 def test_c1_refresh_every_step_with_scaled_logits():
     seen = run_forced("c1", 20, tau_upd=-1, logit_scale=12.0, tau_suffix=0.5)
     assert seen["refresh"] > 10
