@@ -634,6 +634,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
     int* labels = a.labels + (size_t)s * sd.W_max;
     const int per = (W + KM_CL - 1) / KM_CL, w_lo = min(W, rk * per), w_hi = min(W, w_lo + per);     // this CTA's rows
     const int dper = km_columns(d), c_lo = min(d, rk * dper), c_hi = min(d, c_lo + dper), cols = c_hi - c_lo;        // ... and columns
+    const int n_rk = (d + dper - 1) / dper;                  // CTAs with columns (few of them leave the last CTAs none): only these have parts
     float* const part = Cs + (size_t)K * dper;               // [W][K] this CTA's part of the products
     float* const recv = part + (size_t)KM_CL * per * K;      // [CTA][per][K] the parts of this CTA's rows
     const int* forced = a.forced_labels ? a.forced_labels + (size_t)s * sd.W_max : nullptr;
@@ -718,7 +719,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                     }
                 }
             }
-            if (warp < K) {
+            if (rk < n_rk && warp < K) {
                 float n2 = 0.f;
                 for (int c = 4 * lane; c < cols; c += 128) {
                     const float4 v = *reinterpret_cast<const float4*>(Cs + (size_t)warp * dper + c);
@@ -731,7 +732,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                 }
             }
             __syncthreads();
-            for (int e = t; e < W * K; e += KM_THREADS) {
+            if (rk < n_rk) for (int e = t; e < W * K; e += KM_THREADS) {
                 const int w = e / K, o = w / per;
                 const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(recv + ((size_t)rk * per + (w - o * per)) * K + (e - w * K)), o);
                 asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(part[e]) : "memory");
@@ -741,7 +742,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
             if (t < K) {
                 float n2 = 0.f;
 #pragma unroll
-                for (int r = 0; r < KM_CL; ++r) n2 += c2[r][t];
+                for (int r = 0; r < KM_CL; ++r) n2 += r < n_rk ? c2[r][t] : 0.f;
                 inv_c[t] = n2 > 0.f ? rsqrtf(n2) : 0.f;
             }
             __syncthreads();
@@ -752,7 +753,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                 if (w < w_hi && j < K) {
                     float dot = 0.f;
 #pragma unroll
-                    for (int r = 0; r < KM_CL; ++r) dot += recv[((size_t)r * per + (w - w_lo)) * K + j];
+                    for (int r = 0; r < KM_CL; ++r) dot += r < n_rk ? recv[((size_t)r * per + (w - w_lo)) * K + j] : 0.f;
                     cs = dot * inv_c[j] * invn[w];
                 }
                 float best = cs;

@@ -248,6 +248,22 @@ def test_centroid_proxy_own_clustering_matches_oracle():
     assert seen["clusterings"] >= 2, seen
 
 
+@pytest.mark.parametrize("d", [8, 40, 72, 104, 136, 168, 264, 4352])
+def test_own_clustering_at_any_width(d):
+    # K-means splits the columns over eight CTAs: widths that leave the last ones none (8: six of them, 40 to 168: one to three), a
+    # last share that is smaller than the others (264), shares of more than 512 columns (4352).  The inputs are far from ties: the
+    # oracle's largest cosine beats the next one by more than 5e-6 in every assignment (equal
+    # rows apart).
+    m, p, gpu, ora = setup("c1", 0.2, model=dict(d_model=d), batch=2, select_mode=I.SELECT_CLUSTER_TOPK)
+    ora.step()
+    for l in range(m.n_layers):
+        for s in range(p.batch):
+            want = ora.seqs[s].labels[l]
+            assert len(want) > p.n_clusters
+            assert np.array_equal(gpu.read(Bd.READ_LABELS, l)[s, :len(want)], want), (l, s)
+    gpu.destroy()
+
+
 def test_clustering_of_rows_that_are_not_numbers():
     # a NaN embedding in the window: the row's cosines are NaN with every centre, it goes to the lowest cluster (whose
     # centre then is NaN too, so no other row stays there); behind the first attention every row is NaN
