@@ -546,7 +546,13 @@ prep_refresh_kernel(const __nv_bfloat16* h, const int* idx, const int* counts, i
 // single floats, centres in shared memory, a chain per cluster and loops over the labels 130 us, now 82; 64 rows 96, now 56.
 // ---------------------------------------------------------------------------------------
 constexpr int KM_MAX_K = 16, KM_MAX_W = 256, KM_THREADS = 512, KM_CL = 8, KM_SMEM_BYTES = 160 * 1024;
-constexpr float KM_TIE = 1e-6f;            // eight times the unit roundoff of a cosine's fp32 sums
+// A row's fp32 cosines are compared where they differ by more than their sums' rounding can: two chains of at most 40 additions for
+// the product and the centre's norm, 80 x 2^-24.  Centres within that of the best are compared again by products and norms in 64 bits (rows of the
+// lower layers, masked positions above all, are nearly parallel: the cosines of a decision are then within 1e-7 of one another).
+constexpr float KM_NEAR = 5e-6f;
+// What is left is the rounding of the centres, fp32 sums of up to KM_MAX_W unit vectors.  Rows that agree give centres along the same line, each of
+// whose columns is off by at most n 2^-24 of itself, so their cosines are at least 1 - (n 2^-24)^2 / 2: closer than that is a tie.
+constexpr double KM_TIE = 0.5 * (KM_MAX_W / 16777216.0) * (KM_MAX_W / 16777216.0);
 struct KmeansArgs {
     const float* x;            // entry forward: residual-stream rows of this layer [rows][d]
     int d, K, iters;
@@ -565,6 +571,28 @@ __device__ __forceinline__ void km_cluster_sync() {
     __syncthreads();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// a value into the same place of CTA `cta`'s shared memory
+__device__ __forceinline__ void km_push(float* p, float v, int cta) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dsmem_addr((uint32_t)__cvta_generic_to_shared(p), cta)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void km_push(int* p, int v, int cta) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dsmem_addr((uint32_t)__cvta_generic_to_shared(p), cta)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void km_push(double* p, double v, int cta) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dsmem_addr((uint32_t)__cvta_generic_to_shared(p), cta)), "d"(v) : "memory");
+}
+// sum of n products (n a multiple of four, 16-byte aligned) in 64 bits, by a warp
+__device__ __forceinline__ double km_dot(const float* x, const float* y, int n, int lane) {
+    double acc = 0.;
+    for (int c = 4 * lane; c < n; c += 128) {
+        const float4 u = *reinterpret_cast<const float4*>(x + c), v = *reinterpret_cast<const float4*>(y + c);
+        acc = fma((double)u.x, (double)v.x, acc); acc = fma((double)u.y, (double)v.y, acc);
+        acc = fma((double)u.z, (double)v.z, acc); acc = fma((double)u.w, (double)v.w, acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
 __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmeans_kernel(StepDesc sd, KmeansArgs a) {
     KERNEL_PROLOGUE(18);   // kmeans_kernel
     extern __shared__ __align__(16) float Cs[];             // [K][columns of this CTA]: the centres (member sums, not normalised)
@@ -579,6 +607,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
     __shared__ unsigned char ord_last[KM_MAX_W];
     __shared__ int wcnt[KM_MAX_W / 32][KM_MAX_K];
     __shared__ float c2[KM_CL][KM_MAX_K];                    // every CTA's part of |centre|^2
+    __shared__ double c2_64[KM_CL][KM_MAX_K];
     const int s = blockIdx.y, rk = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = KM_THREADS / 32;
     const int W = sd.W, K = a.K, d = a.d;
     auto row_index = [&](int w) { return s * sd.rows_per_seq + (window_pos(sd, w) - sd.e0); };
@@ -637,6 +666,7 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
     const int n_rk = (d + dper - 1) / dper;                  // CTAs with columns (few of them leave the last CTAs none): only these have parts
     float* const part = Cs + (size_t)K * dper;               // [W][K] this CTA's part of the products
     float* const recv = part + (size_t)KM_CL * per * K;      // [CTA][per][K] the parts of this CTA's rows
+    double* const recv_64 = reinterpret_cast<double*>(part); // [CTA][per][K] the same in 64 bits, in the place of both
     const int* forced = a.forced_labels ? a.forced_labels + (size_t)s * sd.W_max : nullptr;
     if (forced && forced[0] >= 0) {
         for (int w = w_lo + t; w < w_hi; w += KM_THREADS) labels[w] = min(max(forced[w], 0), K - 1);
@@ -726,16 +756,12 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                     n2 = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, n2))));
                 }
                 n2 = warp_sum(n2);
-                if (lane < KM_CL) {
-                    const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(&c2[rk][warp]), lane);
-                    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(n2) : "memory");
-                }
+                if (lane < KM_CL) km_push(&c2[rk][warp], n2, lane);
             }
             __syncthreads();
             if (rk < n_rk) for (int e = t; e < W * K; e += KM_THREADS) {
                 const int w = e / K, o = w / per;
-                const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(recv + ((size_t)rk * per + (w - o * per)) * K + (e - w * K)), o);
-                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(part[e]) : "memory");
+                km_push(recv + ((size_t)rk * per + (w - o * per)) * K + (e - w * K), part[e], o);
             }
             km_cluster_sync();
             // ---- labels of this CTA's rows, to every CTA
@@ -759,19 +785,55 @@ __global__ void __cluster_dims__(KM_CL, 1, 1) __launch_bounds__(KM_THREADS) kmea
                 float best = cs;
 #pragma unroll
                 for (int o = 1; o < 16; o <<= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-                // lowest cluster on ties: cosines that differ by less than the rounding of their sums are the same (rows that agree, as
-                // masked positions do, meet centres that are sums of a different number of them)
-                const unsigned tie = __ballot_sync(0xffffffffu, j < K && cs >= best - KM_TIE);      // (no centre: a row of NaN, lowest cluster)
-                const int bj = max(__ffs((tie >> (t & 16)) & 0xffffu) - 1, 0);
+                // the centre with the largest cosine (the lowest cluster for a row of NaN), or (upper half) all those that may have it
+                const unsigned near = (__ballot_sync(0xffffffffu, j < K && cs >= best - KM_NEAR) >> (t & 16)) & 0xffffu;
+                const int bj = max(__ffs(near) - 1, 0);
                 if (w < w_hi) {
                     if (j == 0) labels[w] = bj;
-                    if (j < KM_CL) {
-                        const uint32_t dst = dsmem_addr((uint32_t)__cvta_generic_to_shared(lab + w), j);
-                        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(dst), "r"(bj) : "memory");
-                    }
+                    if (j < KM_CL) km_push(lab + w, __popc(near) > 1 ? (int)(near << 16) : bj, j);
                 }
             }
             km_cluster_sync();
+            // ---- rows with several such centres (the same ones in every CTA): their products in 64 bits
+            const bool any_near = __syncthreads_or(t < W && (lab[min(t, W - 1)] & 0xffff0000) != 0) != 0;
+            if (any_near) {
+                if (rk < n_rk) {
+                    for (int w = warp; w < W; w += nw) {
+                        const int o = w / per;
+                        for (unsigned m = (unsigned)lab[w] >> 16; m; m &= m - 1) {
+                            const int j = __ffs(m) - 1;
+                            const double dot = km_dot(row(w) + c_lo, Cs + (size_t)j * dper, cols, lane);
+                            if (lane == 0) km_push(recv_64 + ((size_t)rk * per + (w - o * per)) * K + j, dot, o);
+                        }
+                    }
+                    if (warp < K) {
+                        const double n2 = km_dot(Cs + (size_t)warp * dper, Cs + (size_t)warp * dper, cols, lane);
+                        if (lane < KM_CL) km_push(&c2_64[rk][warp], n2, lane);
+                    }
+                }
+                km_cluster_sync();
+                for (int w0 = w_lo; w0 < w_hi; w0 += KM_THREADS / 16) {
+                    const int w = w0 + (t >> 4), j = t & 15;
+                    const unsigned near = w < w_hi ? (unsigned)lab[w] >> 16 : 0u;
+                    double cs = -INFINITY;
+                    if ((near >> j) & 1) {
+                        double dot = 0., n2 = 0.;
+                        for (int r = 0; r < n_rk; ++r) { dot += recv_64[((size_t)r * per + (w - w_lo)) * K + j]; n2 += c2_64[r][j]; }
+                        cs = n2 > 0. ? dot / sqrt(n2) * invn[w] : 0.;
+                    }
+                    double best = cs;
+#pragma unroll
+                    for (int o = 1; o < 16; o <<= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+                    // (lowest cluster on ties)
+                    const unsigned tie = (__ballot_sync(0xffffffffu, ((near >> j) & 1) && cs >= best - KM_TIE) >> (t & 16)) & 0xffffu;
+                    const int bj = max(__ffs(tie) - 1, 0);
+                    if (near) {
+                        if (j == 0) labels[w] = bj;
+                        if (j < KM_CL) km_push(lab + w, bj, j);
+                    }
+                }
+                km_cluster_sync();
+            }
             if (it + 1 == a.iters) break;          // the centres of the last update are never used
             // ---- update of this CTA's columns: members added in ascending row order; an empty cluster keeps its centre
             group_rows();
