@@ -432,7 +432,10 @@ attention_flash_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
                 m = tm;
             } else if (__builtin_expect(__any_sync(0xffffffffu, tm > m + FL_SLACK), 0)) {
                 // (the P V of the previous tile has completed: it was issued in front of the scores just read)
-                const float nm = fmaxf(m, tm), al = nm == -INFINITY ? 1.f : ex2(m - nm);
+                // Decided row by row: a row's bits must not hang on the rows that share its warp, or one that has not changed would
+                // drift when it is measured in other company (a block entry's rows, then a refresh step's).
+                const bool up = tm > m + FL_SLACK;
+                const float nm = up ? tm : m, al = up ? ex2(m - nm) : 1.f;
                 l *= al;
                 A2[0] = f2_mul(A2[0], f2_pack(al, al)); A2[1] = f2_mul(A2[1], f2_pack(al, al));
                 m = nm;

@@ -146,6 +146,26 @@ def check_attention(dtype, R, N, nh, nkv, dh, prev_off=0, out_off=0):
         assert (d_out <= M * np.sqrt(2 * np.maximum(kl.cpu().numpy()[:, h], 0)) + 1e-3).all()
 
 
+@pytest.mark.parametrize("N,nh,nkv", [(512, 2, 2), (900, 4, 1), (1101, 2, 1)])
+def test_attention_drift_of_unchanged_rows_in_other_company(monkeypatch, N, nh, nkv):
+    # Rows whose running maximum moves far (by more than 2^8 between key tiles) among rows whose maximum moves a little; then the same
+    # rows sorted by kind, without the last of each: none of them has changed, so every drift is exactly zero.
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", "10")
+    Bd.polestar_reload_env()
+    R, dh = 96, 128
+    far = torch.arange(R) % 3 == 0
+    q = (rnd((R, nh * dh), 1, 1.0) * torch.where(far, 5.0, 0.3)[:, None]).to(torch.bfloat16).cuda()
+    k = (rnd((N, nkv * dh), 2, 1.0) * torch.where(torch.arange(N) < 256, 1.0, 3.0)[:, None]).to(torch.bfloat16).cuda()
+    v = rnd((N, nkv * dh), 3, 1.0, torch.bfloat16).cuda()
+    prev, lse = torch.zeros((R, nh, N), device="cuda"), torch.zeros((R, nh), device="cuda")
+    kl = torch.full((R, nh), -1.0, device="cuda")
+    Bd.polestar_k_attention(q, k, v, prev, lse, kl, None, nh, nkv, dh)
+    rows = torch.cat([torch.nonzero(~far)[:-1, 0], torch.nonzero(far)[:-1, 0]]).cuda()
+    kl = torch.full((len(rows), nh), -1.0, device="cuda")
+    Bd.polestar_k_attention(q[rows].contiguous(), k, v, prev[rows].contiguous(), lse[rows].contiguous(), kl, None, nh, nkv, dh)
+    assert (kl == 0).all()
+
+
 def test_attention_without_recording():
     R, N, nh, dh = 20, 96, 2, 128
     q = rnd((R, nh * dh), 1, 1.0, torch.bfloat16).cuda()
