@@ -1698,10 +1698,11 @@ __global__ void build_head_list_kernel(StepDesc sd, const int* y, int mask_id, c
 // scratch in global memory.
 //
 // Few rows are a latency chain (loads, running maximum, combination), many are bound by the read.  Every thread has CONF_U
-// 16-byte loads in flight and takes one rescaling and independent exponentials per batch; the vocabulary need not be a multiple
+// 16-byte loads in flight and takes one rescaling and independent exponentials (expf: with __expf, 7 - 8 % faster, a term's error grows with
+// its distance from the maximum) per batch; the vocabulary need not be a multiple
 // of four.  us, against 32 chunks of a row in blocks of their own, a rescaling per 16 bytes (single floats in the second) and
-// a second launch that combined them: 32 rows x 126464 9.7 -> 7.4, 64 x 50258 14.0 -> 7.3, 512 x 126464 84 -> 53 (4.9 TB/s),
-// 512 x 2000 32 -> 4.4.
+// a second launch that combined them: 32 rows x 126464 8.9 -> 7.6, 64 x 50258 13.9 -> 7.5, 512 x 126464 78 -> 55 (4.7 TB/s),
+// 512 x 2000 35 -> 4.5.
 // ---------------------------------------------------------------------------------------
 struct ConfPart { float mx_all; float sum; float mx_ex; int arg_ex; };
 constexpr int CONF_CL = 8, CONF_MAX_THREADS = 512, CONF_U = 4;
@@ -1727,8 +1728,8 @@ struct ConfRun {
         const float nm = fmaxf(mx, m), ref = nm == -INFINITY ? 0.f : nm;
         float s = 0.f;
 #pragma unroll
-        for (int u = 0; u < CONF_U; ++u) s += (__expf(x[u].x - ref) + __expf(x[u].y - ref)) + (__expf(x[u].z - ref) + __expf(x[u].w - ref));
-        sum = sum * __expf(mx - ref) + s;
+        for (int u = 0; u < CONF_U; ++u) s += (expf(x[u].x - ref) + expf(x[u].y - ref)) + (expf(x[u].z - ref) + expf(x[u].w - ref));
+        sum = sum * expf(mx - ref) + s;
         mx = nm;
 #pragma unroll
         for (int u = 0; u < CONF_U; ++u) {

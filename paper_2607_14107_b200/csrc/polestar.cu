@@ -385,9 +385,11 @@ static int norm_threads(int rows, int d, int proxies = 0) {
 // Confidence of `rows` logits rows (of *m_count of them, when given).
 static cudaError_t launch_confidence(const float* logits, const int* m_count, int rows, int vocab, int mask_id, int* yhat, float* conf,
                                      cudaStream_t st, int sms) {
-    // Threads per row: at least a batch of loads each, as long as all rows together do not exceed what the GPU holds at once
-    // (1776 threads per SM); in CTAs of 128 to 512, up to eight of them.  us at 4096 / 2048 / 1024 / 512 threads per row: 32 x 126464
-    // 7.4 / 9.9 / 13.7 / 19, 512 x 126464 100 / 63 / 57 / 53, 64 x 50258 9.1 / 7.3 / 8.8 / 12; 512 x 2000 128 4.4, 512 7.1.
+    // Threads per row: at least a batch of loads each, in CTAs of 128 to 512, up to eight of them; all rows together up to 1776 threads
+    // per SM.  That is more than an SM holds at once (1024 at 64 registers): best at few rows and at hundreds, 10 - 25 % slow at 48, 64 and
+    // 128 rows, which start a second wave.  us at 4096 / 2048 / 1024 / 512 threads per row: 32 x 126464 7.6 / 9.7 / 16.0 / 20, 64 x 126464
+    // 14.0 / 11.1 / 16.4 / 30, 128 x 126464 26 / 20.3 / 18.4 / 31, 512 x 126464 93 / 68 / 60 / 55, 64 x 50258 9.9 / 7.5 / 9.0 / 14; 512 x 2000
+    // 128 4.5, 512 8.0.
     const long long most = std::min<long long>(vocab / 16, 1776LL * sms / rows);
     int per_row = 128;
     while (per_row < CONF_CL * CONF_MAX_THREADS && 2 * per_row <= most) per_row *= 2;

@@ -466,6 +466,26 @@ def test_confidence_rows_at_any_alignment(rows, V):
     assert torch.allclose(conf.cpu().double(), want, rtol=2e-5, atol=0)          # as above
 
 
+def test_confidence_of_many_small_terms():
+    # Rows of 128 zeros, one in front of every thread's share, and equal terms e^-x that make up most of the sum.  An exponential by a power
+    # of two of the rounded product x log2(e) would be off by 0.4 to 0.5 spacings of that product, 2^-20, in every term of these rows and to the
+    # same side: 1.5e-7 and more in the mean.  One good to its last place errs to either side: below 2^-24 over the rows.
+    V, rows = 126464, 2048
+    x = np.linspace(5.6, 7.0, 40000).astype(np.float32)
+    prod = x.astype(np.float64) * np.float64(np.float32(math.log2(math.e)))
+    x = x[(prod.astype(np.float32).astype(np.float64) - prod) / 2.0 ** -20 > 0.4]
+    x = x[np.linspace(0, len(x) - 1, rows).astype(int)]
+    logits = torch.empty((rows, V), device="cuda").copy_(torch.from_numpy(-x)[:, None])
+    logits[:, 0:512:4] = 0.0
+    yhat = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+    conf = torch.zeros(rows, device="cuda")
+    Bd.polestar_k_confidence(logits, 3, yhat, conf, torch.empty(rows * 512, dtype=torch.uint8, device="cuda"))
+    want = 1.0 / (128.0 + (V - 128) * np.exp(-x.astype(np.float64)))
+    err = conf.cpu().double().numpy() / want - 1.0
+    assert (yhat == 0).all()
+    assert np.abs(err).max() < 2e-5 and abs(err.mean()) < 2.0 ** -24, (np.abs(err).max(), err.mean())      # (fp32 sums: as above)
+
+
 # ------------------------------------------------------------------ empty inputs
 def test_empty_inputs_are_noops():
     dev = "cuda"
