@@ -156,10 +156,19 @@ def attn_logp_rows(q: np.ndarray, K: np.ndarray, rowwise: bool = False) -> np.nd
     return logp
 
 
-def attn_out_rows(logp: np.ndarray, V: np.ndarray, round_p=_ident, rowwise: bool = False) -> np.ndarray:
-    """o = sum_j p_j v_j per head.  logp [R, n_h, N], V [N, n_kv, dh] -> [R, n_h*dh]."""
+def attn_out_rows(logp: np.ndarray, V: np.ndarray, round_p=_ident, rowwise: bool = False,
+                  lse: Optional[np.ndarray] = None) -> np.ndarray:
+    """o = sum_j p_j v_j per head.  logp [R, n_h, N], V [N, n_kv, dh] -> [R, n_h*dh].
+
+    The probabilities are rounded as they are, or, with the rows' log-sum-exps ``lse`` [R, n_h], before they are
+    normalised: o = sum_j round(exp(s_j)) v_j / sum_j exp(s_j) with the scores s_j = logp_j + lse (up to a power of
+    two, which does not matter to the rounding)."""
     R, nh, N = logp.shape
     V = np.asarray(V, F64)
+    if lse is not None:
+        frac = (lse / math.log(2.0)) % 1.0              # exp(s) = 2^(integer + frac) p
+        logp = logp + (frac * math.log(2.0))[:, :, None]
+        return (attn_out_rows(logp, V, round_p, rowwise).reshape(R, nh, -1) / np.exp2(frac)[:, :, None]).reshape(R, -1)
     nkv, dh = V.shape[1], V.shape[2]
     o = np.empty((R, nh, dh), F64)
     for h in range(nh):
@@ -425,6 +434,9 @@ class _Seq:
         emu = (m.dtype == 1) if emulate_bf16 is None else emulate_bf16
         self.rnd = bf16_round if emu else _ident
         self.N = p.prompt_len + p.gen_len
+        # where bf16 models round the attention probabilities: normalised ones over up to 512 keys, beyond that (heads of
+        # 128) before they are normalised
+        self.normalised_p = not (emu and m.head_dim == 128 and self.N > 512)
         self.y = np.concatenate([np.asarray(prompt, np.int64),
                                  np.full(p.gen_len, m.mask_id, np.int64)])
         L = m.n_layers
@@ -458,11 +470,15 @@ class _Seq:
         k = rnd(rope(k, pos, m.rope_theta))
         return q, k, rnd(v)
 
-    def _finish(self, l, x, logp):
-        """Rest of layer l for rows x with attention rows logp: attention output,
+    def _finish(self, l, x, logp, q):
+        """Rest of layer l for rows x with queries q and attention rows logp: attention output,
         output projection + residual, SwiGLU FFN + residual."""
         m, wl, rnd = self.m, self.w["layers"][l], self.rnd
-        o = rnd(attn_out_rows(logp, self.Vc[l], rnd, self.rowwise))
+        lse = None
+        if not self.normalised_p:
+            heads = (np.arange(m.n_heads) * m.n_kv_heads) // m.n_heads
+            lse = np.einsum("rhd,hd->rh", q, self.Kc[l][0][heads]) / math.sqrt(m.head_dim) - logp[:, :, 0]
+        o = rnd(attn_out_rows(logp, self.Vc[l], rnd, self.rowwise, lse))
         x1 = x + linear(o, wl["wo"], self.rowwise)
         f = rnd(rmsnorm(x1, wl["norm2"], m.rms_eps))
         g = rnd(silu(linear(f, wl["wg"], self.rowwise)) * linear(f, wl["wu"], self.rowwise))
@@ -519,7 +535,7 @@ class _Seq:
                 self.Pprev[l] = logp[wi].copy()
             if l == m.n_layers - 1:
                 self.Aprev = logp[ai].copy()
-            x = self._finish(l, x, logp)
+            x = self._finish(l, x, logp, q)
         tr["labels"] = [None if a is None else a.copy() for a in self.labels]
         tr["x_act"].append(x[ai].copy())
         self.tok_at_h0 = self.y[win].copy()
@@ -577,7 +593,7 @@ class _Seq:
             if l == L - 1:
                 self.delta = kl_rows(logpA, self.Aprev)
                 self.Aprev = logpA.copy()
-            x = self._finish(l, x, logpA)
+            x = self._finish(l, x, logpA, q)
             # 3. drift of the window rows, selection, sparse forward -> next packet
             if refresh and p.select_mode == SELECT_CLUSTER_TOPK:
                 # proxy attention of the centroids, drift per cluster, top-k clusters -> their member rows
@@ -604,7 +620,7 @@ class _Seq:
                     # the selected rows' own attention rows (each row's query from its cached hidden state)
                     qs, _, _ = self._qkv(l, self.Hc[l][S], win[S])
                     Ps = attn_logp_rows(qs, self.Kc[l], self.rowwise)
-                    U_val = self._finish(l, self.Hc[l][S], Ps)
+                    U_val = self._finish(l, self.Hc[l][S], Ps, qs)
                 else:
                     U_val = np.zeros((0, m.d_model), F64)
             elif refresh:
@@ -620,7 +636,7 @@ class _Seq:
                 tr["D"].append(D)
                 tr["sel"].append(S)
                 U_idx = S
-                U_val = self._finish(l, self.Hc[l][S], P[S]) if len(S) else np.zeros((0, m.d_model), F64)
+                U_val = self._finish(l, self.Hc[l][S], P[S], qw[S]) if len(S) else np.zeros((0, m.d_model), F64)
             else:
                 tr["D"].append(None)
                 tr["sel"].append(np.zeros(0, np.int64))

@@ -10,7 +10,8 @@
 //            scores, keep a running maximum m and sum, and write p = 2^(s - m), rounded to bf16, over the scores, where it is the A
 //            operand of O += P V.  Output rows are divided by the sum at the end.  m follows the true maximum only when that has
 //            grown by more than 2^8 (the row's O, sum and drift sum are then rescaled): the scale of p does not matter to its
-//            rounding, and after the first tile it hardly ever moves
+//            rounding, and after the first tile it hardly ever moves.  In forwards m is a whole number (AttnArgs::p_pow2): the rounding of
+//            p is then that of e^score on its own, whatever the order of the tiles, and the oracle's
 //   drift    A = sum p (s - s_old) is accumulated and rescaled like the sum; KL = A / sum - (lse - lse_old), exactly zero for an
 //            unchanged row (s - s_old and lse - lse_old are: same bits in, same bits out)
 //   stored   the stored rows (scaled scores plus one log-sum-exp, as in attn_tc.cuh) pass through two staging patches of [32
@@ -427,7 +428,8 @@ attention_flash_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_c
                 top(ra, rb, 0);
                 top(rc, rd, 2);
             }
-            const float tm = fmaxf(fmaxf(tm4[0], tm4[1]), fmaxf(tm4[2], tm4[3])) * scale2;      // scale2 > 0: the maximum commutes with it
+            float tm = fmaxf(fmaxf(tm4[0], tm4[1]), fmaxf(tm4[2], tm4[3])) * scale2;      // scale2 > 0: the maximum commutes with it
+            if (a.p_pow2) tm = ceilf(tm);
             if (k == 0) {
                 m = tm;
             } else if (__builtin_expect(__any_sync(0xffffffffu, tm > m + FL_SLACK), 0)) {

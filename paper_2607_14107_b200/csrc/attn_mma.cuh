@@ -546,6 +546,8 @@ __global__ void __launch_bounds__(NW * 32) attention_sp_kernel(AttnMmaArgs g) {
     }
     __syncthreads();
     const float lse_lo = lse_sh[r_lo], lse_hi = lse_sh[r_hi];
+    const float ref_lo = a.p_pow2 ? ceilf(lse_lo) : lse_lo, ref_hi = a.p_pow2 ? ceilf(lse_hi) : lse_hi;
+    const float norm_lo = a.p_pow2 ? fast_exp2(ref_lo - lse_lo) : 1.f, norm_hi = a.p_pow2 ? fast_exp2(ref_hi - lse_hi) : 1.f;
     float* prev_lo = prev_sh[r_lo];
     float* prev_hi = prev_sh[r_hi];
     const bool vec = g.vec != 0;
@@ -587,7 +589,7 @@ __global__ void __launch_bounds__(NW * 32) attention_sp_kernel(AttnMmaArgs g) {
                 for (int e = 0; e < 2; ++e) {
                     const bool ok = t * AT_BN + nt * 8 + cpair + e < a.N;
                     const float d_lo = s[i][nt][e] - lse_lo, d_hi = s[i][nt][2 + e] - lse_hi;
-                    const float p_lo = ok ? fast_exp2(d_lo) : 0.f, p_hi = ok ? fast_exp2(d_hi) : 0.f;
+                    const float p_lo = ok ? fast_exp2(s[i][nt][e] - ref_lo) : 0.f, p_hi = ok ? fast_exp2(s[i][nt][2 + e] - ref_hi) : 0.f;
                     lp_lo[nt][e] = d_lo * LN2; lp_hi[nt][e] = d_hi * LN2;       // natural-log probabilities
                     if (ok && a.record_kl) {
                         if (prev_lo) kl_lo += p_lo * (lp_lo[nt][e] - pv_lo[nt][e]);
@@ -634,6 +636,7 @@ __global__ void __launch_bounds__(NW * 32) attention_sp_kernel(AttnMmaArgs g) {
         }
     }
     // ---- combine the warps' partial results (fixed order) ---------------------------------------
+    kl_lo *= norm_lo; kl_hi *= norm_hi;
     kl_lo += __shfl_xor_sync(0xffffffffu, kl_lo, 1); kl_lo += __shfl_xor_sync(0xffffffffu, kl_lo, 2);
     kl_hi += __shfl_xor_sync(0xffffffffu, kl_hi, 1); kl_hi += __shfl_xor_sync(0xffffffffu, kl_hi, 2);
     if ((lane & 3) == 0) { red_kl[warp][r_lo] = kl_lo; red_kl[warp][r_hi] = kl_hi; }
@@ -643,8 +646,8 @@ __global__ void __launch_bounds__(NW * 32) attention_sp_kernel(AttnMmaArgs g) {
 #pragma unroll
         for (int nt = 0; nt < 16; ++nt) {
             const int col = nt * 8 + cpair;
-            *reinterpret_cast<float2*>(o_s + ((size_t)warp * AT_BM + r_lo) * AT_DH + col) = make_float2(o[nt][0], o[nt][1]);
-            *reinterpret_cast<float2*>(o_s + ((size_t)warp * AT_BM + r_hi) * AT_DH + col) = make_float2(o[nt][2], o[nt][3]);
+            *reinterpret_cast<float2*>(o_s + ((size_t)warp * AT_BM + r_lo) * AT_DH + col) = make_float2(o[nt][0] * norm_lo, o[nt][1] * norm_lo);
+            *reinterpret_cast<float2*>(o_s + ((size_t)warp * AT_BM + r_hi) * AT_DH + col) = make_float2(o[nt][2] * norm_hi, o[nt][3] * norm_hi);
         }
     }
     __syncthreads();

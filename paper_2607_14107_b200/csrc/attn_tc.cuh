@@ -416,6 +416,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             }
             lse2 = M + log2f(L);
         }
+        const float ref = a.p_pow2 ? ceilf(lse2) : lse2, norm = a.p_pow2 ? ex2(ref - lse2) : 1.f;
         if (owns) {
             // the owner of a row keeps its log-sum-exp (natural-log units, like the stored rows)
             float* lsep = lsep_sh[row];
@@ -424,7 +425,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             if (lsep && valid) *lsep = lse;
         }
         dbg_clock(8);
-        // pass B: probabilities (normalised before they are rounded to bf16), drift sum, the new stored row, P
+        // pass B: probabilities (normalised before they are rounded to bf16, but for p_pow2), drift sum, the new stored row, P
         float A = 0.f;
         for (int j = 0; j < n_kt; ++j) {
             if (ok && warp_valid) {
@@ -444,7 +445,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                         const bool in = valid && (k16 + i < a.N);
                         const float t = __fmul_rn(__uint_as_float(r[u][i]), scale2);     // (rounded products, never fused into the
                                                                                          // subtraction from the stored value below)
-                        const float p = in ? ex2(t - lse2) : 0.f;      // rows that are not valid hand zeros to the tensor core
+                        const float p = in ? ex2(t - ref) : 0.f;       // rows that are not valid hand zeros to the tensor core
                         s_nat[i] = __fmul_rn(t, LN2_F);
                         if (use_old && in) A = fmaf(p, s_nat[i] - old[16 * u + i], A);
                         pr[i] = p;
@@ -499,10 +500,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int chunk = half * 16 + 4 * u + i;
-                    *reinterpret_cast<uint4*>(dst + ((chunk ^ (lrow & 31)) << 2)) = make_uint4(r[u][4 * i], r[u][4 * i + 1], r[u][4 * i + 2], r[u][4 * i + 3]);
+                    *reinterpret_cast<float4*>(dst + ((chunk ^ (lrow & 31)) << 2)) =
+                        make_float4(__uint_as_float(r[u][4 * i]) * norm, __uint_as_float(r[u][4 * i + 1]) * norm, __uint_as_float(r[u][4 * i + 2]) * norm,
+                                    __uint_as_float(r[u][4 * i + 3]) * norm);
                 }
         }
-        st_p[(size_t)row * OROW + DH + half] = A;
+        st_p[(size_t)row * OROW + DH + half] = A * norm;
         tc_fence_before();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the bulk copies read what was just written
         bar_sync_epi();

@@ -1086,6 +1086,8 @@ struct AttnArgs {
     int N, n_heads, n_kv, head_dim, W_max, B, record_kl;
     int rows_per_seq, batch;   // layout of the forward's rows (stand-alone: n_rows, 1)
     float scale;
+    int p_pow2;                // round exp(score) to bf16 times a power of two (any: it does not matter to the rounding) instead of the normalised
+                               // probability, and normalise in fp32 behind P V: what a kernel that sees every key once can do
     int cluster_K;             // > 0: centroid proxies: pprev / pprev_lse hold [batch][cluster_K] proxy rows per head and
                                // window rows are not recorded
     int rec_lo, rec_hi;        // rows [lo, hi) of every sequence hold all the recorded ones (hi 0: any row may be recorded)

@@ -528,11 +528,11 @@ static bool attention_prefers_stream(const AttnArgs& a, const AttnClusters& resi
     return (double)((tiles + at_once - 1) / at_once) * wave > (drift ? 10 + 4 * key_tiles : 8 + 2 * key_tiles);
 }
 // Which tensor-core kernel: the two-stream one, but for
-//  - forwards over up to 512 keys: they stay with the two kernels that round the NORMALISED probabilities to bf16, as a plain
-//    implementation does.  The two-stream kernel's roundings are as fine (relative error of the output rows against 64 bits, 128 x
-//    512 x 32 2.13e-3 / 2.35e-3, 300 x 2000 x 8 2.29e-3 / 2.35e-3, scores of spread 9 1.74e-3 / 2.11e-3) but fall elsewhere, and over the
-//    layers of an 8B-width model that difference takes the margin to a forward that rounds like a plain one: 6.8 % instead of
-//    3.5 % of the hidden values beyond 2e-2 after two layers at 160 keys.  At these sizes it would save 1 - 4 us a layer;
+//  - forwards over up to ATTN_NORMALISED_KEYS keys: there the bf16 probabilities of P V are rounded after the normalisation, which takes
+//    a first look at all keys; beyond, in every kernel, before it (AttnArgs::p_pow2), so that one pass is enough.  Either rounding is a bf16
+//    model's; but one kernel's forwards against another's, or against an oracle that rounds where the other does, would be off by both: 6.5 %
+//    instead of 3.0 % of the hidden values beyond 2e-2 after two layers of the 8B widths.  The line lies where one pass starts to pay: at
+//    512 keys it would save 1 - 4 of ~20 us a layer, at 128 rows x 1024 keys x 28 heads on 4 it is 30 against 41;
 //  - a single key tile, which leaves one of its streams idle: the streaming kernel (us, two-stream / streaming: 32 rows x 96 keys
 //    x 32 heads with stored rows 9.5 / 7.9, 28 heads on 4 11.4 / 8.3, without 12.2 / 7.0);
 //  - few (row tile, head) pairs with many keys, where the cluster kernel spreads the keys over SMs: by their estimated times, fitted
@@ -540,9 +540,10 @@ static bool attention_prefers_stream(const AttnArgs& a, const AttnClusters& resi
 //    resident clusters x (start + its rows' share of the stored rows; `kt` key tiles per CTA).  us, two-stream / cluster with stored
 //    rows: 8 heads, 128 x 2000 49 / 35, 128 x 1200 32 / 34, 4 heads on 1, 64 x 2048 49 / 23, 28 on 4, 32 x 512 18 / 14, 128 x 1024 30 / 41,
 //    32 / 32 heads 128 x 512 18 / 19, 1 x 1501 (rows of no whole 16 bytes) 53 / 39, 64 x 1501 58 / 105.
+constexpr int ATTN_NORMALISED_KEYS = 512;
 enum AttnForm { ATTN_FLASH, ATTN_STREAM, ATTN_CLUSTER };
 static AttnForm attention_form(const AttnArgs& a, const AttnClusters& resident, int sms) {
-    if (a.rows && a.N <= 512) return attention_prefers_stream(a, resident) ? ATTN_STREAM : ATTN_CLUSTER;
+    if (a.rows && a.N <= ATTN_NORMALISED_KEYS) return attention_prefers_stream(a, resident) ? ATTN_STREAM : ATTN_CLUSTER;
     if (a.N <= ast::KEYS) return ATTN_STREAM;
     if (!attention_tc_applies(a)) return ATTN_FLASH;
     const FlashPlan f = flash_plan(a, sms);
@@ -1128,6 +1129,7 @@ struct Path {
                 a.kl = b.kl; a.N = N; a.n_heads = m.n_heads; a.n_kv = m.n_kv_heads; a.head_dim = m.head_dim;
                 a.W_max = Wm; a.B = B; a.record_kl = sd.record_kl; a.rows_per_seq = sd.rows_per_seq; a.batch = bs;
                 a.scale = 1.0f / sqrtf((float)m.head_dim);
+                a.p_pow2 = N > ATTN_NORMALISED_KEYS;
                 // rows that may be recorded: the window rows, among which an entry step has the active block, or the proxy rows;
                 // and in the last layer the active rows
                 if (within) { a.rec_lo = last ? 0 : B; a.rec_hi = B + sd.W; }

@@ -97,6 +97,26 @@ def test_attention_transposed_operand_would_fail():
     assert np.allclose(O.attn_logp_rows(q, K)[0, 0], ref, atol=1e-14)
 
 
+@pytest.mark.parametrize("spread", [0.3, 3.0])
+def test_probabilities_rounded_before_they_are_normalised(spread):
+    # o = sum round(e^s) v / sum e^s, element by element; any power of two in front of e^s gives the same rows
+    rng = np.random.default_rng(5)
+    q, K, V = rng.standard_normal((3, 4, 8)) * spread, rng.standard_normal((50, 2, 8)), rng.standard_normal((50, 2, 8))
+    logp = O.attn_logp_rows(q, K)
+    s = np.einsum("rhd,nhd->rhn", q, np.repeat(K, 2, axis=1)) / math.sqrt(8)
+    lse = np.log(np.exp(s).sum(-1))
+    want = np.empty((3, 4, 8))
+    for r in range(3):
+        for h in range(4):
+            want[r, h] = sum(O.bf16_round(np.exp(s[r, h, j])) * V[j, h // 2] for j in range(50)) / np.exp(s[r, h]).sum()
+    out = O.attn_out_rows(logp, V, O.bf16_round, lse=lse)
+    assert np.allclose(out, want.reshape(3, 32), atol=1e-12)
+    assert np.allclose(O.attn_out_rows(logp, V, O.bf16_round, lse=lse + 7 * math.log(2.0)), out, atol=1e-12)
+    plain = O.attn_out_rows(logp, V)
+    assert np.allclose(O.attn_out_rows(logp, V, lse=lse), plain, atol=1e-12)
+    assert 0 < np.abs(out - plain).max() < 2.0 ** -8 * np.abs(V).max()         # either rounding: half a bf16 spacing of each term
+
+
 # ---------------------------------------------------------------- KL drift (Eq. 4)
 def test_kl_closed_forms():
     for line in _read("kl.txt"):
