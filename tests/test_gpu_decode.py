@@ -313,10 +313,10 @@ def test_c1b_bf16_norm_staging_inside_the_gemm_tail(monkeypatch):
     assert seen["refresh"] > 3
 
 
-@pytest.mark.parametrize("variant", ["0", "5", "9"])
+@pytest.mark.parametrize("variant", ["0", "5", "9", "10"])
 def test_c1b_long_ragged_sequence(monkeypatch, variant):
-    # N = 1100 + 64 > 1024 keys: the two-pass attention kernel (automatic choice) and the 64-row-tile kernel
-    # (forced) inside the decoding loop; the prompt length is not a multiple of the block size
+    # N = 1100 + 64 > 1024 keys: the automatic choice (two-stream and cluster kernel), the 64-row-tile, the streaming and the
+    # two-stream kernel inside the decoding loop; the prompt length is not a multiple of the block size
     monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
     seen = run_forced("c1b", 5, prompt_len=1100, gen_len=64, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5)
     assert seen["refresh"] >= 2
@@ -344,23 +344,30 @@ def test_c1b_bf16_separate_launches(monkeypatch):
     assert seen["refresh"] > 3
 
 
-@pytest.mark.parametrize("kw", [
-    dict(tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=3),
-    dict(tau_upd=-1, logit_scale=24.0, tau_suffix=0.5, batch=2, select_mode=I.SELECT_CLUSTER_TOPK, n_clusters=5, cluster_k=2),
+GQA = dict(n_heads=8, n_kv_heads=2)
+
+
+@pytest.mark.parametrize("variant,kw", [
+    ("9", dict(tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=3)),
+    ("9", dict(tau_upd=-1, logit_scale=24.0, tau_suffix=0.5, batch=2, select_mode=I.SELECT_CLUSTER_TOPK, n_clusters=5, cluster_k=2)),
+    ("10", dict(tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=3)),
+    ("10", dict(tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=2, model=GQA, prompt_len=160)),
 ])
-def test_c1b_streaming_attention_kernel(monkeypatch, kw):
-    # the streaming tensor-core attention kernel (one CTA per row tile and head, two passes over the key tiles) on every
-    # step of a decode: block entries (recorded rows), plain steps, refresh steps with stored rows / proxy rows
-    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", "9")
+def test_c1b_streaming_attention_kernel(monkeypatch, variant, kw):
+    # the streaming tensor-core attention kernel (one CTA per row tile and head, two passes over the key tiles) and the two-stream
+    # one on every step of a decode: block entries (recorded rows in CTAs of their own), plain steps, refresh steps with
+    # stored rows / proxy rows (of the two-stream kernel: below), grouped heads
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
     seen = run_forced("c1b", 12, **kw)
     assert seen["refresh"] > 3 and seen["entry_window"] >= 0
 
 
+@pytest.mark.parametrize("variant", ["9", "10"])
 @pytest.mark.parametrize("prompt_len", [600, 601])          # 601: rows of 673 floats, which no bulk copy takes
-def test_c1b_streaming_attention_stored_row_forms(monkeypatch, prompt_len):
+def test_c1b_streaming_attention_stored_row_forms(monkeypatch, prompt_len, variant):
     # refresh steps of 24 + 72 rows over six key tiles: the first 32 rows hold the active block's and the window's stored
     # rows (row copies in the last layer, a partly recorded quarter in the others), the other quarters tensor boxes
-    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", "9")
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
     seen = run_forced("c1b", 8, tau_upd=-1, logit_scale=24.0, alpha=0.001, tau_suffix=0.5, batch=2, prompt_len=prompt_len, gen_len=72, block=24,
                       max_steps=24)
     assert seen["refresh"] > 3
@@ -386,9 +393,23 @@ def test_c1b_wide_windows(pre, suf):
     assert seen["refresh"] > 3 and seen["entry_window"] > 0
 
 
-def test_c1b_batch_of_long_sequences_plain_steps():
-    # 19 sequences x 8 heads fill the GPU's SMs, more than 1024 keys, 64-row blocks: the layers of a plain step that record
-    # nothing take the 64-row warp-level attention kernel, the last layer and the refresh steps the streaming kernel
+@pytest.mark.parametrize("variant", ["0", "10"])
+@pytest.mark.parametrize("prompt_len", [616, 603])          # 603: rows of 667 floats
+def test_c1b_centroid_proxies_over_more_than_512_keys(monkeypatch, prompt_len, variant):
+    # the kernel that is chosen there, the two-stream one, with proxy rows as the recorded rows: block entries (684 rows a sequence, in
+    # whose last layer the active block is recorded too) and refresh steps (32 + 96 + 4 rows), grouped heads
+    # (initialised so that the cosines of the first entry's own clusters differ by more than bf16 moves them: 1e-4 and more)
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
+    seen = run_forced("c1b", 9, std=0.05, select_mode=I.SELECT_CLUSTER_TOPK, model=GQA, batch=4, n_clusters=4, cluster_k=2, prompt_len=prompt_len,
+                      tau_upd=-1, logit_scale=8.0, tau_suffix=0.5, max_steps=8)
+    assert seen["refresh"] > 3 and seen["clusterings"] > 4, seen
+
+
+@pytest.mark.parametrize("variant", ["0", "5"])
+def test_c1b_batch_of_long_sequences_plain_steps(monkeypatch, variant):
+    # 19 sequences x 8 heads, more than 1024 keys, 64-row blocks: the two-stream kernel in every step (with more (sequence, head)
+    # pairs than half of the SMs plain steps have no warp-level kernel), and the 64-row warp-level kernel
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
     seen = run_forced("c1b", 7, model=dict(d_model=1024, n_heads=8, n_kv_heads=8), batch=19, prompt_len=1040, gen_len=64, block=64,
                       max_steps=16, tau_upd=5, logit_scale=12.0, alpha=0.001, tau_suffix=0.5)
     assert seen["within"] > seen["refresh"] > 0

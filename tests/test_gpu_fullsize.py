@@ -183,8 +183,8 @@ def test_c3_widths_gqa_batch_matches_oracle():
 def test_c4_shape_reduced_depth_matches_oracle():
     # The long-generation workload's shape at depth 1: LLaDA-8B widths and vocabulary, 1024 + 1024 positions,
     # block 64 (window 192), batch 2.  With 3 steps per block and tau_upd = 25 the first forwards are: a
-    # full-sequence entry (2048 rows per sequence: multi-token-tile GEMMs, the 64-row attention kernel with
-    # recorded rows), a plain step, a refresh step (192 window rows per sequence through drift, select and the
+    # full-sequence entry (2048 rows per sequence: multi-token-tile GEMMs, the two-stream attention kernel with
+    # recorded rows in CTAs of their own), a plain step, a refresh step (192 window rows per sequence through drift, select and the
     # sparse forward) and the window entry of the next block.
     m, p = I.config("c4")
     m = I.reduced_depth(m, 1)

@@ -469,7 +469,7 @@ def test_confidence_rows_at_any_alignment(rows, V):
 def test_confidence_of_many_small_terms():
     # Rows of 128 zeros, one in front of every thread's share, and equal terms e^-x that make up most of the sum.  An exponential by a power
     # of two of the rounded product x log2(e) would be off by 0.4 to 0.5 spacings of that product, 2^-20, in every term of these rows and to the
-    # same side: 1.5e-7 and more in the mean.  One good to its last place errs to either side: below 2^-24 over the rows.
+    # same side: more than 1e-7 in the mean.  One good to its last place errs to either side: below 2^-24 over the rows.
     V, rows = 126464, 2048
     x = np.linspace(5.6, 7.0, 40000).astype(np.float32)
     prod = x.astype(np.float64) * np.float64(np.float32(math.log2(math.e)))
