@@ -28,6 +28,10 @@
 // (302 us: a third of the registers, so spills), three 32-key patches per warp (237), the tile's 128 columns unrolled (246: the
 // loop no longer fits the instruction cache; without stored rows the unrolled form is the faster one, 82 / 91).
 //
+// The method is published: a running maximum and sum in one pass (Milakov and Gimelshein, 2018) over key tiles (FlashAttention: Dao
+// et al., 2022), two row tiles whose softmax and products alternate (FlashAttention-3: Shah et al., 2024), a reference that moves only
+// when the maximum has outgrown it (FlashAttention-4: Dao et al., 2025).  Drift, stored rows, the key split and the code are this library's.
+//
 // Every mbarrier wait is bounded.
 #pragma once
 #include <type_traits>

@@ -1,6 +1,8 @@
 // Bidirectional attention rows with drift for bf16 models, head_dim 128 (Eq. 3, Eq. 4).
 //
-// Three kernels share the tile helpers below; launch_attention_mma picks one from the row and key counts:
+// Three kernels share the tile helpers below; launch_attention_mma picks one from the row and key counts.  By itself a forward takes only
+// the first (plain steps of one block of rows); the others serve stand-alone calls whose output lies at no 16-byte boundary and that the
+// cluster kernel does not take (more keys than it covers, no 8-byte boundary either), and the forced variants:
 //   attention_sp_kernel   16 query rows x 1 head per CTA, keys split over the warps, scores kept in registers
 //                         (N <= 1024): K is read once.  With a single block of rows the keys of a (row tile, head)
 //                         are further split over a cluster of two CTAs.

@@ -251,13 +251,13 @@ static int launch_gemm_simt(const void* A, const void* W, int M, int N_out, int 
     if constexpr (sizeof(T) == 4) {
         // fp32: the K-split kernel wherever its 16-byte loads apply
         if (K % 4 == 0 && ((((uintptr_t)A | (uintptr_t)W)) & 15) == 0 && (M + LAT_TM - 1) / LAT_TM <= 65535) {
-            // A cluster of CTAs over K while the tiles fill less than half of the SMs and every CTA keeps four slices, the ring's
+            // A cluster of CTAs over K, doubled while there is at most one CTA per SM and every CTA keeps four slices, the ring's
             // worth of one round trip: 32 x 256 x 1024 in the pipeline 10.2 -> 5.7 us.
             const dim3 tiles((N_out + LAT_TN - 1) / LAT_TN, (M + LAT_TM - 1) / LAT_TM);
             const long long n_tiles = (long long)tiles.x * tiles.y;
             const int slices = (K + LAT_KC - 1) / LAT_KC;
             int cl = 1;
-            while (cl < 8 && 8 * cl <= slices && 2 * n_tiles * cl <= 2LL * sms) cl *= 2;
+            while (cl < 8 && 8 * cl <= slices && n_tiles * cl <= sms) cl *= 2;
             if (cl > 1)
                 CK(launch_k_cluster3(gemm_f32_kernel<EPI>, dim3(tiles.x, tiles.y, cl), dim3(256), (size_t)LAT_SMEM, st, dim3(1, 1, cl),
                                      (const float*)A, (const float*)W, M, N_out, K, e));
@@ -504,27 +504,26 @@ static FlashPlan flash_plan(const AttnArgs& a, int sms) {
     p.steps = o.key_split ? (n + 1) / 2 : n;
     return p;
 }
-// Which of the two kernels that normalise the probabilities before they round them.  The streaming one as soon as its grid (row tiles x heads x sequences) fills a good
-// part of the GPU -- block entries, batches (with drift, us, cluster / streaming: 256 rows x 512 keys x 32 heads 40 / 25, 512 x
-// 512 x 32 77 / 27) -- or the keys exceed what a cluster of key ranges covers.  Below that the cluster kernel, which spreads
-// the keys of a (row tile, head) over SMs, while all its clusters are resident at once: 128 x 512 x 32 21 / 24, 96 x 512 x 32
-// 19 / 23, 128 x 1200 x 8 39 / 48, 128 x 2000 x 8 41 / 73.  With more clusters than that its time is waves x one wave (13.5 +
-// 0.055 a row us with drift, 12.5 + 0.033 without; two key tiles per CTA 16.5 + 0.18 and 16.5 + 0.02), the streaming kernel's is
-// proportional to the key tiles (10 + 4 each, 8 + 2 without drift): 128 x 512 x 36 39 / 26, 128 x 1024 x 32 62 / 41, without drift
-// 48 / 25, but 40 x 1024 x 16 31 / 39, 32 x 1300 x 32 43 / 48.  (Rows that the streaming kernel can not move in 16-byte pieces stay.)
+// Which of the two kernels that see every key twice, for forwards over up to ATTN_NORMALISED_KEYS keys.  The streaming one as soon as
+// its grid (row tiles x heads x sequences) fills a good part of the GPU -- block entries, batches (with drift, us, cluster / streaming:
+// 256 rows x 512 keys x 32 heads 40 / 25, 512 x 512 x 32 77 / 27).  Below that the cluster kernel, which spreads the keys of a (row tile,
+// head) over SMs, while all its clusters are resident at once: 128 x 512 x 32 21 / 24, 96 x 512 x 32 19 / 23.  With more clusters
+// than that its time is waves x one wave (13.5 + 0.055 a row us with drift, 12.5 + 0.033 without), the streaming kernel's is
+// proportional to the key tiles (10 + 4 each, 8 + 2 without drift): 128 x 512 x 36 39 / 26.  (Rows that the streaming kernel can not
+// move in 16-byte pieces stay.)
 static bool attention_prefers_stream(const AttnArgs& a, const AttnClusters& resident) {
     const int batch = a.batch > 0 ? a.batch : 1;
     const int rps = a.rows_per_seq > 0 ? a.rows_per_seq : a.n_rows;
     const long long tiles = (long long)((rps + ast::ROWS - 1) / ast::ROWS) * batch * a.n_heads;
-    if (tiles >= 64 || a.N > atc::MAX_N) return true;
+    if (tiles >= 64) return true;
     int kt, cl;
-    attention_tc_split(a.N, &kt, &cl);
+    attention_tc_split(a.N, &kt, &cl);                     // (one key tile per CTA)
     const long long at_once = std::max(resident.n[kt - 1][cl], 1);
     if (tiles <= at_once) return false;
     const bool drift = a.pprev || a.aprev;
     if (drift && !stored_rows_in_pieces(a, 4)) return false;
     const double rows = std::min(rps, ast::ROWS), key_tiles = (a.N + ast::KEYS - 1) / ast::KEYS;
-    const double wave = drift ? (kt == 1 ? 13.5 + 0.055 * rows : 16.5 + 0.18 * rows) : (kt == 1 ? 12.5 + 0.033 * rows : 16.5 + 0.02 * rows);
+    const double wave = drift ? 13.5 + 0.055 * rows : 12.5 + 0.033 * rows;
     return (double)((tiles + at_once - 1) / at_once) * wave > (drift ? 10 + 4 * key_tiles : 8 + 2 * key_tiles);
 }
 // Which tensor-core kernel: the two-stream one, but for
