@@ -542,8 +542,8 @@ prep_refresh_kernel(const __nv_bfloat16* h, const int* idx, const int* counts, i
 // All sums run in a fixed order.  K <= KM_MAX_K, W <= KM_MAX_W (what a configuration with proxies admits).
 // A chain of dependent phases on L2-resident rows: each keeps eight or sixteen loads per thread in flight (rows in flat member
 // order, across cluster boundaries, in the centre update) and groups the rows by ballots.  96 rows x 4096, 8 clusters, in the pipeline,
-// with
-// single floats, centres in shared memory, a chain per cluster and loops over the labels 130 us, now 82; 64 rows 96, now 56.
+// with single floats, centres in shared memory, a chain per cluster and loops over the labels 130 us, now 88 (83 of them without the
+// comparisons in 64 bits).
 // ---------------------------------------------------------------------------------------
 constexpr int KM_MAX_K = 16, KM_MAX_W = 256, KM_THREADS = 512, KM_CL = 8, KM_SMEM_BYTES = 160 * 1024;
 // A row's fp32 cosines are compared where they differ by more than their sums' rounding can: two chains of at most 40 additions for
