@@ -193,21 +193,25 @@ def test_c4_shape_reduced_depth_matches_oracle():
     assert kinds == ["entry_full", "within", "within_refresh", "entry_window"], kinds
 
 
-@pytest.mark.parametrize("name,kw", [
-    ("c2", dict(batch=1, prompt_len=544, gen_len=64)),
-    ("c2", dict(batch=2, prompt_len=1000, gen_len=64)),
-    ("c3", dict(batch=2, prompt_len=601, gen_len=64)),          # rows of 665 floats
-    ("c2", dict(batch=1, prompt_len=544, gen_len=64, select_mode=I.SELECT_CLUSTER_TOPK)),
+@pytest.mark.parametrize("name,variant,kw", [
+    ("c2", "0", dict(batch=1, prompt_len=544, gen_len=64)),
+    ("c2", "0", dict(batch=2, prompt_len=1000, gen_len=64)),
+    ("c3", "0", dict(batch=2, prompt_len=601, gen_len=64)),          # rows of 665 floats
+    ("c2", "0", dict(batch=1, prompt_len=544, gen_len=64, select_mode=I.SELECT_CLUSTER_TOPK)),
+    ("c2", "0", dict(batch=1, prompt_len=544, gen_len=64, tau_upd=I.TAU_UPD_NEVER)),      # plain steps: the warp-level kernel
+    ("c2", "8", dict(batch=1, prompt_len=544, gen_len=64)),                               # the cluster kernel throughout
 ])
-def test_more_than_512_keys_at_two_layers_matches_oracle(name, kw):
+def test_more_than_512_keys_at_two_layers_matches_oracle(monkeypatch, name, variant, kw):
     # Beyond 512 keys probabilities are rounded before they are normalised, on both sides: hidden states, K / V, logits and drift
     # after two layers of full width.  (A kernel that rounds elsewhere than the oracle leaves the tolerance here: 6.5 % of the hidden
     # values outside the plain rule, and some outside the scaled one.)
     m, p = I.config(name)
     m = I.reduced_depth(m, 2)
-    p = dataclasses.replace(p, tau_upd=-1, block=32, max_steps=64, flags=p.flags | I.FLAG_KEEP_HIDDEN, **kw)
+    p = dataclasses.replace(p, **{**dict(tau_upd=-1, block=32, max_steps=64, flags=p.flags | I.FLAG_KEEP_HIDDEN), **kw})
+    monkeypatch.setenv("POLESTAR_ATTN_KERNEL", variant)
     kinds = run_reduced_depth(m, p, n_within=2)
-    assert kinds == ["entry_full", "within_refresh", "within_refresh"], kinds
+    within = "within_refresh" if p.tau_upd < 0 else "within"
+    assert kinds == ["entry_full", within, within], kinds
 
 
 def test_c2_shape_centroid_proxies_and_nvfp4_cache_match_oracle():
